@@ -1,7 +1,8 @@
 // fa2.cu -- ForceAtlas2 on the supergraph (Section 3.1, Algorithm 1).
 //
 // One iteration is a fixed chain of kernels with no host round trip:
-//   k_frame     bounding square of the positions (last-block finalise)
+//   k_frame     bounding square of the positions (last-block finalise); the
+//               later steps of a run find it made by the tail before them
 //   k_keys      fixed-point coordinates U and 2L-bit Morton keys; clears the
 //               step's counters (the captured step has no memset nodes)
 //   radix sort  (key, body) pairs -> Morton order: LSD passes on the bits
@@ -30,7 +31,7 @@
 //               barriers): per node gravity, total force, swing and
 //               traction, summed exactly (integer accumulation); the global
 //               speed (per graph in the batched form); per node the local
-//               speed, the displacement and Fprev = F
+//               speed, the displacement and Fprev = F; the next step's frame
 //   (k_node gives the forces alone, without a step)
 //
 // The opening test and the centre it uses are computed with explicit
@@ -47,8 +48,13 @@ namespace bgv {
 namespace {
 constexpr int kThreads = 256;
 constexpr int kMaxFrameBlocks = 1024;  // frame-kernel grid: 2 blocks per SM, at most this many
-constexpr int kMaxNodeBlocks = 2048;   // node-kernel grid: 4 blocks per SM (measured best), at most this many
+constexpr int kMaxNodeBlocks = 2048;   // node-kernel and tail grids: at most this many blocks
 inline int frame_blocks() { return sm_count() * 2 < kMaxFrameBlocks ? sm_count() * 2 : kMaxFrameBlocks; }
+// Bodies per warp when `blocks` blocks share K of them, in whole rows of 32.
+inline int64_t warp_share(int64_t K, int blocks) {
+    const int64_t warps = int64_t(blocks) * (kThreads / 32);
+    return ((K + warps - 1) / warps + 31) / 32 * 32;
+}
 inline int node_blocks() { return sm_count() * 4 < kMaxNodeBlocks ? sm_count() * 4 : kMaxNodeBlocks; }
 
 typedef unsigned __int128 u128;
@@ -68,105 +74,141 @@ __device__ __forceinline__ unsigned long long spread_bits(uint32_t v) {
 __device__ __forceinline__ float pow2_neg(int level) { return __int_as_float((127 - level) << 23); }
 
 // ----------------------------------------------------------------- frame
-__global__ void __launch_bounds__(kThreads) k_frame(const float2 *__restrict__ pos, int64_t K, float4 *part,
-                                                    float4 *frame, unsigned int *ticket) {
-    float lx = INFINITY, ly = INFINITY, hx = -INFINITY, hy = -INFINITY;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < K; i += stride) {
-        const float2 p = pos[i];
-        lx = fminf(lx, p.x); ly = fminf(ly, p.y);
-        hx = fmaxf(hx, p.x); hy = fmaxf(hy, p.y);
-    }
+// Frame of a bounding box: origin, side = max extent * (1 + 2^-20).
+__device__ __forceinline__ float4 frame_of(float lx, float ly, float hx, float hy) {
+    const float ex = __fsub_rn(hx, lx), ey = __fsub_rn(hy, ly);
+    const float ext = ex > ey ? ex : ey;
+    float side = __fmul_rn(ext, 1.00000095367431640625f);  // 1 + 2^-20
+    if (!(ext > 0.0f)) side = 1.0f;
+    return make_float4(lx, ly, side, 0.0f);
+}
+
+__device__ __forceinline__ float4 box_empty() { return make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY); }
+__device__ __forceinline__ void box_add(float4 &b, float2 p) {
+    b.x = fminf(b.x, p.x); b.y = fminf(b.y, p.y);
+    b.z = fmaxf(b.z, p.x); b.w = fmaxf(b.w, p.y);
+}
+__device__ __forceinline__ void box_merge(float4 &b, const float4 &o) {
+    b.x = fminf(b.x, o.x); b.y = fminf(b.y, o.y);
+    b.z = fmaxf(b.z, o.z); b.w = fmaxf(b.w, o.w);
+}
+__device__ __forceinline__ void box_warp(float4 &b) {
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        lx = fminf(lx, __shfl_xor_sync(0xFFFFFFFFu, lx, d));
-        ly = fminf(ly, __shfl_xor_sync(0xFFFFFFFFu, ly, d));
-        hx = fmaxf(hx, __shfl_xor_sync(0xFFFFFFFFu, hx, d));
-        hy = fmaxf(hy, __shfl_xor_sync(0xFFFFFFFFu, hy, d));
-    }
-    __shared__ float4 wpart[kThreads / 32];
-    __shared__ bool last;
-    if ((threadIdx.x & 31) == 0) wpart[threadIdx.x >> 5] = make_float4(lx, ly, hx, hy);
+    for (int d = 16; d > 0; d >>= 1)
+        box_merge(b, make_float4(__shfl_xor_sync(0xFFFFFFFFu, b.x, d), __shfl_xor_sync(0xFFFFFFFFu, b.y, d),
+                                 __shfl_xor_sync(0xFFFFFFFFu, b.z, d), __shfl_xor_sync(0xFFFFFFFFu, b.w, d)));
+}
+// Block-wide box; every thread calls it, thread 0 receives the result.
+__device__ __forceinline__ void box_block(float4 &b) {
+    __shared__ float4 wbox[kThreads / 32];
+    box_warp(b);
+    if ((threadIdx.x & 31) == 0) wbox[threadIdx.x >> 5] = b;
     __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < kThreads / 32; ++w) box_merge(b, wbox[w]);
+    __syncthreads();
+}
+
+// The frame of all blocks' boxes: block partials, then the last block reduces
+// them, all threads at once (min and max do not depend on the order).  Every
+// thread of every block calls it.
+__device__ __forceinline__ void box_to_frame(float4 b, float4 *part, float4 *frame, unsigned int *ticket) {
+    __shared__ bool last;
+    box_block(b);
     if (threadIdx.x == 0) {
-        float4 r = wpart[0];
-        for (int w = 1; w < kThreads / 32; ++w) {
-            r.x = fminf(r.x, wpart[w].x); r.y = fminf(r.y, wpart[w].y);
-            r.z = fmaxf(r.z, wpart[w].z); r.w = fmaxf(r.w, wpart[w].w);
-        }
-        part[blockIdx.x] = r;
+        part[blockIdx.x] = b;
         __threadfence();
         last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
-    // the last block reduces the block partials, all threads at once
-    // (min and max do not depend on the order)
     __threadfence();
-    float4 r = make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
-        const float4 q = __ldcg(&part[b]);
-        r.x = fminf(r.x, q.x); r.y = fminf(r.y, q.y);
-        r.z = fmaxf(r.z, q.z); r.w = fmaxf(r.w, q.w);
+    b = box_empty();
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x) box_merge(b, __ldcg(&part[k]));
+    box_block(b);
+    if (threadIdx.x == 0) {
+        *frame = frame_of(b.x, b.y, b.z, b.w);
+        *ticket = 0u;
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        r.x = fminf(r.x, __shfl_xor_sync(0xFFFFFFFFu, r.x, d));
-        r.y = fminf(r.y, __shfl_xor_sync(0xFFFFFFFFu, r.y, d));
-        r.z = fmaxf(r.z, __shfl_xor_sync(0xFFFFFFFFu, r.z, d));
-        r.w = fmaxf(r.w, __shfl_xor_sync(0xFFFFFFFFu, r.w, d));
-    }
-    __syncthreads();  // wpart is reused
-    if ((threadIdx.x & 31) == 0) wpart[threadIdx.x >> 5] = r;
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    r = wpart[0];
-    for (int w = 1; w < kThreads / 32; ++w) {
-        r.x = fminf(r.x, wpart[w].x); r.y = fminf(r.y, wpart[w].y);
-        r.z = fmaxf(r.z, wpart[w].z); r.w = fmaxf(r.w, wpart[w].w);
-    }
-    const float ex = __fsub_rn(r.z, r.x), ey = __fsub_rn(r.w, r.y);
-    const float ext = ex > ey ? ex : ey;
-    float side = __fmul_rn(ext, 1.00000095367431640625f);  // 1 + 2^-20
-    if (!(ext > 0.0f)) side = 1.0f;
-    *frame = make_float4(r.x, r.y, side, 0.0f);
-    *ticket = 0u;
 }
 
-// Batched form: one block per graph; graph g owns bodies [koff[g], koff[g+1]).
-__global__ void __launch_bounds__(kThreads) k_frame_seg(const float2 *__restrict__ pos,
-                                                        const int64_t *__restrict__ koff, float4 *__restrict__ frames,
-                                                        int32_t *__restrict__ bgraph) {
-    const int g = blockIdx.x;
-    const int64_t a = koff[g], b = koff[g + 1];
-    float lx = INFINITY, ly = INFINITY, hx = -INFINITY, hy = -INFINITY;
-    for (int64_t i = a + threadIdx.x; i < b; i += blockDim.x) {
-        const float2 p = pos[i];
-        lx = fminf(lx, p.x); ly = fminf(ly, p.y);
-        hx = fmaxf(hx, p.x); hy = fmaxf(hy, p.y);
-        bgraph[i] = g;
+// First step of a run, and single steps: later steps of a run find the frame
+// made by the step before (k_tail).
+__global__ void __launch_bounds__(kThreads) k_frame(const float2 *__restrict__ pos, int64_t K, float4 *part,
+                                                    float4 *frame, unsigned int *ticket) {
+    float4 b = box_empty();
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < K; i += stride) box_add(b, pos[i]);
+    box_to_frame(b, part, frame, ticket);
+}
+
+// Bounding boxes of the batched form: four ordered integers per graph (a
+// float's bits, flipped so that unsigned order is float order), so a box is
+// the atomic min and max of its parts, whatever their order.
+__device__ __forceinline__ uint32_t box_key(float f) {
+    const uint32_t b = __float_as_uint(f);
+    return (b & 0x80000000u) ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ float box_val(uint32_t k) {
+    return __uint_as_float((k & 0x80000000u) ? k & 0x7FFFFFFFu : ~k);
+}
+__device__ __forceinline__ uint4 box_keys_empty() {
+    return make_uint4(box_key(INFINITY), box_key(INFINITY), box_key(-INFINITY), box_key(-INFINITY));
+}
+__device__ __forceinline__ void box_publish(uint4 *box, const float4 &b) {
+    atomicMin(&box->x, box_key(b.x));
+    atomicMin(&box->y, box_key(b.y));
+    atomicMax(&box->z, box_key(b.z));
+    atomicMax(&box->w, box_key(b.w));
+}
+
+__global__ void __launch_bounds__(kThreads) k_box_init(int32_t G, uint4 *__restrict__ box) {
+    for (int32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x)
+        box[g] = box_keys_empty();
+}
+
+// Frames from the finished boxes, which are emptied for the next step.
+__global__ void __launch_bounds__(kThreads) k_frame_fin(int32_t G, uint4 *__restrict__ box,
+                                                        float4 *__restrict__ frames) {
+    for (int32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
+        const uint4 b = box[g];
+        frames[g] = frame_of(box_val(b.x), box_val(b.y), box_val(b.z), box_val(b.w));
+        box[g] = box_keys_empty();
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        lx = fminf(lx, __shfl_xor_sync(0xFFFFFFFFu, lx, d));
-        ly = fminf(ly, __shfl_xor_sync(0xFFFFFFFFu, ly, d));
-        hx = fmaxf(hx, __shfl_xor_sync(0xFFFFFFFFu, hx, d));
-        hy = fmaxf(hy, __shfl_xor_sync(0xFFFFFFFFu, hy, d));
+}
+
+// Graph of body i: the largest g with koff[g] <= i.
+__device__ __forceinline__ int32_t body_graph(const int64_t *__restrict__ koff, int32_t G, int64_t i) {
+    int32_t lo = 0, hi = G;
+    while (hi - lo > 1) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (koff[mid] <= i) lo = mid; else hi = mid;
     }
-    __shared__ float4 wpart[kThreads / 32];
-    if ((threadIdx.x & 31) == 0) wpart[threadIdx.x >> 5] = make_float4(lx, ly, hx, hy);
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    float4 r = wpart[0];
-    for (int w = 1; w < kThreads / 32; ++w) {
-        r.x = fminf(r.x, wpart[w].x); r.y = fminf(r.y, wpart[w].y);
-        r.z = fmaxf(r.z, wpart[w].z); r.w = fmaxf(r.w, wpart[w].w);
+    return lo;
+}
+
+// Batched form, first step of a run: the graph of every body and the boxes.
+// Warp w takes bodies [w per, (w + 1) per) and walks the graphs in them (one
+// block per graph left most of the GPU idle behind the largest graphs: 110 us
+// for 6.0 M bodies in 160 graphs).
+__global__ void __launch_bounds__(kThreads) k_frame_seg(const float2 *__restrict__ pos, int64_t K, int64_t per,
+                                                        const int64_t *__restrict__ koff, int32_t G,
+                                                        uint4 *__restrict__ box, int32_t *__restrict__ bgraph) {
+    const int lane = threadIdx.x & 31;
+    int64_t lo = ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * per;
+    if (lo >= K) return;
+    const int64_t end = lo + per < K ? lo + per : K;
+    for (int32_t g = body_graph(koff, G, lo); lo < end; ++g) {
+        const int64_t hi = koff[g + 1] < end ? koff[g + 1] : end;
+        float4 b = box_empty();
+        for (int64_t i = lo + lane; i < hi; i += 32) {
+            box_add(b, pos[i]);
+            bgraph[i] = g;
+        }
+        box_warp(b);
+        if (lane == 0) box_publish(&box[g], b);
+        lo = hi;
     }
-    const float ex = __fsub_rn(r.z, r.x), ey = __fsub_rn(r.w, r.y);
-    const float ext = ex > ey ? ex : ey;
-    float side = __fmul_rn(ext, 1.00000095367431640625f);  // 1 + 2^-20
-    if (!(ext > 0.0f)) side = 1.0f;
-    frames[g] = make_float4(r.x, r.y, side, 0.0f);
 }
 
 // ------------------------------------------------------------------ keys
@@ -1099,14 +1141,6 @@ __device__ __forceinline__ float2 swing_traction(float m, float fx, float fy, fl
     return make_float2(__fmul_rn(m, sw), __fmul_rn(__fmul_rn(0.5f, m), tr));
 }
 
-// The step's tail in one persistent kernel (all blocks resident at once,
-// cooperative launch): per node the total force and the swing and traction
-// products; a grid barrier; the global speed (every block merges the block
-// partials in block order, so all blocks hold the same value; batched: one
-// block per graph sums that graph's rows, then a second barrier); then per
-// node the local speed and the displacement, Fprev = F.  The barrier waits
-// are bounded and report BGV_DEV_TIMEOUT.
-// full == nullptr: no CSR entries, no attraction.
 __device__ __forceinline__ float2 force_sum(float2 fa, float m, float2 pi, float2 fr, float kg, int strong) {
     float gx, gy;
     if (strong) {
@@ -1154,59 +1188,90 @@ __global__ void __launch_bounds__(kThreads) k_node(int64_t K, const float2 *__re
     }
 }
 
-constexpr int kTailItems = 4;  // nodes a thread takes per pass
-__global__ void __launch_bounds__(kThreads) k_tail(int64_t K, const float2 *__restrict__ att,
+// The step's tail in one persistent kernel (all blocks resident at once,
+// cooperative launch): per node the total force and the swing and traction
+// products, summed exactly; a grid barrier; the global speed; then per node
+// the local speed and the displacement, Fprev = F, and the bounding box of the
+// new positions, so that the next step of a run starts with its frame.  The
+// barrier waits are bounded and report BGV_DEV_TIMEOUT.
+// Warp w takes nodes [w per, (w + 1) per), four to a lane and pass, and the
+// grid has no more blocks than it takes to give every thread kTailItems nodes:
+// a barrier over hundreds of blocks cost more than the work of a few thousand
+// nodes (measured at K = 60,013: 21.4 us with 608 blocks).
+// Batched (kB): a warp walks the graphs in its nodes and leaves one exact
+// partial per graph, at slot w + g (every step along the walk raises one of the
+// two, so slots are distinct); after the barrier a warp per graph merges its
+// partials and sets its speed; a second barrier.  (One block per graph summing
+// that graph's rows took 569 us for 6.0 M nodes in 160 graphs; with this split
+// and the frames from the tail, 300 steps of that batch take 556.9 ms instead
+// of 689.2, and 200 steps of a 1,000-node layout 12.4 ms instead of 14.7.)
+// att == nullptr: no CSR entries, no attraction.
+constexpr int kTailItems = 4;  // nodes a lane takes per pass, every load issued before the arithmetic
+
+// Merge of one (S, T) pair per lane; lane 0 receives the result.
+__device__ __forceinline__ void xsum_warp(XSum &S, XSum &T) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const XSum oS = xsum_shfl_down(S, d), oT = xsum_shfl_down(T, d);
+        S = xsum_merge(S, oS);
+        T = xsum_merge(T, oT);
+    }
+}
+
+template <bool kB>
+__global__ void __launch_bounds__(kThreads) k_tail(int64_t K, int64_t per, const float2 *__restrict__ att,
                                                    const uint32_t *__restrict__ mass, float2 *__restrict__ pos,
                                                    const float2 *__restrict__ Frep, float kg, int strong,
                                                    float2 *__restrict__ F, float2 *__restrict__ Fprev, XPart *part,
                                                    double *speed, float tau, float ks, float ksmax, WsHeader *hdr,
-                                                   float2 *__restrict__ rowst, const int64_t *__restrict__ koff,
-                                                   const int32_t *__restrict__ bgraph, int32_t G, int spin_limit) {
+                                                   const int64_t *__restrict__ koff, int32_t G, uint4 *box,
+                                                   float4 *frame_part, float4 *frame, int spin_limit) {
     __shared__ double sp_sh;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    const int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const bool batched = rowst != nullptr;
-    const double sp_old = batched ? 0.0 : *speed;  // read by every block before anyone writes it
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t warps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    const int64_t c_lo = warp * per < K ? warp * per : K;
+    const int64_t c_hi = c_lo + per < K ? c_lo + per : K;
+    const double sp_old = kB ? 0.0 : *speed;  // read by every block before anyone writes it
+    const float2 z = make_float2(0.0f, 0.0f);
+    const int32_t g_first = kB && c_lo < c_hi ? body_graph(koff, G, c_lo) : 0;
     XSum S = xsum_zero(), T = xsum_zero();
-    // kTailItems nodes per pass, every load issued before the arithmetic (the
-    // exact sums do not depend on the order of the terms)
-    for (int64_t i0 = t0; i0 < K; i0 += stride * kTailItems) {
-        uint32_t mk[kTailItems];
-        float2 pk[kTailItems], rk[kTailItems], ak[kTailItems], qk[kTailItems];
+    auto sum_forces = [&](int64_t lo, int64_t hi) {
+        for (int64_t i0 = lo + lane; i0 < hi; i0 += 32 * kTailItems) {
+            uint32_t mk[kTailItems];
+            float2 pk[kTailItems], rk[kTailItems], ak[kTailItems], qk[kTailItems];
 #pragma unroll
-        for (int k = 0; k < kTailItems; ++k) {
-            const int64_t i = i0 + stride * k;
-            const bool in = i < K;
-            const float2 z = make_float2(0.0f, 0.0f);
-            mk[k] = in ? mass[i] : 0u;
-            pk[k] = in ? pos[i] : z;
-            rk[k] = in ? Frep[i] : z;
-            ak[k] = in && att ? att[i] : z;
-            qk[k] = in ? Fprev[i] : z;
-        }
+            for (int k = 0; k < kTailItems; ++k) {
+                const int64_t i = i0 + 32 * k;
+                const bool in = i < hi;
+                mk[k] = in ? mass[i] : 0u;
+                pk[k] = in ? pos[i] : z;
+                rk[k] = in ? Frep[i] : z;
+                ak[k] = in && att ? att[i] : z;
+                qk[k] = in ? Fprev[i] : z;
+            }
 #pragma unroll
-        for (int k = 0; k < kTailItems; ++k) {
-            const int64_t i = i0 + stride * k;
-            if (i >= K) continue;
-            const float m = __uint2float_rn(mk[k]);
-            const float2 f = force_sum(ak[k], m, pk[k], rk[k], kg, strong);
-            F[i] = f;
-            const float2 st = swing_traction(m, f.x, f.y, qk[k].x, qk[k].y);
-            if (batched) {
-                rowst[i] = st;
-            } else {
+            for (int k = 0; k < kTailItems; ++k) {
+                const int64_t i = i0 + 32 * k;
+                if (i >= hi) continue;
+                const float m = __uint2float_rn(mk[k]);
+                const float2 f = force_sum(ak[k], m, pk[k], rk[k], kg, strong);
+                F[i] = f;
+                const float2 st = swing_traction(m, f.x, f.y, qk[k].x, qk[k].y);
                 xsum_add(S, st.x);
                 xsum_add(T, st.y);
             }
         }
-    }
-    if (!batched) {
+    };
+    if (!kB) {
+        sum_forces(c_lo, c_hi);
         xsum_block(S, T);
         if (threadIdx.x == 0) {
             part[2 * blockIdx.x] = xsum_pack(S);
             part[2 * blockIdx.x + 1] = xsum_pack(T);
         }
         if (!grid_barrier(&hdr->bar, spin_limit, &hdr->status)) return;
+        // every block merges the block partials, so all hold the same speed
         S = xsum_zero();
         T = xsum_zero();
         for (unsigned bk = threadIdx.x; bk < gridDim.x; bk += blockDim.x) {
@@ -1226,20 +1291,33 @@ __global__ void __launch_bounds__(kThreads) k_tail(int64_t K, const float2 *__re
         }
         __syncthreads();
     } else {
-        if (!grid_barrier(&hdr->bar, spin_limit, &hdr->status)) return;
-        for (int32_t g = blockIdx.x; g < G; g += gridDim.x) {  // one block per graph
-            const int64_t a = koff[g], b = koff[g + 1];
-            XSum Sg = xsum_zero(), Tg = xsum_zero();
-            for (int64_t i = a + threadIdx.x; i < b; i += blockDim.x) {
-                const float2 v = __ldcg(&rowst[i]);
-                xsum_add(Sg, v.x);
-                xsum_add(Tg, v.y);
+        int32_t g = g_first;
+        for (int64_t lo = c_lo; lo < c_hi; ++g) {
+            const int64_t hi = koff[g + 1] < c_hi ? koff[g + 1] : c_hi;
+            S = xsum_zero();
+            T = xsum_zero();
+            sum_forces(lo, hi);
+            xsum_warp(S, T);
+            if (lane == 0) {
+                part[2 * (warp + g)] = xsum_pack(S);
+                part[2 * (warp + g) + 1] = xsum_pack(T);
             }
-            xsum_block(Sg, Tg);
-            if (threadIdx.x == 0) {
-                const double Ssum = xsum_value(Sg), Tsum = xsum_value(Tg);
-                speed[g] = speed_update(speed[g], Ssum, Tsum, tau);
-                if (g == 0) {
+            lo = hi;
+        }
+        if (!grid_barrier(&hdr->bar, spin_limit, &hdr->status)) return;
+        for (int64_t q = warp; q < G; q += warps) {  // a warp per graph: the warps its nodes lie in
+            const int64_t w0 = koff[q] / per, w1 = (koff[q + 1] - 1) / per;
+            S = xsum_zero();
+            T = xsum_zero();
+            for (int64_t w = w0 + lane; w <= w1; w += 32) {
+                S = xsum_merge(S, xsum_unpack(&part[2 * (w + q)]));
+                T = xsum_merge(T, xsum_unpack(&part[2 * (w + q) + 1]));
+            }
+            xsum_warp(S, T);
+            if (lane == 0) {
+                const double Ssum = xsum_value(S), Tsum = xsum_value(T);
+                speed[q] = speed_update(speed[q], Ssum, Tsum, tau);
+                if (q == 0) {
                     hdr->S = Ssum;
                     hdr->T = Tsum;
                     hdr->steps_total += 1;
@@ -1248,26 +1326,41 @@ __global__ void __launch_bounds__(kThreads) k_tail(int64_t K, const float2 *__re
         }
         if (!grid_barrier(&hdr->bar, spin_limit, &hdr->status)) return;
     }
-    const float sp_all = float(sp_sh);
-    for (int64_t i0 = t0; i0 < K; i0 += stride * kTailItems) {
-        float2 fk[kTailItems], qk[kTailItems], pk[kTailItems];
-        float sk[kTailItems];
+    float4 b = box_empty();
+    auto move = [&](int64_t lo, int64_t hi, float sp) {
+        for (int64_t i0 = lo + lane; i0 < hi; i0 += 32 * kTailItems) {
+            float2 fk[kTailItems], qk[kTailItems], pk[kTailItems];
 #pragma unroll
-        for (int k = 0; k < kTailItems; ++k) {
-            const int64_t i = i0 + stride * k;
-            const bool in = i < K;
-            const float2 z = make_float2(0.0f, 0.0f);
-            fk[k] = in ? __ldcg(&F[i]) : z;  // written by this kernel before the barrier
-            qk[k] = in ? Fprev[i] : z;
-            pk[k] = in ? pos[i] : z;
-            sk[k] = in && batched ? float(__ldcg(&speed[bgraph[i]])) : sp_all;
+            for (int k = 0; k < kTailItems; ++k) {
+                const int64_t i = i0 + 32 * k;
+                const bool in = i < hi;
+                fk[k] = in ? F[i] : z;  // written by this thread before the barrier
+                qk[k] = in ? Fprev[i] : z;
+                pk[k] = in ? pos[i] : z;
+            }
+#pragma unroll
+            for (int k = 0; k < kTailItems; ++k) {
+                const int64_t i = i0 + 32 * k;
+                if (i >= hi) continue;
+                const float2 p = displaced(pk[k], fk[k], qk[k], sp, ks, ksmax);
+                pos[i] = p;
+                Fprev[i] = fk[k];
+                box_add(b, p);
+            }
         }
-#pragma unroll
-        for (int k = 0; k < kTailItems; ++k) {
-            const int64_t i = i0 + stride * k;
-            if (i >= K) continue;
-            pos[i] = displaced(pk[k], fk[k], qk[k], sk[k], ks, ksmax);
-            Fprev[i] = fk[k];
+    };
+    if (!kB) {
+        move(c_lo, c_hi, float(sp_sh));
+        box_to_frame(b, frame_part, frame, &hdr->bbox_ticket);
+    } else {
+        int32_t g = g_first;
+        for (int64_t lo = c_lo; lo < c_hi; ++g) {
+            const int64_t hi = koff[g + 1] < c_hi ? koff[g + 1] : c_hi;
+            b = box_empty();
+            move(lo, hi, float(__ldcg(&speed[g])));
+            box_warp(b);
+            if (lane == 0) box_publish(&box[g], b);
+            lo = hi;
         }
     }
 }
@@ -1329,7 +1422,7 @@ struct Fa2Scratch {
     float4 *frame;         // frames: one per graph
     float4 *frame_part;
     int32_t *bgraph;       // batched form: graph of each body
-    float2 *rowst;         // batched form: per-row swing, traction
+    uint4 *box;            // batched form: bounding box of each graph (ordered integers)
     SortBuffers sort;
     RunFixBuffers runfix;
     float4 *body;          // sorted bodies: x, y, mass, index
@@ -1350,7 +1443,7 @@ struct Fa2Scratch {
     float2 *full;          // attraction per row
     int32_t *rows_short, *rows_med, *rows_long;  // plan: rows by length class
     uint32_t *att_counts;  // plan: the three list lengths
-    XPart *part;  // per node-kernel block: exact S and T partials
+    XPart *part;  // exact S and T partials: per tail block; batched: per warp and graph (slot warp + graph)
     HsBuffers hs;  // hinted sort of the Morton keys
 };
 
@@ -1358,9 +1451,9 @@ static void carve_fa2(Carver &c, int64_t K, int64_t nnz, int32_t G, Fa2Scratch &
     const size_t k = size_t(K > 0 ? K : 1);
     const bool batched = G > 1;
     s.frame = c.take<float4>(size_t(G > 1 ? G : 1));
-    s.frame_part = c.take<float4>(kMaxFrameBlocks);
+    s.frame_part = c.take<float4>(kMaxNodeBlocks);
     s.bgraph = batched ? c.take<int32_t>(k) : nullptr;
-    s.rowst = batched ? c.take<float2>(k) : nullptr;
+    s.box = batched ? c.take<uint4>(size_t(G)) : nullptr;
     carve_sort(c, int64_t(k), true, s.sort);
     carve_run_fix(c, int64_t(k), s.runfix);
     s.body = c.take<float4>(k);
@@ -1385,7 +1478,7 @@ static void carve_fa2(Carver &c, int64_t K, int64_t nnz, int32_t G, Fa2Scratch &
     s.rows_med = c.take<int32_t>(k);
     s.rows_long = c.take<int32_t>(k);
     s.att_counts = c.take<uint32_t>(4);
-    s.part = c.take<XPart>(2 * size_t(kMaxNodeBlocks));
+    s.part = c.take<XPart>(2 * (batched ? size_t(kMaxNodeBlocks) * (kThreads / 32) + size_t(G) : size_t(kMaxNodeBlocks)));
     carve_hs(c, s.hs);
 }
 
@@ -1616,11 +1709,24 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
                                                                         s.att_counts, s.full);
         BGV_TRY(launch_status());
     }
-    if (batched)
-        note_launch(), k_frame_seg<<<G, kThreads, 0, st>>>(pos, koff, s.frame, s.bgraph);
-    else
-        note_launch(), k_frame<<<frame_blocks(), kThreads, 0, st>>>(pos, K, s.frame_part, s.frame, &hdr->bbox_ticket);
-    BGV_TRY(launch_status());
+    // the tail of the previous step of a run left the frame (batched: the
+    // boxes) of the positions it wrote
+    if (batched) {
+        const int gg = grid_for(G, kThreads, sm_count());
+        if (!hinted) {
+            const int fb = grid_for(K, kThreads * kTailItems, node_blocks());
+            note_launch(), k_box_init<<<gg, kThreads, 0, st>>>(G, s.box);
+            BGV_TRY(launch_status());
+            note_launch(), k_frame_seg<<<fb, kThreads, 0, st>>>(pos, K, warp_share(K, fb), koff, G, s.box, s.bgraph);
+            BGV_TRY(launch_status());
+        }
+        note_launch(), k_frame_fin<<<gg, kThreads, 0, st>>>(G, s.box, s.frame);
+        BGV_TRY(launch_status());
+    } else if (!hinted) {
+        note_launch(), k_frame<<<grid_for(K, kThreads, frame_blocks()), kThreads, 0, st>>>(pos, K, s.frame_part,
+                                                                                         s.frame, &hdr->bbox_ticket);
+        BGV_TRY(launch_status());
+    }
     const int64_t mom_tiles = (K + kMomTile - 1) / kMomTile;
     // the sorted order lands in the buffer pair the radix sort ends in, so
     // the next iteration finds its hint there whichever sort made it
@@ -1706,20 +1812,19 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
             reinterpret_cast<float2 *>(Fa), reinterpret_cast<float2 *>(Fg));
         BGV_TRY(launch_status());
     } else {
-        float2 *rowst = batched ? s.rowst : nullptr;
-        const int64_t *koff_d = batched ? koff : nullptr;
-        const int32_t *bgraph = s.bgraph;
         int32_t g_count = G;
         float kg = p.kg, tau = p.tau, ks = p.ks, ksmax = p.ksmax;
         int strong = p.strong_gravity, limit = spin_limit();
-        int64_t k_count = K;
+        const void *tail = batched ? reinterpret_cast<const void *>(k_tail<true>)
+                                   : reinterpret_cast<const void *>(k_tail<false>);
+        const int want = grid_for(K, kThreads * kTailItems, sm_count() * tune.tail_blocks_per_sm);
+        const int blocks = coop_blocks(tail, kThreads, want);
+        int64_t k_count = K, per = warp_share(K, blocks);
         XPart *part = s.part;
         const float2 *frep = s.Frep;
-        void *args[] = {&k_count, &att, &mass, &pos, &frep, &kg, &strong, &F, &Fprev, &part, &speed, &tau, &ks,
-                        &ksmax, &hdr, &rowst, &koff_d, &bgraph, &g_count, &limit};
-        const int blocks = coop_blocks(reinterpret_cast<const void *>(k_tail), kThreads,
-                                       sm_count() * tune.tail_blocks_per_sm);
-        BGV_TRY(launch_coop(reinterpret_cast<const void *>(k_tail), blocks, kThreads, args, st));
+        void *args[] = {&k_count, &per, &att, &mass, &pos, &frep, &kg, &strong, &F, &Fprev, &part, &speed, &tau, &ks,
+                        &ksmax, &hdr, &koff, &g_count, &s.box, &s.frame_part, &s.frame, &limit};
+        BGV_TRY(launch_coop(tail, blocks, kThreads, args, st));
     }
     BGV_TRY(mark(8));
     return BGV_OK;
