@@ -248,10 +248,10 @@ __device__ __forceinline__ bool grid_barrier(GridBar *h, int spin_limit, uint32_
 }
 
 // Blocks of `threads` threads that a cooperative launch of `kernel` can keep
-// resident at once, at most `want` (at least 1).
-int coop_blocks(const void *kernel, int threads, int want);
+// resident at once, at most `want` (at least 1); `smem`: dynamic shared memory.
+int coop_blocks(const void *kernel, int threads, int want, size_t smem = 0);
 // Cooperative launch on `st` (all blocks resident together).
-int launch_coop(const void *kernel, int blocks, int threads, void **args, cudaStream_t st);
+int launch_coop(const void *kernel, int blocks, int threads, void **args, cudaStream_t st, size_t smem = 0);
 
 // --------------------------------------------------------- stage internals
 // Enqueue-only stage bodies used by the public entry points and the
@@ -281,6 +281,8 @@ struct CommScratch {
     uint4 *bstate;                  // batched form: (degree, label, threshold, first threshold)
     unsigned long long *best;       // packed (edge index, label) proposals
     uint32_t *jump;                 // labels after a pointer-jumping step
+    uint32_t *map;                  // bit map of the nodes that pass the round's threshold
+    uint32_t *any;                  // [2] a bit of the round's map is set (by round parity)
 };
 void carve_comm(Carver &c, int64_t m, int32_t n, CommScratch &s, bool batched = false);
 // growth 0: the threshold is multiplied by its first value every round (the

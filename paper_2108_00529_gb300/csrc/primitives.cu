@@ -23,18 +23,19 @@ static std::atomic<int> g_spin_limit{1 << 22};
 int spin_limit() { return g_spin_limit.load(std::memory_order_relaxed); }
 int set_spin_limit(int limit) { return g_spin_limit.exchange(limit, std::memory_order_relaxed); }
 
-int coop_blocks(const void *kernel, int threads, int want) {
+int coop_blocks(const void *kernel, int threads, int want, size_t smem) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess) per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess) per_sm = 1;
     const int most = (per_sm > 0 ? per_sm : 1) * sm_count();
     const int b = want < most ? want : most;
     return b > 0 ? b : 1;
 }
 
-int launch_coop(const void *kernel, int blocks, int threads, void **args, cudaStream_t st) {
+int launch_coop(const void *kernel, int blocks, int threads, void **args, cudaStream_t st, size_t smem) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(blocks));
     cfg.blockDim = dim3(unsigned(threads));
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
