@@ -103,6 +103,12 @@ inline int grid_for(int64_t work, int threads, int64_t cap_blocks = -1) {
 
 __device__ __forceinline__ void raise_status(uint32_t *status, uint32_t bits) { atomicOr(status, bits); }
 
+// Place of counter f of an array (a multiple of 1,024 counters) in shared memory:
+// the bank is the exclusive-or of f's 5-bit digits.  On skewed graphs the low
+// bits of ids are far from uniform (two thirds of them 0 in R-MAT), and counters
+// in plain order would pile up on a few banks.
+__device__ __forceinline__ uint32_t swz(uint32_t f) { return f ^ ((f >> 5) & 31u) ^ ((f >> 10) & 31u); }
+
 // ------------------------------------------------------------- hash family
 // h_i(x) = ((a_i x + b_i) mod (2^31 - 1)) mod width; coefficients from
 // SplitMix64 (Steele, Lea, Flood 2014) at state seed + i.
@@ -175,6 +181,39 @@ int radix_sort_high(SortBuffers &b, const RunFixBuffers &r, int64_t cap, const i
                     cudaStream_t s, int *result_buffer, uint32_t *dev_status, bool counters_cleared = false);
 // The buffer pair radix_sort_high(cap, end_bit) leaves its result in.
 int radix_sort_high_result(int64_t cap, int end_bit);
+
+// radix_sort in its cooperative form, run only if *guard (device) is above
+// guard_min; the result is in buffer pair 0 (an even number of passes).
+int radix_sort_guarded(SortBuffers &b, int64_t cap, const int64_t *d_count, int end_bit, cudaStream_t s,
+                       uint32_t *dev_status, const uint32_t *guard, uint32_t guard_min);
+
+// ------------------------------------------------------------- pair sort
+// Sorted keys row << b | col of both directions of every edge (u, v) with
+// node_map[u] != node_map[v]; b = bits_for(*K_dev) (at least 1).  See
+// pairsort.cu.  For ids of at most kPairSortBits bits; *moved is 0 if node_map
+// is the identity.  buf0 and buf1 hold 2 m keys each; the result is in buf0 and
+// its length in *nkeys, unless *guard comes out non-zero: then the keys are
+// too lopsided, and the caller sorts them (k_cut_pairs and the guarded LSD sort).
+constexpr int kPairSortBits = 28;
+struct PsBucket {
+    uint32_t start, count;        // its keys: [start, start + count)
+    unsigned long long lo, span;  // its key values: [lo, lo + span)
+    uint32_t flags, pad;
+};
+struct PsControl {
+    uint32_t groups, buckets, over, guard, ticket, pad[3];
+};
+struct PairSortScratch {
+    uint32_t *total, *bstart, *bfine, *cursor;
+    uint16_t *bmap;
+    PsControl *ctl;
+    PsBucket *list, *over;
+    uint32_t list_cap, over_cap;
+};
+void carve_pair_sort(Carver &c, int64_t m, int32_t n, PairSortScratch &s);
+int pair_sort(const int32_t *edges, int64_t m, int32_t n, const int32_t *node_map, const int64_t *K_dev,
+              const uint32_t *moved, const PairSortScratch &s, unsigned long long *buf0, unsigned long long *buf1,
+              unsigned long long *nkeys, uint32_t *status, cudaStream_t st);
 
 // Sort autotuner: times the onesweep passes at 8 and at 16 keys per thread
 // and the cooperative sort for 2^14, 2^16, ... up to max_keys; sets the
@@ -313,12 +352,13 @@ struct SuperScratch {
     unsigned long long *nkeys;  // device count of (row, col) keys
     int64_t *nnz;           // device count of CSR entries
     unsigned long long *sketch;  // [rows * width], batched form: one per graph
-    uint32_t *start;        // [2m + 1] first sorted key of every CSR entry
-    int32_t *supidx;        // [2m] superedge of every CSR entry, -1 for col < row
+    uint32_t *moved;        // a label differs from its node
+    unsigned long long *cut_cursor;  // k_cut_pairs: keys written
     uint32_t *red_flags;    // look-back flags of the CSR pass, then its tile counter
     unsigned long long *red_agg, *red_incl;
     void *scan_tmp;
     SortBuffers sort_pairs;   // 2m keys
+    PairSortScratch ps;
 };
 void carve_super(Carver &c, int64_t m, int32_t n, int32_t rows, int32_t width, SuperScratch &s, int32_t G = 1);
 // With `batch`, community labels are node ids of their own graph, so the

@@ -721,6 +721,14 @@ int radix_sort(SortBuffers &b, int64_t cap, const int64_t *d_count, int end_bit,
     return BGV_OK;
 }
 
+int radix_sort_guarded(SortBuffers &b, int64_t cap, const int64_t *d_count, int end_bit, cudaStream_t s,
+                       uint32_t *dev_status, const uint32_t *guard, uint32_t guard_min) {
+    const int passes = ((end_bit + 7) / 8 + 1) & ~1;
+    if (passes > kMaxPasses) return BGV_EINVAL;
+    BGV_CUDA(cudaMemsetAsync(b.counts, 0, sizeof(uint32_t) * size_t(sort_counter_words()), s));
+    return coop_sort(b, cap, d_count, 0, passes, s, dev_status, guard, guard_min);
+}
+
 // ----------------------------------------------- sort with a local finish
 // For keys whose order is almost always decided above their lowest
 // kLowBits = 24 bits (Morton keys of spread-out points: in rmat22x layouts

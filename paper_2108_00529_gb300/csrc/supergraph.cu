@@ -4,17 +4,18 @@
 //
 // 1. Dense relabel: mark the labels in use, exclusive-scan the marks; the
 //    rank of a label is its supernode id (ascending label order).
-// 2. Cut edges: one edge pass emits, for every edge whose endpoints lie in
-//    different supernodes a != c, both directed pairs (a, c) and (c, a) as
-//    u64 keys row << b | col.  Blocks compact their keys in shared memory
-//    and take their output range with one atomic per 1,024 edges.
-// 3. Stable LSD radix sort of the keys over 2 * bits(n) bits.  The sorted
-//    keys are the symmetric CSR in row order with repeated pairs adjacent.
+// 2. Cut edges: every edge whose endpoints lie in different supernodes a != c
+//    gives both directed pairs (a, c) and (c, a) as u64 keys row << b | col, b =
+//    bits of the supernode ids.
+// 3. The sorted keys are the symmetric CSR in row order with repeated pairs
+//    adjacent.  From kPairSortMin edges up they are bucketed straight from the
+//    edge list and sorted in shared memory (pairsort.cu); fewer edges, and keys
+//    too lopsided for that, are written out (k_cut_pairs) and LSD sorted.
 // 4. One pass over the sorted keys (decoupled look-back over tiles) collapses
 //    repeated pairs: distinct pairs become CSR entries (ascending neighbours
 //    per row, row offsets from the row changes) and the pairs with col > row
-//    the superedges (src < dst, sorted ascending); a second pass turns run
-//    starts into multiplicities (edge weights).
+//    the superedges (src < dst, sorted ascending); the length of a run of equal
+//    keys is the pair's weight.
 // 5. Community-size sketch: every node adds its sketched degree at the
 //    hash of its label (u64 counters); mass = 1 + the row minimum.
 #include "bgv_internal.cuh"
@@ -23,16 +24,25 @@ namespace bgv {
 namespace {
 constexpr int kThreads = 256;
 
+// Bits of ids 0..K-1 (bits_for on the device).
+__device__ __forceinline__ int id_bits(int64_t K) { return K <= 2 ? 1 : 64 - __clzll(K - 1); }
+
+// *moved is set if a label differs from its node: with none, node_map comes
+// out as the identity and the edge passes need not look nodes up.
 __global__ void __launch_bounds__(kThreads) k_mark_labels(const int32_t *__restrict__ labels, int32_t n,
-                                                          uint32_t *__restrict__ flags, uint32_t *status) {
+                                                          uint32_t *__restrict__ flags, uint32_t *moved,
+                                                          uint32_t *status) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    int diff = 0;
     for (int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; v < n; v += stride) {
         const int32_t l = labels[v];
+        diff |= l != int32_t(v);
         if (static_cast<uint32_t>(l) < static_cast<uint32_t>(n))
             flags[l] = 1u;
         else
             raise_status(status, BGV_DEV_BADLABEL);
     }
+    if (__syncthreads_or(diff) && threadIdx.x == 0) *moved = 1u;
 }
 
 __global__ void __launch_bounds__(kThreads) k_map_nodes(const int32_t *__restrict__ labels, int32_t n,
@@ -101,9 +111,12 @@ __device__ __forceinline__ uint32_t block_exclusive_u32(uint32_t x, uint32_t *to
 }
 
 __global__ void __launch_bounds__(kThreads) k_cut_pairs(const int32_t *__restrict__ edges, int64_t m, int32_t n,
-                                                        const int32_t *__restrict__ node_map, int shift,
+                                                        const int32_t *__restrict__ node_map, const int64_t *K_dev,
                                                         unsigned long long *__restrict__ keys,
-                                                        unsigned long long *nkeys, uint32_t *status) {
+                                                        unsigned long long *nkeys, const uint32_t *guard,
+                                                        uint32_t *status) {
+    if (guard && *guard == 0u) return;  // the bucket sort has the keys
+    const int shift = id_bits(*K_dev);
     __shared__ unsigned long long stage[kCutKeys];
     __shared__ unsigned long long base_sh;
     const int4 *e2 = reinterpret_cast<const int4 *>(edges);
@@ -156,12 +169,15 @@ __global__ void __launch_bounds__(kThreads) k_cut_pairs(const int32_t *__restric
 // the distinct pairs (heads) and, among them, those with col > row (the
 // superedges).  The tile's two counts are scanned as one u64 (heads in the
 // low 32 bits: at most 2 m < 2^32 of them), then a decoupled look-back gives
-// the tile's offsets.  Outputs are staged in shared memory and written in
-// coalesced runs: csr_adj and the run start of every distinct pair, the
-// superedge index of each CSR entry (or -1), ssrc/sdst of the superedges,
-// and csr_off of every row that starts in the tile (and of the empty rows
-// before it).  The last tile writes the totals, start[nnz] and the offsets of
-// the rows after the last pair.
+// the tile's offsets.  A pair's weight is the distance to the next head; for
+// the tile's last pair the run may go on past the tile, where thread 0 looks
+// for its end (one key as a rule; galloping for long runs).  Outputs are staged
+// in shared memory and written in coalesced runs: csr_adj and csr_w of every
+// distinct pair, ssrc/sdst/sw of the superedges, and csr_off of every row that
+// starts in the tile (and of the empty rows before it).  The last tile writes
+// the totals and the offsets of the rows after the last pair.  (Run starts and
+// superedge indices written here and turned into weights by a second pass cost
+// 16 more bytes per entry: 709 us for both passes at 68 M entries.)
 constexpr int kRedItems = 8;
 constexpr int kRedTile = kThreads * kRedItems;
 enum : uint32_t { kRedAgg = 1u, kRedIncl = 2u };
@@ -200,18 +216,18 @@ __device__ __forceinline__ unsigned long long block_exclusive_u64(unsigned long 
 constexpr int kRedGapList = 64;  // long runs of empty rows a tile fills with all its threads
 
 __global__ void __launch_bounds__(kThreads) k_csr_reduce(const unsigned long long *__restrict__ keys,
-                                                         const unsigned long long *nkeys_dev, int64_t cap, int shift,
+                                                         const unsigned long long *nkeys_dev, int64_t cap,
                                                          const int64_t *K_dev, int32_t *__restrict__ csr_off,
-                                                         int32_t *__restrict__ csr_adj, uint32_t *__restrict__ start,
-                                                         int32_t *__restrict__ supidx, int32_t *__restrict__ ssrc,
-                                                         int32_t *__restrict__ sdst, uint32_t *flags,
+                                                         int32_t *__restrict__ csr_adj, uint32_t *__restrict__ csr_w,
+                                                         int32_t *__restrict__ ssrc, int32_t *__restrict__ sdst,
+                                                         uint32_t *__restrict__ sw, uint32_t *flags,
                                                          unsigned long long *agg, unsigned long long *incl,
                                                          int64_t *Es_dev, int64_t *nnz_dev, uint32_t *dev_status,
                                                          int spin_limit) {
     __shared__ unsigned long long skey[kRedTile + kRedTile / 8];
     __shared__ uint16_t ent_e[kRedTile];   // element of every distinct pair of the tile
-    __shared__ uint16_t sup_e[kRedTile];   // element of every superedge of the tile
-    __shared__ int32_t ssup[kRedTile];     // superedge index of every distinct pair, or -1
+    __shared__ uint16_t sup_d[kRedTile];   // distinct pair of every superedge of the tile
+    __shared__ uint32_t run_end_sh;        // where the run of the tile's last key ends, from the tile's start
     __shared__ long long gap_lo[kRedGapList], gap_hi[kRedGapList];
     __shared__ int32_t gap_val[kRedGapList];
     __shared__ int gaps;
@@ -220,6 +236,7 @@ __global__ void __launch_bounds__(kThreads) k_csr_reduce(const unsigned long lon
     int64_t nk = int64_t(*nkeys_dev);
     nk = nk < cap ? nk : cap;
     const int64_t K = *K_dev;
+    const int shift = id_bits(K);
     const int64_t tiles = (nk + kRedTile - 1) / kRedTile;
     if (threadIdx.x == 0) {
         tile_sh = atomicAdd(&flags[tiles > 0 ? tiles : 1], 1u);
@@ -233,7 +250,6 @@ __global__ void __launch_bounds__(kThreads) k_csr_reduce(const unsigned long lon
         if (tile == 0 && threadIdx.x == 0) {
             *Es_dev = 0;
             *nnz_dev = 0;
-            start[0] = 0u;
         }
         return;
     }
@@ -273,6 +289,22 @@ __global__ void __launch_bounds__(kThreads) k_csr_reduce(const unsigned long lon
         }
         __threadfence();
         atomicExch(&flags[tile], tile == 0 ? kRedIncl : kRedAgg);
+    }
+    if (threadIdx.x == 32) {
+        const unsigned long long k = skey[red_slot(tn - 1)];
+        int64_t lo = t0 + tn, step = 1;  // keys[lo - 1] is in the run
+        while (lo < nk && keys[lo] == k) {
+            lo += step;
+            step <<= 1;
+        }
+        int64_t up = lo < nk ? lo : nk;  // the run's end lies in [lo - step / 2, up]
+        lo = lo - (step >> 1);
+        if (lo < t0 + tn) lo = t0 + tn;
+        while (lo < up) {
+            const int64_t mid = (lo + up) >> 1;
+            if (keys[mid] <= k) lo = mid + 1; else up = mid;
+        }
+        run_end_sh = uint32_t(lo - t0);
     }
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
@@ -326,13 +358,7 @@ __global__ void __launch_bounds__(kThreads) k_csr_reduce(const unsigned long lon
         const unsigned long long k = skey[red_slot(e)];
         const long long row = static_cast<long long>(k >> shift);
         ent_e[dl] = uint16_t(e);
-        if ((ups >> j) & 1u) {
-            ssup[dl] = int32_t(u_excl + ul);
-            sup_e[ul] = uint16_t(e);
-            ++ul;
-        } else {
-            ssup[dl] = -1;
-        }
+        if ((ups >> j) & 1u) sup_d[ul++] = uint16_t(dl);
         if (row > prev_row) {
             const int32_t v = int32_t(d_excl + dl);
             if (row - prev_row <= 32) {
@@ -352,16 +378,19 @@ __global__ void __launch_bounds__(kThreads) k_csr_reduce(const unsigned long lon
         ++dl;
     }
     __syncthreads();
+    auto weight = [&](uint32_t j) {
+        return (j + 1 < d_tile ? uint32_t(ent_e[j + 1]) : run_end_sh) - uint32_t(ent_e[j]);
+    };
     for (uint32_t j = threadIdx.x; j < d_tile; j += kThreads) {
-        const int e = ent_e[j];
-        csr_adj[d_excl + j] = int32_t(skey[red_slot(e)] & col_mask);
-        start[d_excl + j] = uint32_t(t0 + e);
-        supidx[d_excl + j] = ssup[j];
+        csr_adj[d_excl + j] = int32_t(skey[red_slot(ent_e[j])] & col_mask);
+        csr_w[d_excl + j] = weight(j);
     }
     for (uint32_t j = threadIdx.x; j < u_tile; j += kThreads) {
-        const unsigned long long k = skey[red_slot(sup_e[j])];
+        const uint32_t d = sup_d[j];
+        const unsigned long long k = skey[red_slot(ent_e[d])];
         ssrc[u_excl + j] = int32_t(k >> shift);
         sdst[u_excl + j] = int32_t(k & col_mask);
+        sw[u_excl + j] = weight(d);
     }
     const int ng = gaps < kRedGapList ? gaps : kRedGapList;
     for (int g = 0; g < ng; ++g)
@@ -371,24 +400,9 @@ __global__ void __launch_bounds__(kThreads) k_csr_reduce(const unsigned long lon
         const long long last_row = static_cast<long long>(skey[red_slot(tn - 1)] >> shift);
         for (long long r = last_row + 1 + threadIdx.x; r <= K; r += kThreads) csr_off[r] = int32_t(D);
         if (threadIdx.x == 0) {
-            start[D] = uint32_t(nk);
             *Es_dev = U;
             *nnz_dev = D;
         }
-    }
-}
-
-// Multiplicities: CSR entry j covers sorted keys start[j] .. start[j+1].
-__global__ void __launch_bounds__(kThreads) k_csr_weights(const uint32_t *__restrict__ start,
-                                                          const int32_t *__restrict__ supidx, const int64_t *nnz_dev,
-                                                          uint32_t *__restrict__ csr_w, uint32_t *__restrict__ sw) {
-    const int64_t D = *nnz_dev;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < D; j += stride) {
-        const uint32_t w = start[j + 1] - start[j];
-        csr_w[j] = w;
-        const int32_t u = supidx[j];
-        if (u >= 0) sw[u] = w;
     }
 }
 
@@ -454,6 +468,10 @@ __global__ void __launch_bounds__(kThreads) k_mass(const int32_t *__restrict__ l
 
 }  // namespace
 
+// Below, the LSD sort's few launches are shorter than the bucket sort's.
+constexpr int64_t kPairSortMin = int64_t(1) << 17;
+static bool use_pair_sort(int64_t m, int32_t n) { return m >= kPairSortMin && bits_for(n) <= kPairSortBits; }
+
 void carve_super(Carver &c, int64_t m, int32_t n, int32_t rows, int32_t width, SuperScratch &s, int32_t G) {
     const int64_t keys = 2 * (m > 0 ? m : 1);  // both directions of every edge at most
     s.flags = c.take<uint32_t>(size_t(n) + 1);
@@ -462,14 +480,15 @@ void carve_super(Carver &c, int64_t m, int32_t n, int32_t rows, int32_t width, S
     s.nkeys = c.take<unsigned long long>(1);
     s.nnz = c.take<int64_t>(1);
     s.sketch = c.take<unsigned long long>(size_t(rows) * size_t(width) * size_t(G > 1 ? G : 1));
-    s.start = c.take<uint32_t>(size_t(keys) + 1);
-    s.supidx = c.take<int32_t>(size_t(keys));
+    s.moved = c.take<uint32_t>(1);
+    s.cut_cursor = c.take<unsigned long long>(1);
     const int64_t tiles = (keys + kRedTile - 1) / kRedTile;
     s.red_flags = c.take<uint32_t>(size_t(tiles) + 2);
     s.red_agg = c.take<unsigned long long>(size_t(tiles) + 1);
     s.red_incl = c.take<unsigned long long>(size_t(tiles) + 1);
     s.scan_tmp = c.take<char>(scan_tmp_bytes(int64_t(n) + 1));
     carve_sort(c, keys, false, s.sort_pairs);
+    if (use_pair_sort(m, n)) carve_pair_sort(c, m, n, s.ps);
 }
 
 int run_supergraph(const int32_t *edges, int64_t m, int32_t n, const int32_t *labels, const uint32_t *deg_est,
@@ -481,12 +500,12 @@ int run_supergraph(const int32_t *edges, int64_t m, int32_t n, const int32_t *la
     const int32_t *node_off = batch ? batch->node_off : nullptr;
     const size_t mats = batch ? size_t(batch->G) : 1;
     const int gn = grid_for(n, kThreads, sm_count() * 8);
-    const int shift = bits_for(n);  // supernode ids < K <= n fit in `shift` bits
     const int64_t cap = 2 * (m > 0 ? m : 1);
 
     // 1. dense relabel
     BGV_CUDA(cudaMemsetAsync(s.flags, 0, sizeof(uint32_t) * (size_t(n) + 1), st));
-    note_launch(), k_mark_labels<<<gn, kThreads, 0, st>>>(labels, n, s.flags, status);
+    BGV_CUDA(cudaMemsetAsync(s.moved, 0, sizeof(uint32_t), st));
+    note_launch(), k_mark_labels<<<gn, kThreads, 0, st>>>(labels, n, s.flags, s.moved, status);
     BGV_TRY(launch_status());
     BGV_TRY(scan_exclusive(s.flags, s.rank, n, nullptr, reinterpret_cast<unsigned long long *>(K_dev), false,
                            s.scan_tmp, st));
@@ -494,30 +513,37 @@ int run_supergraph(const int32_t *edges, int64_t m, int32_t n, const int32_t *la
     BGV_TRY(launch_status());
 
     // 2-3. both directions of every cut edge -> sorted (row, col) keys
-    BGV_CUDA(cudaMemsetAsync(s.nkeys, 0, sizeof(unsigned long long), st));
     SortBuffers pairs = s.sort_pairs;
+    const int64_t *nkeys = reinterpret_cast<const int64_t *>(s.nkeys);
+    const bool bucketed = use_pair_sort(m, n);
+    const uint32_t *guard = bucketed ? &s.ps.ctl->guard : nullptr;
+    unsigned long long *cut_cursor = bucketed ? s.cut_cursor : s.nkeys;
+    BGV_CUDA(cudaMemsetAsync(cut_cursor, 0, sizeof(unsigned long long), st));
+    if (bucketed)
+        BGV_TRY(pair_sort(edges, m, n, node_map, K_dev, s.moved, s.ps, pairs.keys[0], pairs.keys[1], s.nkeys, status,
+                          st));
     if (m > 0) {
         const int64_t chunks = ((m + 1) / 2 + kCutPairs - 1) / kCutPairs;
         note_launch(), k_cut_pairs<<<grid_for(chunks, 1, sm_count() * 8), kThreads, 0, st>>>(
-            edges, m, n, node_map, shift, pairs.keys[0], s.nkeys, status);
+            edges, m, n, node_map, K_dev, pairs.keys[0], cut_cursor, guard, status);
         BGV_TRY(launch_status());
     }
-    const int64_t *nkeys = reinterpret_cast<const int64_t *>(s.nkeys);
     // A row's pairs tie on their low 16 bits far too often for a local
     // finish on them (hub rows), so every digit gets an LSD pass.
+    const int end_bit = 2 * bits_for(n);  // supernode ids < K <= n
     int res = 0;
-    BGV_TRY(radix_sort(pairs, cap, nkeys, 2 * shift, st, &res, status));
+    if (bucketed)
+        BGV_TRY(radix_sort_guarded(pairs, cap, nkeys, end_bit, st, status, guard, 0u));
+    else
+        BGV_TRY(radix_sort(pairs, cap, nkeys, end_bit, st, &res, status));
     const unsigned long long *sorted = pairs.keys[res];
 
-    // 4. distinct pairs -> CSR entries and superedges, then multiplicities
+    // 4. distinct pairs -> CSR entries and superedges with their weights
     const int64_t tiles = (cap + kRedTile - 1) / kRedTile;
     BGV_CUDA(cudaMemsetAsync(s.red_flags, 0, sizeof(uint32_t) * (size_t(tiles) + 2), st));
     note_launch(), k_csr_reduce<<<unsigned(tiles), kThreads, 0, st>>>(
-        sorted, s.nkeys, cap, shift, K_dev, csr_off, csr_adj, s.start, s.supidx, ssrc, sdst, s.red_flags, s.red_agg,
-        s.red_incl, Es_dev, s.nnz, status, spin_limit());
-    BGV_TRY(launch_status());
-    note_launch(), k_csr_weights<<<grid_for(cap, kThreads, sm_count() * 8), kThreads, 0, st>>>(s.start, s.supidx, s.nnz,
-                                                                                             csr_w, sw);
+        sorted, s.nkeys, cap, K_dev, csr_off, csr_adj, csr_w, ssrc, sdst, sw, s.red_flags, s.red_agg, s.red_incl,
+        Es_dev, s.nnz, status, spin_limit());
     BGV_TRY(launch_status());
 
     // 5. community sizes
@@ -541,8 +567,8 @@ namespace {
 struct WaitCheckReduce {
     unsigned long long *keys, *nkeys, *agg, *incl;
     int64_t *K, *Es, *nnz;
-    int32_t *csr_off, *csr_adj, *supidx, *ssrc, *sdst;
-    uint32_t *start, *flags;
+    int32_t *csr_off, *csr_adj, *ssrc, *sdst;
+    uint32_t *csr_w, *sw, *flags;
 };
 void carve_wait_check_reduce(Carver &c, WaitCheckReduce &w) {
     const size_t n = 2 * kRedTile;
@@ -555,10 +581,10 @@ void carve_wait_check_reduce(Carver &c, WaitCheckReduce &w) {
     w.nnz = c.take<int64_t>(1);
     w.csr_off = c.take<int32_t>(2);
     w.csr_adj = c.take<int32_t>(n);
-    w.supidx = c.take<int32_t>(n);
+    w.csr_w = c.take<uint32_t>(n);
+    w.sw = c.take<uint32_t>(n);
     w.ssrc = c.take<int32_t>(n);
     w.sdst = c.take<int32_t>(n);
-    w.start = c.take<uint32_t>(n + 1);
     w.flags = c.take<uint32_t>(3);
 }
 }  // namespace
@@ -581,9 +607,9 @@ int wait_check_reduce(void *scratch, uint32_t *dev_status, cudaStream_t st) {
     BGV_CUDA(cudaMemcpyAsync(w.nkeys, &nk, sizeof(nk), cudaMemcpyHostToDevice, st));
     BGV_CUDA(cudaMemcpyAsync(w.K, &K, sizeof(K), cudaMemcpyHostToDevice, st));
     BGV_CUDA(cudaMemcpyAsync(w.flags + 2, &one, sizeof(one), cudaMemcpyHostToDevice, st));
-    note_launch(), k_csr_reduce<<<1, kThreads, 0, st>>>(w.keys, w.nkeys, int64_t(nk), 1, w.K, w.csr_off, w.csr_adj,
-                                                        w.start, w.supidx, w.ssrc, w.sdst, w.flags, w.agg, w.incl,
-                                                        w.Es, w.nnz, dev_status, spin_limit());
+    note_launch(), k_csr_reduce<<<1, kThreads, 0, st>>>(w.keys, w.nkeys, int64_t(nk), w.K, w.csr_off, w.csr_adj,
+                                                        w.csr_w, w.ssrc, w.sdst, w.sw, w.flags, w.agg, w.incl, w.Es,
+                                                        w.nnz, dev_status, spin_limit());
     BGV_TRY(launch_status());
     return cudaStreamSynchronize(st) == cudaSuccess ? BGV_OK : BGV_ECUDA;
 }
