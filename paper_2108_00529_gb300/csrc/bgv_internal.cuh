@@ -308,6 +308,8 @@ struct BatchView {
 };
 struct SketchScratch {
     uint32_t *deg;
+    uint16_t *local;    // endpoints by node range (null: counted with global atomics)
+    uint32_t *ranges;   // endpoints per range, then its list's cursor
 };
 void carve_sketch(Carver &c, int64_t m, int32_t n, int32_t rows, int32_t width, SketchScratch &s);
 // With `batch`, `sketch` holds G matrices of rows x width, one per graph.
