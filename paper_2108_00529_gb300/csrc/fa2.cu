@@ -7,17 +7,9 @@
 //               step's counters (the captured step has no memset nodes)
 //   radix sort  (key, body) pairs -> Morton order: LSD passes on the bits
 //               above 24, then each run of equal high bits ordered locally
-//   k_gather_moments
-//               bodies in Morton order, and exact prefix sums of (m, m*Ux,
-//               m*Uy) in 64/128-bit integers over that order (one pass,
-//               decoupled look-back), so a node's moments are a difference
-//   k_tree      binary radix tree over the sorted keys, one thread per
-//               internal node (exponential + binary search on key prefixes),
-//               and the quadtree cells: binary nodes whose 2-bit level
-//               exceeds their parent's, FP32 centre of mass from the exact
-//               moments
-//   k_preorder  cells and bodies laid out in depth-first pre-order with skip
-//               indices (positions from a prefix count of cells per body)
+//   k_tile*     bodies in Morton order, quadtree cells with FP32 centres from
+//               exact integer moments, and the depth-first pre-order with skip
+//               indices (tree.cuh)
 //   k_repulse   Barnes-Hut repulsion: one thread per body walks the
 //               pre-order array without a stack (accept -> skip past the
 //               subtree, open -> next element); every body takes its own
@@ -42,6 +34,7 @@
 
 #include "bgv_internal.cuh"
 #include "hsort.cuh"
+#include "tree.cuh"
 
 namespace bgv {
 
@@ -57,9 +50,6 @@ inline int64_t warp_share(int64_t K, int blocks) {
 }
 inline int node_blocks() { return sm_count() * 4 < kMaxNodeBlocks ? sm_count() * 4 : kMaxNodeBlocks; }
 
-typedef unsigned __int128 u128;
-
-
 __device__ __forceinline__ unsigned long long spread_bits(uint32_t v) {
     unsigned long long x = v;
     x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
@@ -69,9 +59,6 @@ __device__ __forceinline__ unsigned long long spread_bits(uint32_t v) {
     x = (x | (x << 1)) & 0x5555555555555555ull;
     return x;
 }
-
-// Exact power-of-two scale 2^-level for 0 <= level <= 126.
-__device__ __forceinline__ float pow2_neg(int level) { return __int_as_float((127 - level) << 23); }
 
 // ----------------------------------------------------------------- frame
 // Frame of a bounding box: origin, side = max extent * (1 + 2^-20).
@@ -212,14 +199,6 @@ __global__ void __launch_bounds__(kThreads) k_frame_seg(const float2 *__restrict
 }
 
 // ------------------------------------------------------------------ keys
-// Fixed-point position of a body in its graph's frame: U = floor(2^32 (p -
-// origin) / side) per axis, FP32 with round-to-nearest steps.
-__device__ __forceinline__ uint2 fixed_point(float2 p, float4 fr) {
-    const float ux = __fdiv_rn(__fsub_rn(p.x, fr.x), fr.z);
-    const float uy = __fdiv_rn(__fsub_rn(p.y, fr.y), fr.z);
-    return make_uint2(__float2uint_rz(__fmul_rn(ux, 4294967296.0f)), __float2uint_rz(__fmul_rn(uy, 4294967296.0f)));
-}
-
 // Morton key of the body's fixed-point position in its graph's frame; in the
 // batched form the graph id sits above the 2L Morton bits, so each graph's
 // bodies stay together and form their own subtree.
@@ -242,7 +221,7 @@ struct MortonOf {
 };
 
 // Also clears, for the kernels after it, the step's counters (2 words), the
-// moment look-back flags and the sort's digit counters: the launches that
+// tiles' flags and the sort's digit counters: the launches that
 // would otherwise clear them sit on the step's dependency chain.
 __global__ void __launch_bounds__(kThreads) k_keys(const float2 *__restrict__ pos, int64_t K,
                                                    const float4 *__restrict__ frames,
@@ -261,480 +240,6 @@ __global__ void __launch_bounds__(kThreads) k_keys(const float2 *__restrict__ po
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < K; i += stride) {
         keys[i] = morton_key(pos, frames, bgraph, L, i);
         vals[i] = uint32_t(i);
-    }
-}
-
-// ------------------------------------------------------------------ tree
-// Binary radix tree over the Morton-sorted keys, built node-parallel: for
-// internal node i (0 <= i < K-1) the direction, far end and split of its
-// range are found by exponential and binary search on delta(i, j), the
-// common-prefix length of keys i and j, with the positions breaking ties
-// between equal keys (Karras, HPG 2012).  No node waits for another.
-__device__ __forceinline__ int key_delta(const unsigned long long *__restrict__ keys, int64_t K, int keybits,
-                                         int64_t i, unsigned long long ki, int64_t j) {
-    if (j < 0 || j >= K) return -1;
-    const unsigned long long kj = __ldg(&keys[j]);
-    if (ki != kj) return __clzll(static_cast<long long>(ki ^ kj)) - (64 - keybits);
-    return keybits + __clz(static_cast<int>(uint32_t(i) ^ uint32_t(j)));
-}
-
-// Exact moment prefix sums over the Morton order: P[s] = sum over bodies
-// t < s of (m, m*Ux, m*Uy), in 64/128-bit integers, so every node's moments
-// are P[last+1] - P[first] (exact, order-free).
-constexpr int kMomItems = 4;
-constexpr int kMomTile = kThreads * kMomItems;
-
-struct Mom {
-    unsigned long long M;
-    u128 X, Y;
-};
-__device__ __forceinline__ Mom mom_add(Mom a, const Mom &b) {
-    a.M += b.M;
-    a.X += b.X;
-    a.Y += b.Y;
-    return a;
-}
-__device__ __forceinline__ Mom mom_shfl_up(const Mom &a, int d) {
-    Mom r;
-    r.M = __shfl_up_sync(0xFFFFFFFFu, a.M, d);
-    const unsigned long long xl = __shfl_up_sync(0xFFFFFFFFu, static_cast<unsigned long long>(a.X), d);
-    const unsigned long long xh = __shfl_up_sync(0xFFFFFFFFu, static_cast<unsigned long long>(a.X >> 64), d);
-    const unsigned long long yl = __shfl_up_sync(0xFFFFFFFFu, static_cast<unsigned long long>(a.Y), d);
-    const unsigned long long yh = __shfl_up_sync(0xFFFFFFFFu, static_cast<unsigned long long>(a.Y >> 64), d);
-    r.X = (u128(xh) << 64) | xl;
-    r.Y = (u128(yh) << 64) | yl;
-    return r;
-}
-__device__ __forceinline__ void mom_store(Mom v, unsigned long long *PM, ulonglong2 *PX, ulonglong2 *PY, int64_t s) {
-    PM[s] = v.M;
-    PX[s] = make_ulonglong2(static_cast<unsigned long long>(v.X), static_cast<unsigned long long>(v.X >> 64));
-    PY[s] = make_ulonglong2(static_cast<unsigned long long>(v.Y), static_cast<unsigned long long>(v.Y >> 64));
-}
-__device__ __forceinline__ Mom mom_load(const unsigned long long *PM, const ulonglong2 *PX, const ulonglong2 *PY,
-                                        int64_t s) {
-    const ulonglong2 x = PX[s], y = PY[s];
-    return Mom{PM[s], (u128(x.y) << 64) | x.x, (u128(y.y) << 64) | y.x};
-}
-
-// Moment prefix of one body in one 32-byte record (one sector per access):
-// M in 64 bits, the coordinate sums in 96 (their totals stay below 2^95).
-struct __align__(32) MomP {
-    unsigned long long M, xl, yl;
-    uint32_t xh, yh;
-};
-__device__ __forceinline__ uint4 momp_first_half(unsigned long long M, u128 X) {
-    return make_uint4(uint32_t(M), uint32_t(M >> 32), uint32_t(X), uint32_t(X >> 32));
-}
-__device__ __forceinline__ uint4 momp_second_half(u128 X, u128 Y) {
-    return make_uint4(uint32_t(Y), uint32_t(Y >> 32), uint32_t(X >> 64), uint32_t(Y >> 64));
-}
-__device__ __forceinline__ void momp_store(MomP *P, int64_t s, const Mom &v) {
-    uint4 *p = reinterpret_cast<uint4 *>(P + s);
-    p[0] = momp_first_half(v.M, v.X);
-    p[1] = momp_second_half(v.X, v.Y);
-}
-__device__ __forceinline__ Mom momp_load(const MomP *P, int64_t s) {
-    const uint4 *p = reinterpret_cast<const uint4 *>(P + s);
-    const uint4 a = p[0], b = p[1];
-    const unsigned long long xl = (static_cast<unsigned long long>(a.w) << 32) | a.z;
-    const unsigned long long yl = (static_cast<unsigned long long>(b.y) << 32) | b.x;
-    return Mom{(static_cast<unsigned long long>(a.y) << 32) | a.x, (u128(b.z) << 64) | xl, (u128(b.w) << 64) | yl};
-}
-
-// Block-wide exclusive scan of one Mom per thread; returns the prefix and
-// the block total.
-__device__ __forceinline__ Mom mom_block_exclusive(Mom v, Mom *total) {
-    __shared__ unsigned long long sM[kThreads / 32];
-    __shared__ ulonglong2 sX[kThreads / 32], sY[kThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    Mom inc = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const Mom o = mom_shfl_up(inc, d);
-        if (lane >= d) inc = mom_add(inc, o);
-    }
-    if (lane == 31) mom_store(inc, sM, sX, sY, warp);
-    __syncthreads();
-    Mom before{0ull, 0, 0}, all{0ull, 0, 0};
-    for (int w = 0; w < kThreads / 32; ++w) {
-        const Mom t = mom_load(sM, sX, sY, w);
-        if (w < warp) before = mom_add(before, t);
-        all = mom_add(all, t);
-    }
-    __syncthreads();
-    *total = all;
-    Mom ex = mom_add(before, inc);
-    ex.M -= v.M;
-    ex.X -= v.X;
-    ex.Y -= v.Y;
-    return ex;
-}
-
-// Sorted bodies and moment prefix sums in one pass, with a decoupled
-// look-back across tiles.  Tiles of kMomTile sorted positions are taken in
-// order from a counter (a tile waits only on tiles already taken, so the
-// waits end); a thread gathers kMomItems consecutive positions: the body's
-// position, mass and index (body[s]), and its fixed-point coordinates
-// recomputed from the position as the keys were.  The tile publishes its
-// total, the block adds the totals or inclusive prefixes of the tiles before
-// it (up to kMomLookBack at a time), and the prefix records go out through
-// shared memory so that every store is coalesced.  Also clears the
-// per-body cell counters that k_tree fills.  P[K], the grand total, is
-// written by the last tile.
-struct MomTile {
-    unsigned long long M, xl, xh, yl, yh, pad;
-};
-enum : uint32_t { kMomAgg = 1u, kMomIncl = 2u };  // look-back flags (0: nothing published)
-constexpr int kMomLBItems = 4;                          // predecessors per thread and round
-constexpr int kMomLookBack = kThreads * kMomLBItems;    // predecessors per round
-
-__device__ __forceinline__ void mom_tile_store(MomTile *t, const Mom &v) {
-    t->M = v.M;
-    t->xl = static_cast<unsigned long long>(v.X);
-    t->xh = static_cast<unsigned long long>(v.X >> 64);
-    t->yl = static_cast<unsigned long long>(v.Y);
-    t->yh = static_cast<unsigned long long>(v.Y >> 64);
-}
-__device__ __forceinline__ Mom mom_tile_load(const MomTile *t) {  // from L2: written by other blocks
-    return Mom{__ldcg(&t->M), (u128(__ldcg(&t->xh)) << 64) | __ldcg(&t->xl),
-               (u128(__ldcg(&t->yh)) << 64) | __ldcg(&t->yl)};
-}
-__device__ __forceinline__ Mom mom_warp_sum(Mom v) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        Mom o;
-        o.M = __shfl_xor_sync(0xFFFFFFFFu, v.M, d);
-        const unsigned long long xl = __shfl_xor_sync(0xFFFFFFFFu, static_cast<unsigned long long>(v.X), d);
-        const unsigned long long xh = __shfl_xor_sync(0xFFFFFFFFu, static_cast<unsigned long long>(v.X >> 64), d);
-        const unsigned long long yl = __shfl_xor_sync(0xFFFFFFFFu, static_cast<unsigned long long>(v.Y), d);
-        const unsigned long long yh = __shfl_xor_sync(0xFFFFFFFFu, static_cast<unsigned long long>(v.Y >> 64), d);
-        o.X = (u128(xh) << 64) | xl;
-        o.Y = (u128(yh) << 64) | yl;
-        v = mom_add(v, o);
-    }
-    return v;
-}
-// Staging slot of tile element e: one 16-byte pad after every 8 elements, so
-// the per-thread writes (stride 8) fall in different banks.
-__device__ __forceinline__ int stage_slot(int e) { return e + (e >> 3); }
-__global__ void __launch_bounds__(kThreads, 4) k_gather_moments(
-    const uint32_t *__restrict__ perm, int64_t K, const float2 *__restrict__ pos, const uint32_t *__restrict__ mass,
-    const float4 *__restrict__ frames, const int32_t *__restrict__ bgraph, float4 *__restrict__ body,
-    MomP *__restrict__ P, uint32_t *__restrict__ start_count, uint32_t *__restrict__ start_levels, uint32_t *flags, MomTile *agg,
-    MomTile *incl, uint32_t *dev_status, int spin_limit) {
-    __shared__ uint4 stage[2 * (kMomTile + kMomTile / 8)];  // bodies, then two halves per prefix record
-    __shared__ unsigned tile_sh;
-    __shared__ int near_sh;
-    __shared__ unsigned long long red_sh[kThreads / 32][5];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t tiles = (K + kMomTile - 1) / kMomTile;
-    if (threadIdx.x == 0) tile_sh = atomicAdd(&flags[tiles], 1u);
-    __syncthreads();
-    const int64_t tile = tile_sh;
-    if (tile >= tiles) return;
-    const int64_t t0 = tile * kMomTile;
-    const int64_t s0 = t0 + int64_t(threadIdx.x) * kMomItems;
-    // sorted position s holds body perm[s]
-    uint32_t m[kMomItems], ux[kMomItems], uy[kMomItems];
-    Mom acc{0ull, 0, 0};
-#pragma unroll
-    for (int k = 0; k < kMomItems; ++k) {
-        const int64_t sk = s0 + k;
-        uint4 b = make_uint4(0u, 0u, 0u, 0u);
-        m[k] = 0u;
-        ux[k] = 0u;
-        uy[k] = 0u;
-        if (sk < K) {
-            const uint32_t i = perm[sk];
-            const float2 p = pos[i];
-            const uint2 U = fixed_point(p, frames[bgraph ? bgraph[i] : 0]);
-            m[k] = mass[i];
-            ux[k] = U.x;
-            uy[k] = U.y;
-            b = make_uint4(__float_as_uint(p.x), __float_as_uint(p.y), __float_as_uint(__uint2float_rn(m[k])), i);
-        }
-        stage[stage_slot(threadIdx.x * kMomItems + k)] = b;
-        acc.M += m[k];
-        acc.X += u128(m[k]) * ux[k];
-        acc.Y += u128(m[k]) * uy[k];
-    }
-    Mom total;
-    Mom run = mom_block_exclusive(acc, &total);  // synchronises: the staged bodies are complete
-    if (threadIdx.x == 0) {
-        mom_tile_store(tile == 0 ? &incl[0] : &agg[tile], total);
-        __threadfence();
-        atomicExch(&flags[tile], tile == 0 ? kMomIncl : kMomAgg);
-    }
-#pragma unroll
-    for (int r = 0; r < kMomItems; ++r) {
-        const int e = r * kThreads + threadIdx.x;
-        const int64_t sk = t0 + e;
-        if (sk < K) {
-            const uint4 v = stage[stage_slot(e)];
-            body[sk] = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z),
-                                   __uint_as_float(v.w));
-            start_count[sk] = 0u;
-            start_levels[sk] = 0u;
-        }
-    }
-    // Look-back by the whole block, kMomLookBack predecessors per round: the
-    // nearest tile with an inclusive prefix in the window ends it; the tiles
-    // after it must have published their totals.
-    Mom excl{0ull, 0, 0};
-    {
-        int64_t hi = tile - 1;
-        int spins = 0;
-        while (hi >= 0) {
-            if (threadIdx.x == 0) near_sh = -1;
-            __syncthreads();
-            uint32_t f[kMomLBItems];
-#pragma unroll
-            for (int r = 0; r < kMomLBItems; ++r) {
-                const int64_t idx = hi - (r * kThreads + threadIdx.x);
-                f[r] = idx >= 0 ? *reinterpret_cast<volatile uint32_t *>(&flags[idx]) : 0u;
-                if (idx >= 0 && f[r] == kMomIncl) atomicMax(&near_sh, int(idx));
-            }
-            __syncthreads();
-            const int64_t near = near_sh;
-            const int64_t win_lo = hi - kMomLookBack + 1 > 0 ? hi - kMomLookBack + 1 : 0;
-            const int64_t lo = near >= 0 ? near : win_lo;
-            bool pending = false;
-#pragma unroll
-            for (int r = 0; r < kMomLBItems; ++r) {
-                const int64_t idx = hi - (r * kThreads + threadIdx.x);
-                pending |= idx >= lo && f[r] == 0u;
-            }
-            if (__syncthreads_or(pending)) {
-                if (++spins > spin_limit) {
-                    if (threadIdx.x == 0) raise_status(dev_status, BGV_DEV_TIMEOUT);
-                    break;
-                }
-                __nanosleep(64);
-                continue;
-            }
-            __threadfence();
-            Mom v{0ull, 0, 0};
-#pragma unroll
-            for (int r = 0; r < kMomLBItems; ++r) {
-                const int64_t idx = hi - (r * kThreads + threadIdx.x);
-                if (idx >= lo) v = mom_add(v, mom_tile_load(f[r] == kMomIncl ? &incl[idx] : &agg[idx]));
-            }
-            v = mom_warp_sum(v);
-            if (lane == 0) {
-                red_sh[warp][0] = v.M;
-                red_sh[warp][1] = static_cast<unsigned long long>(v.X);
-                red_sh[warp][2] = static_cast<unsigned long long>(v.X >> 64);
-                red_sh[warp][3] = static_cast<unsigned long long>(v.Y);
-                red_sh[warp][4] = static_cast<unsigned long long>(v.Y >> 64);
-            }
-            __syncthreads();
-#pragma unroll
-            for (int w = 0; w < kThreads / 32; ++w)
-                excl = mom_add(excl, Mom{red_sh[w][0], (u128(red_sh[w][2]) << 64) | red_sh[w][1],
-                                         (u128(red_sh[w][4]) << 64) | red_sh[w][3]});
-            if (near >= 0) break;
-            hi = lo - 1;
-        }
-    }
-    if (threadIdx.x == 0 && tile > 0) {
-        mom_tile_store(&incl[tile], mom_add(excl, total));
-        __threadfence();
-        atomicExch(&flags[tile], kMomIncl);
-    }
-    const Mom tile_pre = excl;
-    __syncthreads();  // the bodies have left the staging buffer
-    run = mom_add(run, tile_pre);
-    if (tile == tiles - 1 && threadIdx.x == 0) momp_store(P, K, mom_add(tile_pre, total));
-    // the prefix records through the staging buffer (the bodies have left
-    // it), then out with consecutive threads on consecutive 16-byte halves
-    uint4 *stage2 = stage;
-    {
-        unsigned long long rm = run.M;
-        u128 rx = run.X, ry = run.Y;
-#pragma unroll
-        for (int k = 0; k < kMomItems; ++k) {
-            const int slot = 2 * stage_slot(threadIdx.x * kMomItems + k);
-            stage2[slot] = momp_first_half(rm, rx);
-            stage2[slot + 1] = momp_second_half(rx, ry);
-            rm += m[k];
-            rx += u128(m[k]) * ux[k];
-            ry += u128(m[k]) * uy[k];
-        }
-    }
-    __syncthreads();
-    uint4 *P4 = reinterpret_cast<uint4 *>(P);
-#pragma unroll
-    for (int r = 0; r < 2 * kMomItems; ++r) {
-        const int u = r * kThreads + threadIdx.x;  // 16-byte half u of the tile: record u / 2
-        if (t0 + (u >> 1) < K) P4[2 * t0 + u] = stage2[2 * stage_slot(u >> 1) + (u & 1)];
-    }
-}
-
-// 2-bit quadtree level of a binary node with split prefix length delta (the
-// graph bits come first): -1 above a graph's root, L for coincident keys.
-__device__ __forceinline__ int node_level(int delta, int kb, int L, int gbits) {
-    return delta >= kb ? L : (delta < gbits ? -1 : ((delta - gbits) >> 1));
-}
-
-// Binary radix tree and quadtree cells in one pass, one thread per internal
-// node (Karras, HPG 2012): the node's range and split prefix length come
-// from an exponential and a binary search on key prefixes.  Its parent's
-// split is the nearer of the two pairs just outside the range (the far one
-// shares a shorter prefix), so the node knows its parent's level without
-// waiting for anyone.  A node is a quadtree cell when its level exceeds its
-// parent's (a chain of single-child cells collapses into its deepest cell,
-// which takes the opening test for the whole chain).  For each cell: FP32
-// centre from the exact moments, mass, and the squared side used by the
-// opening test (+inf for a leaf that is never accepted); cells are counted
-// per first body, and their levels recorded there, for the pre-order
-// layout.
-// A binary node can only be a quadtree cell if the split inside its range
-// lies at a deeper 2-bit level than the split just outside it; both follow
-// from the keys of the node and its two neighbours.  The test runs over all
-// nodes (three coalesced key loads each) and lists the candidates, one
-// atomic per block; the range searches then run densely over the list.
-__global__ void __launch_bounds__(kThreads) k_tree_mark(const unsigned long long *__restrict__ keys, int64_t K,
-                                                        int L, int gbits, int8_t *__restrict__ cell_level,
-                                                        uint32_t *__restrict__ cand, uint32_t *cand_count) {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    bool is_cand = false;
-    if (i < K - 1) {
-        const int kb = 2 * L + gbits;
-        const unsigned long long ki = __ldg(&keys[i]);
-        const int dnext = key_delta(keys, K, kb, i, ki, i + 1), dprev = key_delta(keys, K, kb, i, ki, i - 1);
-        const int d = dnext > dprev ? 1 : -1;
-        const int dmin = d > 0 ? dprev : dnext;
-        // The node's split lies between its parent's (dmin) and that of the
-        // pair (i, i + d) inside its range: when those two share a level,
-        // the node shares it with its parent and is no cell.
-        is_cand = node_level(d > 0 ? dnext : dprev, kb, L, gbits) != node_level(dmin, kb, L, gbits);
-        if (!is_cand) cell_level[i] = -1;
-    }
-    // block-wide compaction: one atomic per block on the shared counter
-    __shared__ uint32_t warp_n[kThreads / 32], block_base;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned mask = __ballot_sync(0xFFFFFFFFu, is_cand);
-    if (lane == 0) warp_n[warp] = uint32_t(__popc(mask));
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t t = 0;
-        for (int w = 0; w < kThreads / 32; ++w) {
-            const uint32_t c = warp_n[w];
-            warp_n[w] = t;
-            t += c;
-        }
-        block_base = t ? atomicAdd(cand_count, t) : 0u;
-    }
-    __syncthreads();
-    if (is_cand) cand[block_base + warp_n[warp] + __popc(mask & ((1u << lane) - 1u))] = uint32_t(i);
-}
-
-// Binary radix tree and quadtree cells, one thread per listed candidate
-// (Karras, HPG 2012): the node's range and split prefix length come from an
-// exponential and a binary search on key prefixes.  Its parent's split is
-// the nearer of the two pairs just outside the range (the far one shares a
-// shorter prefix), so the node knows its parent's level without waiting for
-// anyone.  A node is a quadtree cell when its level exceeds its parent's (a
-// chain of single-child cells collapses into its deepest cell, which takes
-// the opening test for the whole chain).  For each cell: FP32 centre from
-// the exact moments, mass, and the squared side used by the opening test
-// (+inf for a leaf that is never accepted); cells are counted per first
-// body, and their levels recorded there, for the pre-order layout.
-__global__ void __launch_bounds__(kThreads) k_tree(const unsigned long long *__restrict__ keys, int64_t K, int L,
-                                                   int gbits, int leaf_cap, const float4 *__restrict__ frames,
-                                                   const int32_t *__restrict__ bgraph,
-                                                   const MomP *__restrict__ P, int2 *__restrict__ range,
-                                                   int8_t *__restrict__ cell_level, float4 *__restrict__ cell,
-                                                   uint32_t *__restrict__ start_count,
-                                                   uint32_t *__restrict__ start_levels,
-                                                   unsigned long long *tree_nodes, const uint32_t *__restrict__ cand,
-                                                   const uint32_t *cand_count) {
-    const int64_t count = *cand_count;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    const int kb = 2 * L + gbits;
-    uint32_t tops = 0;
-    for (int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; q < count; q += stride) {
-        const int64_t i = cand[q];
-        const unsigned long long ki = __ldg(&keys[i]);
-        const int dnext = key_delta(keys, K, kb, i, ki, i + 1), dprev = key_delta(keys, K, kb, i, ki, i - 1);
-        const int d = dnext > dprev ? 1 : -1;
-        const int dmin = d > 0 ? dprev : dnext;
-        int64_t lmax = 2;
-        while (key_delta(keys, K, kb, i, ki, i + lmax * d) > dmin) lmax <<= 1;
-        int64_t l = 0;
-        for (int64_t t = lmax >> 1; t >= 1; t >>= 1)
-            if (key_delta(keys, K, kb, i, ki, i + (l + t) * d) > dmin) l += t;
-        const int64_t j = i + l * d;
-        const int dnode = key_delta(keys, K, kb, i, ki, j);
-        const int64_t first = i < j ? i : j, last = i < j ? j : i;
-        const int lev = node_level(dnode, kb, L, gbits);
-        const int par_lev = node_level(dmin, kb, L, gbits);
-        const bool top = par_lev < lev;
-        cell_level[i] = static_cast<int8_t>(top ? lev : -1);
-        if (top) {
-            ++tops;
-            range[i] = make_int2(int32_t(first), int32_t(last));
-            const int cnt = int(last - first) + 1;
-            const bool leaf = cnt <= leaf_cap || lev >= L;
-            // A leaf made by the depth limit (coincident keys, more than
-            // leaf_cap bodies) hides a chain of non-leaf cells with the same
-            // bodies between its parent's level and L; the deepest of them,
-            // at level L - 1, takes the opening test for the whole chain.
-            const bool testable = leaf && cnt > leaf_cap && par_lev + 1 <= L - 1;
-            // positions of graph g in Morton order are its index range too
-            const float4 fr = frames[bgraph ? bgraph[first] : 0];
-            const Mom hi = momp_load(P, last + 1), lo = momp_load(P, first);
-            const unsigned long long M = hi.M - lo.M;
-            const u128 X = hi.X - lo.X, Y = hi.Y - lo.Y;
-            const uint32_t qx = M ? uint32_t(X / M) : 0u, qy = M ? uint32_t(Y / M) : 0u;
-            const float two_m32 = 2.3283064365386963e-10f;  // 2^-32
-            const float cx = __fadd_rn(fr.x, __fmul_rn(fr.z, __fmul_rn(__uint2float_rn(qx), two_m32)));
-            const float cy = __fadd_rn(fr.y, __fmul_rn(fr.z, __fmul_rn(__uint2float_rn(qy), two_m32)));
-            const float sl = __fmul_rn(fr.z, pow2_neg(testable ? L - 1 : lev));
-            const float side2 = (leaf && !testable) ? INFINITY : __fmul_rn(sl, sl);
-            cell[i] = make_float4(cx, cy, __ull2float_rn(M), side2);
-            atomicAdd(&start_count[first], 1u);
-            atomicOr(&start_levels[first], 1u << lev);
-        }
-    }
-#pragma unroll
-    for (int dd = 16; dd > 0; dd >>= 1) tops += __shfl_xor_sync(0xFFFFFFFFu, tops, dd);
-    if ((threadIdx.x & 31) == 0 && tops) atomicAdd(tree_nodes, static_cast<unsigned long long>(tops));
-}
-
-// Pre-order layout of cells and bodies.  With T[s] = number of cells whose
-// first body precedes s (exclusive scan of the per-body counts):
-//   body s           -> s + T[s+1]       (every cell starting at or before s
-//                                          comes first)
-//   cell [a, b]      -> a + T[a] + (its ancestors that also start at a)
-//   skip(cell [a,b]) -> b + 1 + T[b+1]   (the element after its subtree)
-// The cells starting at body a are nested with strictly increasing levels,
-// so a cell's ancestors among them are those of a lower level in
-// start_levels[a].  Elements are float4 (x, y, mass, side^2), side^2 = -1
-// for a body.
-__global__ void __launch_bounds__(kThreads) k_preorder(int64_t K, const int2 *__restrict__ range,
-                                                       const int8_t *__restrict__ cell_level,
-                                                       const uint32_t *__restrict__ start_levels,
-                                                       const float4 *__restrict__ cell,
-                                                       const uint32_t *__restrict__ T,
-                                                       const float4 *__restrict__ body, float4 *__restrict__ geo,
-                                                       int32_t *__restrict__ skip) {
-    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (t < K) {
-        const int64_t pre = t + T[t + 1];
-        const float4 b = body[t];
-        geo[pre] = make_float4(b.x, b.y, b.z, -1.0f);
-        skip[pre] = int32_t(pre + 1);
-    }
-    if (t < K - 1) {
-        const int lev = cell_level[t];
-        if (lev >= 0) {
-            const int2 rg = range[t];
-            const int dep = __popc(start_levels[rg.x] & ((1u << lev) - 1u));
-            const int64_t pre = rg.x + int64_t(T[rg.x]) + dep;
-            geo[pre] = cell[t];
-            skip[pre] = int32_t(int64_t(rg.y) + 1 + T[rg.y + 1]);
-        }
     }
 }
 
@@ -1219,7 +724,7 @@ __device__ __forceinline__ void xsum_warp(XSum &S, XSum &T) {
 }
 
 template <bool kB>
-__global__ void __launch_bounds__(kThreads) k_tail(int64_t K, int64_t per, const float2 *__restrict__ att,
+__global__ void __launch_bounds__(kThreads, 3) k_tail(int64_t K, int64_t per, const float2 *__restrict__ att,
                                                    const uint32_t *__restrict__ mass, float2 *__restrict__ pos,
                                                    const float2 *__restrict__ Frep, float kg, int strong,
                                                    float2 *__restrict__ F, float2 *__restrict__ Fprev, XPart *part,
@@ -1426,17 +931,8 @@ struct Fa2Scratch {
     SortBuffers sort;
     RunFixBuffers runfix;
     float4 *body;          // sorted bodies: x, y, mass, index
-    int2 *range;           // per binary node that is a cell: its bodies
-    int8_t *cell_level;    // per binary node: its level if a cell, else -1
-    MomP *P;               // moment prefix sums, K + 1 records
-    uint32_t *mom_flags;   // look-back flags per tile, the tile counter, the tree candidate count
-    uint32_t *cand;        // binary nodes that may be quadtree cells
-    MomTile *mom_agg, *mom_incl;
-    float4 *cell;          // per binary node: centre, mass, side^2 (cells only)
-    uint32_t *start_count; // cells per first body
-    uint32_t *start_levels;  // levels of the cells per first body (bit mask)
-    uint32_t *T;           // exclusive scan of start_count, K + 1 entries
-    void *scan_tmp;
+    TileArrays tree;
+    uint32_t *T;           // cells whose first body precedes each body, K + 1 entries
     float4 *geo;           // pre-order elements (cells and bodies)
     int32_t *skip;         // pre-order index after each element's subtree
     float2 *Frep;
@@ -1457,19 +953,8 @@ static void carve_fa2(Carver &c, int64_t K, int64_t nnz, int32_t G, Fa2Scratch &
     carve_sort(c, int64_t(k), true, s.sort);
     carve_run_fix(c, int64_t(k), s.runfix);
     s.body = c.take<float4>(k);
-    const size_t tiles = (k + kMomTile - 1) / kMomTile;
-    s.range = c.take<int2>(k);
-    s.cell_level = c.take<int8_t>(k);
-    s.P = c.take<MomP>(k + 1);
-    s.mom_flags = c.take<uint32_t>(tiles + 2);  // look-back flags, tile counter, tree candidate count
-    s.mom_agg = c.take<MomTile>(tiles);
-    s.mom_incl = c.take<MomTile>(tiles);
-    s.cell = c.take<float4>(k);
-    s.cand = c.take<uint32_t>(k);
-    s.start_count = c.take<uint32_t>(k + 1);
-    s.start_levels = c.take<uint32_t>(k);
+    carve_tiles(c, int64_t(k), s.tree);
     s.T = c.take<uint32_t>(k + 1);
-    s.scan_tmp = c.take<char>(scan_tmp_bytes(int64_t(k) + 1));
     s.geo = c.take<float4>(2 * k);
     s.skip = c.take<int32_t>(2 * k);
     s.Frep = c.take<float2>(k);
@@ -1516,31 +1001,27 @@ int run_fa2_init(int64_t K, const bgv_fa2_params &p, float *pos, float *Fprev, d
     return launch_status();
 }
 
-// Bounded-wait self check of the moment pass: one block as tile 1 of two
-// tiles of bodies (all at the origin, body 0 everywhere, mass 0, frame side
-// 1) whose tile 0 never runs, so its look-back must give up at the spin
-// limit.  Writes stay within the two tiles' bodies and prefix records.
+// Bounded-wait self check of the moment look-back: one k_tile block as tile 1 of
+// two tiles of bodies (all at the origin, body 0 everywhere, mass 0, frame side
+// 1) whose tile 0 never runs, so its look-back must give up at the spin limit.
+// Equal keys make no cells, and every write stays within the two tiles' arrays.
 namespace {
 struct WaitCheckMoments {
-    uint32_t *perm, *mass, *start_count, *start_levels, *flags;
+    unsigned long long *keys;
+    uint32_t *perm, *mass;
     float2 *pos;
     float4 *frame, *body;
-    MomP *P;
-    MomTile *agg, *incl;
+    TileArrays tree;
 };
 void carve_wait_check_moments(Carver &c, WaitCheckMoments &w) {
-    const size_t K = 2 * kMomTile;
+    const size_t K = 2 * kTile;
+    w.keys = c.take<unsigned long long>(K);
     w.perm = c.take<uint32_t>(K);
     w.mass = c.take<uint32_t>(K);
-    w.start_count = c.take<uint32_t>(K);
-    w.start_levels = c.take<uint32_t>(K);
-    w.flags = c.take<uint32_t>(3);
     w.pos = c.take<float2>(K);
     w.frame = c.take<float4>(1);
     w.body = c.take<float4>(K);
-    w.P = c.take<MomP>(K + 1);
-    w.agg = c.take<MomTile>(2);
-    w.incl = c.take<MomTile>(2);
+    carve_tiles(c, int64_t(K), w.tree);
 }
 }  // namespace
 
@@ -1559,10 +1040,9 @@ int wait_check_moments(void *scratch, uint32_t *dev_status, cudaStream_t st) {
     const float4 frame = make_float4(0.0f, 0.0f, 1.0f, 0.0f);
     const uint32_t one = 1u;  // the tile counter (after the two tiles' flags)
     BGV_CUDA(cudaMemcpyAsync(w.frame, &frame, sizeof(frame), cudaMemcpyHostToDevice, st));
-    BGV_CUDA(cudaMemcpyAsync(w.flags + 2, &one, sizeof(one), cudaMemcpyHostToDevice, st));
-    note_launch(), k_gather_moments<<<1, kThreads, 0, st>>>(w.perm, 2 * kMomTile, w.pos, w.mass, w.frame, nullptr,
-                                                            w.body, w.P, w.start_count, w.start_levels, w.flags,
-                                                            w.agg, w.incl, dev_status, spin_limit());
+    BGV_CUDA(cudaMemcpyAsync(w.tree.flags + 2, &one, sizeof(one), cudaMemcpyHostToDevice, st));
+    note_launch(), k_tile<<<1, kTileThreads, 0, st>>>(w.keys, w.perm, 2 * kTile, w.pos, w.mass, w.frame, nullptr, 24, 0,
+                                                      1, w.body, w.tree, dev_status, spin_limit());
     BGV_TRY(launch_status());
     return cudaStreamSynchronize(st) == cudaSuccess ? BGV_OK : BGV_ECUDA;
 }
@@ -1727,23 +1207,22 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
                                                                                          s.frame, &hdr->bbox_ticket);
         BGV_TRY(launch_status());
     }
-    const int64_t mom_tiles = (K + kMomTile - 1) / kMomTile;
     // the sorted order lands in the buffer pair the radix sort ends in, so
     // the next iteration finds its hint there whichever sort made it
     const int res = radix_sort_high_result(K, 2 * L + gbits);
     if (hinted && fa2_order() == 1 && K <= hs_max_keys()) {
         // the previous iteration's sorted ids are the hint; the sort also
-        // clears the step counters and the moment flags, as k_keys does
+        // clears the step counters and the tiles' flags, as k_keys does
         const MortonOf key_of{pos, s.frame, s.bgraph, L};
         HsClears clr;
         clr.u64 = &hdr->interactions;  // interactions, tree_nodes
         clr.n_u64 = 2;
-        clr.u32 = s.mom_flags;
-        clr.n_u32 = mom_tiles + 2;
+        clr.u32 = s.tree.flags;
+        clr.n_u32 = tile_flag_words(K);
         const uint32_t *hint = s.sort.vals[res];
         BGV_TRY(hinted_sort_samples(key_of, hint, K, s.hs, &hdr->status, st, clr));
         BGV_TRY(mark(1));
-        // the pre-order arrays are free until k_preorder: the buckets' slots
+        // the pre-order arrays are free until k_tile_emit: the buckets' slots
         unsigned long long *slot_key = reinterpret_cast<unsigned long long *>(s.geo);
         uint32_t *slot_id = reinterpret_cast<uint32_t *>(slot_key + K);
         BGV_TRY(hinted_sort_place(key_of, hint, K, s.hs, s.sort.keys[res ^ 1], s.sort.vals[res ^ 1], slot_key, slot_id,
@@ -1751,7 +1230,7 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
     } else {
         const int gk = grid_for(K, kThreads, sm_count() * 16);
         note_launch(), k_keys<<<gk, kThreads, 0, st>>>(pos, K, s.frame, s.bgraph, L, s.sort.keys[0], s.sort.vals[0],
-                                                       &hdr->interactions, s.mom_flags, mom_tiles + 2, s.sort.counts,
+                                                       &hdr->interactions, s.tree.flags, tile_flag_words(K), s.sort.counts,
                                                        sort_counter_words());
         BGV_TRY(launch_status());
         BGV_TRY(mark(1));
@@ -1760,28 +1239,19 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
         if (got != res) return BGV_EINVAL;  // radix_sort_high_result disagrees with the sort
     }
     BGV_TRY(mark(2));
-    {
-        note_launch(), k_gather_moments<<<unsigned(mom_tiles), kThreads, 0, st>>>(
-            s.sort.vals[res], K, pos, mass, s.frame, s.bgraph, s.body, s.P, s.start_count,
-            s.start_levels, s.mom_flags, s.mom_agg, s.mom_incl, &hdr->status, spin_limit());
-        BGV_TRY(launch_status());
-    }
-    BGV_TRY(mark(3));
     if (K >= 2) {
-        const unsigned gt = unsigned((K + kThreads - 1) / kThreads);
-        const unsigned gi = unsigned((K - 1 + kThreads - 1) / kThreads);
-        uint32_t *cand_count = s.mom_flags + mom_tiles + 1;  // cleared by k_keys
-        note_launch(), k_tree_mark<<<gi, kThreads, 0, st>>>(s.sort.keys[res], K, L, gbits, s.cell_level, s.cand,
-                                                            cand_count);
+        const unsigned tiles = unsigned(tile_count(K));
+        note_launch(), k_tile<<<tiles, kTileThreads, 0, st>>>(s.sort.keys[res], s.sort.vals[res], K, pos, mass, s.frame,
+                                                              s.bgraph, L, gbits, p.leaf_cap, s.body, s.tree,
+                                                              &hdr->status, spin_limit());
         BGV_TRY(launch_status());
-        note_launch(), k_tree<<<grid_for(K, kThreads, sm_count() * 8), kThreads, 0, st>>>(
-            s.sort.keys[res], K, L, gbits, p.leaf_cap, s.frame, s.bgraph, s.P, s.range, s.cell_level, s.cell,
-            s.start_count, s.start_levels, &hdr->tree_nodes, s.cand, cand_count);
+        BGV_TRY(mark(3));
+        const unsigned per = kTileThreads / 32;  // tiles per block
+        note_launch(), k_tile_cross<<<(tiles + per - 1) / per, kTileThreads, 0, st>>>(K, L, p.leaf_cap, s.frame,
+                                                                                    s.bgraph, s.tree, &hdr->tree_nodes);
         BGV_TRY(launch_status());
         BGV_TRY(mark(4));
-        BGV_TRY(scan_exclusive(s.start_count, s.T, K, nullptr, nullptr, true, s.scan_tmp, st));
-        note_launch(), k_preorder<<<gt, kThreads, 0, st>>>(K, s.range, s.cell_level, s.start_levels, s.cell, s.T,
-                                                           s.body, s.geo, s.skip);
+        note_launch(), k_tile_emit<<<tiles, kTileThreads, 0, st>>>(K, s.body, s.tree, s.T, s.geo, s.skip);
         BGV_TRY(launch_status());
         BGV_TRY(mark(5));
         const float theta2 = p.theta * p.theta;
@@ -1799,6 +1269,7 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
         BGV_TRY(launch_status());
     } else {
         BGV_CUDA(cudaMemsetAsync(s.Frep, 0, sizeof(float2), st));
+        BGV_TRY(mark(3));
         BGV_TRY(mark(4));
         BGV_TRY(mark(5));
     }
