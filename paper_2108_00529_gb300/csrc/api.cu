@@ -130,8 +130,11 @@ int check_layout_params(const bgv_layout_params *p) {
 int fa2_loop(int64_t K, int64_t nnz, const int32_t *off, const int32_t *adj, const uint32_t *w, const uint32_t *mass,
              const bgv_fa2_params &p, int32_t iterations, int32_t use_graph, float *pos, float *F, float *Fprev,
              double *speed, WsHeader *hdr, void *scratch, cudaStream_t st, int32_t G = 1,
-             const int64_t *koff = nullptr) {
+             const int64_t *koff = nullptr, int64_t Kmax = -1) {
     if (iterations <= 0 || K <= 0) return BGV_OK;
+    if (G <= 1) Kmax = K;
+    if (Kmax > 0 && small_fits(Kmax, nnz, G))
+        return run_fa2_small(K, Kmax, nnz, off, adj, w, mass, p, iterations, pos, F, Fprev, speed, hdr, st, G, koff);
     if (!use_graph || st == nullptr || iterations < 2) {
         for (int32_t t = 0; t < iterations; ++t)
             BGV_TRY(run_fa2(1, K, nnz, off, adj, w, mass, p, pos, F, Fprev, speed, nullptr, nullptr, nullptr, hdr,
@@ -169,6 +172,13 @@ int fa2_loop(int64_t K, int64_t nnz, const int32_t *off, const int32_t *adj, con
     cudaGraphExecDestroy(exec);
     cudaGraphDestroy(graph);
     return rc;
+}
+
+// Bodies of the largest graph of a batch (host offsets).
+int64_t largest_graph(int32_t G, const int64_t *koff) {
+    int64_t most = 0;
+    for (int32_t g = 0; g < G; ++g) most = std::max(most, koff[g + 1] - koff[g]);
+    return most;
 }
 
 // Whole-graph CSR (ForceAtlas2 on the graph itself): the supergraph of the
@@ -468,7 +478,7 @@ int layout_batched_device(const int32_t *edges_local, const int64_t *edge_off, c
     const int64_t K = K_off[G], Es = Es_off[G];
     BGV_TRY(run_fa2_init(K, p->fa2, xy, b.Fprev, b.speed, st, G, bb.koff));
     BGV_TRY(fa2_loop(K, 2 * Es, b.csr_off, b.csr_adj, b.csr_w, b.mass, p->fa2, p->iterations, p->use_graph, xy, b.F,
-                     b.Fprev, b.speed, hdr, b.scratch, st, G, bb.koff));
+                     b.Fprev, b.speed, hdr, b.scratch, st, G, bb.koff, largest_graph(G, K_off)));
     if (radius) {
         note_launch(), k_radius<<<grid_for(K, 256, sm_count() * 8), 256, 0, st>>>(b.mass, b.K_dev, radius);
         BGV_TRY(launch_status());
@@ -731,6 +741,9 @@ int bgv_fa2_step(int64_t K, int64_t nnz, const int32_t *csr_off, const int32_t *
     BGV_TRY(check_fa2_args(K, nnz, csr_off, csr_adj, csr_w, mass, p, pos, ws, ws_bytes));
     if (K == 0) return BGV_OK;
     if (!F || !Fprev || !speed) return BGV_EINVAL;
+    if (small_fits(K, nnz, 1))
+        return run_fa2_small(K, K, nnz, csr_off, csr_adj, csr_w, mass, *p, 1, pos, F, Fprev, speed, header(ws),
+                             as_stream(stream), 1, nullptr);
     return run_fa2(1, K, nnz, csr_off, csr_adj, csr_w, mass, *p, pos, F, Fprev, speed, nullptr, nullptr, nullptr,
                    header(ws), static_cast<char *>(ws) + kHeaderBytes, as_stream(stream));
 }
@@ -964,7 +977,7 @@ int bgv_fa2_run_batched(int32_t G, const int64_t *koff, int64_t nnz, const int32
     char *scratch = nullptr;
     BGV_TRY(fa2_batched_setup(G, koff, K, p->max_depth, ws, st, &dkoff, &scratch));
     return fa2_loop(K, nnz, csr_off, csr_adj, csr_w, mass, *p, iterations, use_graph, pos, F, Fprev, speed,
-                    header(ws), scratch, st, G, dkoff);
+                    header(ws), scratch, st, G, dkoff, largest_graph(G, koff));
 }
 
 size_t bgv_autotune_fa2_ws_size(int64_t K, int64_t nnz) {

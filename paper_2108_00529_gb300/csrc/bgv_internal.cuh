@@ -404,6 +404,13 @@ int run_fa2(int mode, int64_t K, int64_t nnz, const int32_t *csr_off, const int3
             float *Fr, float *Fa, float *Fg, WsHeader *hdr, void *scratch, cudaStream_t st,
             cudaEvent_t *marks = nullptr, bool build_plan = true, int32_t G = 1, const int64_t *koff = nullptr,
             bool hinted = false);
+// The same steps (mode 1) of G graphs of at most Kmax bodies each, when a cluster
+// of blocks can keep a graph in shared memory; no scratch, same results.
+bool small_fits(int64_t Kmax, int64_t nnz, int32_t G);
+int run_fa2_small(int64_t K, int64_t Kmax, int64_t nnz, const int32_t *csr_off, const int32_t *csr_adj,
+                  const uint32_t *csr_w, const uint32_t *mass, const bgv_fa2_params &p, int32_t iterations, float *pos,
+                  float *F, float *Fprev, double *speed, WsHeader *hdr, cudaStream_t st, int32_t G,
+                  const int64_t *koff);
 // `hinted`: the scratch holds the previous step's Morton order of the same
 // bodies (the step before ran on this scratch with the same K and G), which
 // then serves as the hint of the hinted sort (when fa2_order() is 1).

@@ -33,8 +33,10 @@
 #include <atomic>
 
 #include "bgv_internal.cuh"
+#include "forces.cuh"
 #include "hsort.cuh"
 #include "tree.cuh"
+#include "small.cuh"
 
 namespace bgv {
 
@@ -50,41 +52,7 @@ inline int64_t warp_share(int64_t K, int blocks) {
 }
 inline int node_blocks() { return sm_count() * 4 < kMaxNodeBlocks ? sm_count() * 4 : kMaxNodeBlocks; }
 
-__device__ __forceinline__ unsigned long long spread_bits(uint32_t v) {
-    unsigned long long x = v;
-    x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
-    x = (x | (x << 8)) & 0x00FF00FF00FF00FFull;
-    x = (x | (x << 4)) & 0x0F0F0F0F0F0F0F0Full;
-    x = (x | (x << 2)) & 0x3333333333333333ull;
-    x = (x | (x << 1)) & 0x5555555555555555ull;
-    return x;
-}
-
 // ----------------------------------------------------------------- frame
-// Frame of a bounding box: origin, side = max extent * (1 + 2^-20).
-__device__ __forceinline__ float4 frame_of(float lx, float ly, float hx, float hy) {
-    const float ex = __fsub_rn(hx, lx), ey = __fsub_rn(hy, ly);
-    const float ext = ex > ey ? ex : ey;
-    float side = __fmul_rn(ext, 1.00000095367431640625f);  // 1 + 2^-20
-    if (!(ext > 0.0f)) side = 1.0f;
-    return make_float4(lx, ly, side, 0.0f);
-}
-
-__device__ __forceinline__ float4 box_empty() { return make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY); }
-__device__ __forceinline__ void box_add(float4 &b, float2 p) {
-    b.x = fminf(b.x, p.x); b.y = fminf(b.y, p.y);
-    b.z = fmaxf(b.z, p.x); b.w = fmaxf(b.w, p.y);
-}
-__device__ __forceinline__ void box_merge(float4 &b, const float4 &o) {
-    b.x = fminf(b.x, o.x); b.y = fminf(b.y, o.y);
-    b.z = fmaxf(b.z, o.z); b.w = fmaxf(b.w, o.w);
-}
-__device__ __forceinline__ void box_warp(float4 &b) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1)
-        box_merge(b, make_float4(__shfl_xor_sync(0xFFFFFFFFu, b.x, d), __shfl_xor_sync(0xFFFFFFFFu, b.y, d),
-                                 __shfl_xor_sync(0xFFFFFFFFu, b.z, d), __shfl_xor_sync(0xFFFFFFFFu, b.w, d)));
-}
 // Block-wide box; every thread calls it, thread 0 receives the result.
 __device__ __forceinline__ void box_block(float4 &b) {
     __shared__ float4 wbox[kThreads / 32];
@@ -244,14 +212,9 @@ __global__ void __launch_bounds__(kThreads) k_keys(const float2 *__restrict__ po
 }
 
 // -------------------------------------------------------------- repulsion
-// Barnes-Hut traversal without a stack, one body per thread, over the
-// pre-order array.  At element `cur` (a cell or a body) the thread accepts it
-// -- sums its monopole and moves to skip[cur], past its subtree -- or enters
-// it (cur + 1).  A body is always accepted except the thread's own (its
-// side^2 is -1); a cell holding the thread's body is always entered; any
-// other cell is accepted by the FP32 opening test of the definition.  Each
-// body sees exactly its own interaction set in depth-first order; threads of
-// a warp are Morton neighbours, so they mostly read the same elements.
+// Barnes-Hut traversal, one body per thread (bh_walk).  Each body sees exactly
+// its own interaction set in depth-first order; threads of a warp are Morton
+// neighbours, so they mostly read the same elements.
 template <int kRT>
 __global__ void __launch_bounds__(kRT) k_repulse(const float4 *__restrict__ geo, const int32_t *__restrict__ skip,
                                                       const uint32_t *__restrict__ T,
@@ -275,22 +238,7 @@ __global__ void __launch_bounds__(kRT) k_repulse(const float4 *__restrict__ geo,
             cur = uint32_t(a + T[a]);
             end = uint32_t(b + T[b]);
         }
-        float fx = 0.0f, fy = 0.0f;
-        while (cur < end) {
-            const float4 e = geo[cur];
-            const uint32_t sk = uint32_t(skip[cur]);
-            const float dx = __fsub_rn(bi.x, e.x), dy = __fsub_rn(bi.y, e.y);
-            const float d2 = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
-            // accepted: not an element holding the body (cur <= self < sk) and
-            // the opening test passes; no branch, so lanes stay converged
-            const bool accept = self - cur >= sk - cur && e.w < __fmul_rn(theta2, d2);
-            const float f = accept && d2 > 0.0f ? __fdividef(kmi * e.z, d2) : 0.0f;
-            fx += f * dx;
-            fy += f * dy;
-            inter += accept ? 1u : 0u;
-            cur = accept ? sk : cur + 1;
-        }
-        Frep[__float_as_int(bi.w)] = make_float2(fx, fy);
+        Frep[__float_as_int(bi.w)] = bh_walk(geo, skip, bi, kmi, theta2, self, cur, end, inter);
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) inter += __shfl_xor_sync(0xFFFFFFFFu, inter, d);
@@ -312,7 +260,6 @@ __global__ void __launch_bounds__(kRT) k_repulse(const float4 *__restrict__ geo,
 // then a fixed tree).  Every worker first issues kAttIn loads of neighbour
 // ids and weights, then their position gathers, so they are in flight
 // together.  An empty row is a short row of sum 0.
-constexpr int kAttMedium = 4096;
 // loads in flight per worker; with 5 blocks of 256 per SM (at most 51
 // registers) that is 320 outstanding gathers per SM
 constexpr int kAttIn = 8;
@@ -355,10 +302,6 @@ __global__ void __launch_bounds__(kThreads) k_att_plan(int64_t K, const int32_t 
         }
         __syncthreads();
     }
-}
-
-__device__ __forceinline__ bool valid_row(int32_t j, int64_t K) {
-    return static_cast<uint64_t>(int64_t(j)) < static_cast<uint64_t>(K);  // an invalid entry adds nothing
 }
 
 // Short rows: one lane each.
@@ -511,172 +454,7 @@ __global__ void __launch_bounds__(kThreads) k_att_long(int64_t K, const int32_t 
     }
 }
 
-// --------------------------------------------- node forces, swing, speed
-// Global swing and traction (the sums that set the adaptive speed):
-// S = sum m_i swing_i and T = sum m_i traction_i over FP32 per-node products,
-// which are non-negative.  They are summed EXACTLY: each product f * 2^q
-// (f its 24-bit significand) is added as a fixed-point integer into a
-// 128-bit accumulator V whose unit 2^q0 sits kXHead binary places below the
-// largest term seen so far (q0 moves up, with V shifted down, when a larger
-// term arrives).  A term below the unit loses only its bits under 2^q0, less
-// than 2^-95 of the largest term, so the accumulated value equals the exact
-// sum to about 2^-64 relative even over 2^31 terms; integer addition does not
-// depend on the order of the merges.  The total is rounded once to FP64, so S
-// and T are the correctly rounded sums of the products (Kahan or Neumaier
-// compensation in FP64 would leave about two units in the last place, and
-// FP64 arithmetic runs at a small fraction of the integer rate on this GPU).
-constexpr int kXHead = 72;          // each term < 2^(24 + 72): 2^31 terms fit in 127 bits
-constexpr int kXNoAnchor = -100000; // anchor of an empty accumulator
-struct XSum {
-    u128 V;
-    int q0;
-    int bad;  // 1: an infinite term, 2: a NaN term
-};
-__device__ __forceinline__ XSum xsum_zero() { return XSum{0, kXNoAnchor, 0}; }
-
-__device__ __forceinline__ void xsum_add(XSum &a, float x) {
-    const uint32_t b = __float_as_uint(x) & 0x7FFFFFFFu;  // terms are >= 0 (a -0 adds nothing)
-    const int e = int(b >> 23);
-    if (e == 255) {
-        a.bad |= (b & 0x7FFFFFu) ? 2 : 1;
-        return;
-    }
-    const uint32_t f = e ? ((b & 0x7FFFFFu) | 0x800000u) : b;
-    const int q = (e ? e : 1) - 150;  // x = f * 2^q
-    if (f == 0u) return;
-    if (q - kXHead > a.q0) {  // a new largest term: move the anchor up
-        const int d = q - kXHead - a.q0;
-        a.V = d >= 128 ? u128(0) : (a.V >> d);
-        a.q0 = q - kXHead;
-    }
-    const int sh = q - a.q0;  // <= kXHead
-    if (sh >= 0)
-        a.V += u128(f) << sh;
-    else if (sh > -24)
-        a.V += u128(f >> -sh);
-}
-
-__device__ __forceinline__ XSum xsum_merge(XSum a, XSum b) {
-    if (b.q0 > a.q0) {
-        const XSum t = a;
-        a = b;
-        b = t;
-    }
-    const int d = a.q0 - b.q0;
-    if (d < 128) a.V += b.V >> d;
-    a.bad |= b.bad;
-    return a;
-}
-
-__device__ __forceinline__ XSum xsum_shfl_down(const XSum &a, int d) {
-    XSum r;
-    r.V = (u128(__shfl_down_sync(0xFFFFFFFFu, static_cast<unsigned long long>(a.V >> 64), d)) << 64) |
-          __shfl_down_sync(0xFFFFFFFFu, static_cast<unsigned long long>(a.V), d);
-    r.q0 = __shfl_down_sync(0xFFFFFFFFu, a.q0, d);
-    r.bad = __shfl_down_sync(0xFFFFFFFFu, a.bad, d);
-    return r;
-}
-
-// The accumulated value rounded once to FP64 (round to nearest even): the top
-// 64 bits of V, with a sticky bit for the rest, converted, then scaled.
-__device__ __forceinline__ double xsum_value(const XSum &a) {
-    if (a.bad) return (a.bad & 2) ? __longlong_as_double(0x7FF8000000000000ll) : __longlong_as_double(0x7FF0000000000000ll);
-    const unsigned long long hi = static_cast<unsigned long long>(a.V >> 64);
-    if (!hi) return ldexp(__ull2double_rn(static_cast<unsigned long long>(a.V)), a.q0);
-    const int sh = 64 - __clzll(static_cast<long long>(hi));  // bits of V above its top 64
-    unsigned long long t = static_cast<unsigned long long>(a.V >> sh);
-    if (a.V & ((u128(1) << sh) - 1)) t |= 1ull;  // sticky: far below the rounding position
-    return ldexp(__ull2double_rn(t), a.q0 + sh);
-}
-
-// Stored form of one accumulator (per-block partials).
-struct XPart {
-    unsigned long long lo, hi;
-    int q0, bad;
-};
-__device__ __forceinline__ XPart xsum_pack(const XSum &a) {
-    return XPart{static_cast<unsigned long long>(a.V), static_cast<unsigned long long>(a.V >> 64), a.q0, a.bad};
-}
-__device__ __forceinline__ XSum xsum_unpack(const XPart *p) {  // from L2: written by other blocks
-    const unsigned long long lo = __ldcg(&p->lo), hi = __ldcg(&p->hi);
-    return XSum{(u128(hi) << 64) | lo, __ldcg(&p->q0), __ldcg(&p->bad)};
-}
-
-// Block-wide merge of one (S, T) pair per thread in a fixed tree; thread 0
-// receives the result.
-__device__ __forceinline__ void xsum_block(XSum &S, XSum &T) {
-    __shared__ XPart sS[kThreads / 32], sT[kThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        const XSum oS = xsum_shfl_down(S, d), oT = xsum_shfl_down(T, d);
-        S = xsum_merge(S, oS);
-        T = xsum_merge(T, oT);
-    }
-    if (lane == 0) {
-        sS[warp] = xsum_pack(S);
-        sT[warp] = xsum_pack(T);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < kThreads / 32; ++k) {
-            S = xsum_merge(S, XSum{(u128(sS[k].hi) << 64) | sS[k].lo, sS[k].q0, sS[k].bad});
-            T = xsum_merge(T, XSum{(u128(sT[k].hi) << 64) | sT[k].lo, sT[k].q0, sT[k].bad});
-        }
-    }
-    __syncthreads();
-}
-
-__device__ __forceinline__ double speed_update(double sp, double Ssum, double Tsum, float tau) {
-    if (Ssum > 0.0) {
-        const double target = double(tau) * Tsum / Ssum;
-        const double rise = target - sp, cap = 0.5 * sp;
-        sp += rise < cap ? rise : cap;
-    }
-    return sp;
-}
-
-// Per-node swing and traction products, FP32 with every rounding explicit
-// (no contraction), so they can be recomputed bit for bit from F, Fprev and
-// the mass: m |F - Fprev| and (m / 2) |F + Fprev|.
-__device__ __forceinline__ float2 swing_traction(float m, float fx, float fy, float px, float py) {
-    const float sx = __fsub_rn(fx, px), sy = __fsub_rn(fy, py), tx = __fadd_rn(fx, px), ty = __fadd_rn(fy, py);
-    const float sw = sqrtf(__fadd_rn(__fmul_rn(sx, sx), __fmul_rn(sy, sy)));
-    const float tr = sqrtf(__fadd_rn(__fmul_rn(tx, tx), __fmul_rn(ty, ty)));
-    return make_float2(__fmul_rn(m, sw), __fmul_rn(__fmul_rn(0.5f, m), tr));
-}
-
-__device__ __forceinline__ float2 force_sum(float2 fa, float m, float2 pi, float2 fr, float kg, int strong) {
-    float gx, gy;
-    if (strong) {
-        gx = -kg * m * pi.x;
-        gy = -kg * m * pi.y;
-    } else {
-        const float rr = sqrtf(pi.x * pi.x + pi.y * pi.y);
-        gx = rr > 0.0f ? -kg * m * pi.x / rr : 0.0f;
-        gy = rr > 0.0f ? -kg * m * pi.y / rr : 0.0f;
-    }
-    return make_float2(fr.x + fa.x + gx, fr.y + fa.y + gy);
-}
-
-// Total force on node i: repulsion fr, attraction full[i] (none if null),
-// gravity.
-__device__ __forceinline__ float2 node_force(int64_t i, const float2 *__restrict__ full, float m, float2 pi, float2 fr,
-                                             float kg, int strong) {
-    return force_sum(full ? full[i] : make_float2(0.0f, 0.0f), m, pi, fr, kg, strong);
-}
-
-__device__ __forceinline__ float2 displaced(float2 p, float2 f, float2 fp, float sp, float ks, float ksmax) {
-    const float sx = f.x - fp.x, sy = f.y - fp.y;
-    const float swing = sqrtf(sx * sx + sy * sy);
-    float s = ks * sp / (1.0f + sp * sqrtf(swing));
-    const float fn = sqrtf(f.x * f.x + f.y * f.y);
-    if (fn > 0.0f && s * fn > ksmax) s = ksmax / fn;
-    p.x += s * f.x;
-    p.y += s * f.y;
-    return p;
-}
-
+// ------------------------------------------------- node forces and tail
 // Forces only (no state change): repulsion, attraction and gravity per node.
 __global__ void __launch_bounds__(kThreads) k_node(int64_t K, const float2 *__restrict__ att,
                                                    const uint32_t *__restrict__ mass, const float2 *__restrict__ pos,
@@ -712,16 +490,6 @@ __global__ void __launch_bounds__(kThreads) k_node(int64_t K, const float2 *__re
 // of 689.2, and 200 steps of a 1,000-node layout 12.4 ms instead of 14.7.)
 // att == nullptr: no CSR entries, no attraction.
 constexpr int kTailItems = 4;  // nodes a lane takes per pass, every load issued before the arithmetic
-
-// Merge of one (S, T) pair per lane; lane 0 receives the result.
-__device__ __forceinline__ void xsum_warp(XSum &S, XSum &T) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        const XSum oS = xsum_shfl_down(S, d), oT = xsum_shfl_down(T, d);
-        S = xsum_merge(S, oS);
-        T = xsum_merge(T, oT);
-    }
-}
 
 template <bool kB>
 __global__ void __launch_bounds__(kThreads, 3) k_tail(int64_t K, int64_t per, const float2 *__restrict__ att,
@@ -770,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_tail(int64_t K, int64_t per, co
     };
     if (!kB) {
         sum_forces(c_lo, c_hi);
-        xsum_block(S, T);
+        xsum_block<kThreads>(S, T);
         if (threadIdx.x == 0) {
             part[2 * blockIdx.x] = xsum_pack(S);
             part[2 * blockIdx.x + 1] = xsum_pack(T);
@@ -783,7 +551,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_tail(int64_t K, int64_t per, co
             S = xsum_merge(S, xsum_unpack(&part[2 * bk]));
             T = xsum_merge(T, xsum_unpack(&part[2 * bk + 1]));
         }
-        xsum_block(S, T);
+        xsum_block<kThreads>(S, T);
         if (threadIdx.x == 0) {
             const double Ssum = xsum_value(S), Tsum = xsum_value(T);
             sp_sh = speed_update(sp_old, Ssum, Tsum, tau);
@@ -1319,6 +1087,64 @@ int run_fa2(int mode, int64_t K, int64_t nnz, const int32_t *csr_off, const int3
     BGV_CUDA(cudaEventRecord(ev.join, hp));
     BGV_CUDA(cudaStreamWaitEvent(st, ev.join, 0));
     return rc;
+}
+
+// Steps of graphs that a cluster of blocks keeps in shared memory (small.cuh):
+// G graphs of at most Kmax bodies, koff on the device (null for one graph).
+// A cluster takes its SMs whole, so a batch of more clusters than two rounds of
+// the GPU's SMs runs faster side by side in the general path's launches.
+bool small_fits(int64_t Kmax, int64_t nnz, int32_t G) {
+    return Kmax <= kSmallMax && nnz <= kSmallEntries * (G > 1 ? G : 1) &&
+           int64_t(G > 1 ? G : 1) * small_cluster(Kmax) <= 2 * int64_t(sm_count());
+}
+
+int run_fa2_small(int64_t K, int64_t Kmax, int64_t nnz, const int32_t *csr_off, const int32_t *csr_adj,
+                  const uint32_t *csr_w, const uint32_t *mass, const bgv_fa2_params &p, int32_t iterations, float *pos,
+                  float *F, float *Fprev, double *speed, WsHeader *hdr, cudaStream_t st, int32_t G,
+                  const int64_t *koff) {
+    SmallArgs a{};
+    a.K = K;
+    a.koff = G > 1 ? koff : nullptr;
+    a.off = nnz > 0 ? csr_off : nullptr;
+    a.adj = csr_adj;
+    a.w = csr_w;
+    a.mass = mass;
+    a.pos = reinterpret_cast<float2 *>(pos);
+    a.F = reinterpret_cast<float2 *>(F);
+    a.Fprev = reinterpret_cast<float2 *>(Fprev);
+    a.speed = speed;
+    a.hdr = hdr;
+    a.theta2 = p.theta * p.theta;
+    a.kr = p.kr;
+    a.kg = p.kg;
+    a.tau = p.tau;
+    a.ks = p.ks;
+    a.ksmax = p.ksmax;
+    a.strong = p.strong_gravity;
+    a.L = p.max_depth;
+    a.leaf_cap = p.leaf_cap;
+    a.att_short = fa2_tune().att_short;
+    const int C = small_cluster(Kmax);
+    BGV_CUDA(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(SmallMem))));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned((G > 1 ? G : 1) * C));
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = sizeof(SmallMem);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = unsigned(C);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    for (int32_t done = 0; done < iterations; done += kSmallChunk) {
+        a.iterations = iterations - done < kSmallChunk ? iterations - done : kSmallChunk;
+        BGV_CUDA(cudaMemsetAsync(&hdr->interactions, 0, 2 * sizeof(unsigned long long), st));  // and tree_nodes
+        note_launch();
+        BGV_CUDA(cudaLaunchKernelEx(&cfg, k_small, a));
+    }
+    return BGV_OK;
 }
 
 }  // namespace bgv
