@@ -9,14 +9,15 @@
 // it to cut the global passes to two (count, scatter) and to sort the rest
 // in shared memory, with kernels that need no grid-wide residency.
 //
-// Method: a sample sort whose buckets follow the hint.
-//   1. Samples: the ids at ns evenly spaced places of the hint and their
-//      keys, ranked among themselves by counting (ns^2 comparisons spread
-//      over many threads; equal pairs ranked by sample index) and stored in
-//      (key, id) order.  Splitter u (1 <= u < nb) is sample u*s, with s
-//      samples per bucket; bucket u holds the pairs x with
-//      splitter(u) <= x < splitter(u+1), splitter(0) = -inf, splitter(nb) =
-//      +inf.
+// Method: a bucket sort whose buckets follow the hint.
+//   1. Splitters.  ForceAtlas2 still holds the previous iteration's sorted
+//      (key, id) pairs: every kHsBucket-th of them is a splitter (HsPrevious), in
+//      order already, with about as many new pairs between two as old ones.
+//      The public entry point has no earlier keys: it takes the ids at ns evenly
+//      spaced places of the hint and their keys, ranks them among themselves by
+//      counting (equal pairs by sample index), and every s-th is a splitter
+//      (HsSampled).  Bucket u holds the pairs x with splitter(u) <= x <
+//      splitter(u+1), splitter(0) = -inf, splitter(nb) = +inf.
 //   2. Count: every pair's key and bucket (the search starts at the bucket
 //      its place in the hint would have, so a good hint needs one or two
 //      probes), counted per bucket with one atomic per bucket per warp; the
@@ -24,9 +25,11 @@
 //   3. Scatter: every pair to its bucket (one atomic per bucket per warp).
 //   4. Bucket sort: one block per bucket.  Up to kHsCap pairs it sorts in
 //      shared memory, as single words (key - min key) << idbits | id when the
-//      bucket's keys span few enough bits, else as pairs: each thread's 4 or
-//      8 through a sorting network in registers, then merges of sorted runs
-//      by merge path.  A larger bucket (a poor hint) is sorted in chunks and
+//      bucket's keys span few enough bits: words go to bins by their high bits
+//      (shared-memory atomics) and are ranked inside their bins, which hold a
+//      word or two; a bin too full for that (keys crowded in a corner of the
+//      bucket), or keys too far apart for one word, take a merge sort in
+//      shared memory.  A larger bucket (a poor hint) is sorted in chunks and
 //      merged in global memory by the same block.
 // The result is the (key, id) order for any hint: a poor hint only makes the
 // buckets uneven.  A hint entry >= K raises BGV_DEV_BADHINT and is read as
@@ -47,34 +50,58 @@ constexpr int kHsItems = 8;             // pairs (or words) per thread
 constexpr int kHsPairCap = kHsThreads * kHsItems;  // 2048: a chunk of the pair sort
 constexpr int kHsCap = kHsPairCap;      // larger buckets take the chunked path
 constexpr int kHsRankSlices = 16;       // slices of the samples per ranking thread
+constexpr int kHsBins = 2048;           // bins of a bucket's words
+constexpr uint32_t kHsRankBin = 32;     // largest bin ranked by counting
 constexpr int kHsSmem = kHsCap + kHsCap / 16;  // skewed shared-memory slots
 
 inline int64_t hs_max_keys() { return int64_t(kHsMaxBuckets) * kHsBucket; }
 
 // Small device arrays of the sort (the large ones are the caller's).
 struct HsBuffers {
-    unsigned long long *smp_key;  // [kHsMaxSamples] samples in hint order
+    unsigned long long *smp_key;  // [kHsMaxSamples] samples in hint order (public entry point only)
     uint32_t *smp_id;             // [kHsMaxSamples]
     uint32_t *smp_rank;           // [kHsMaxSamples]
     unsigned long long *spl_key;  // [kHsMaxBuckets] splitter u at u - 1
     uint32_t *spl_id;             // [kHsMaxBuckets]
-    uint32_t *count;              // [kHsMaxBuckets] pairs per bucket
-    uint32_t *cursor;             // [kHsMaxBuckets] scatter cursors
-    uint32_t *start;              // [kHsMaxBuckets + 1] bucket starts
+    uint32_t *count;              // [nb] pairs per bucket; zero between sorts, with all that follows:
+    uint32_t *cursor;             // [nb] scatter cursors
     uint32_t *ticket;             // [2] last-block tickets
+    uint32_t *start;              // [nb + 1] bucket starts
 };
 
-inline void carve_hs(Carver &c, HsBuffers &h) {
-    h.smp_key = c.take<unsigned long long>(kHsMaxSamples);
-    h.smp_id = c.take<uint32_t>(kHsMaxSamples);
-    h.smp_rank = c.take<uint32_t>(kHsMaxSamples);
-    h.spl_key = c.take<unsigned long long>(kHsMaxBuckets);
-    h.spl_id = c.take<uint32_t>(kHsMaxBuckets);
-    h.count = c.take<uint32_t>(kHsMaxBuckets);
-    h.cursor = c.take<uint32_t>(kHsMaxBuckets);
-    h.start = c.take<uint32_t>(kHsMaxBuckets + 1);
-    h.ticket = c.take<uint32_t>(2);
+inline int hs_buckets(int64_t K) { return K > kHsBucket ? int((K + kHsBucket - 1) / kHsBucket) : 1; }
+// Words from `count` on that are zero before a sort (and after it).
+inline int64_t hs_counter_words(int64_t K) { return 2 * int64_t(hs_buckets(K)) + 2; }
+
+inline void carve_hs(Carver &c, int64_t K, bool sampled, HsBuffers &h) {
+    const size_t nb = size_t(hs_buckets(K));
+    h = HsBuffers{};
+    if (sampled) {
+        h.smp_key = c.take<unsigned long long>(kHsMaxSamples);
+        h.smp_id = c.take<uint32_t>(kHsMaxSamples);
+        h.smp_rank = c.take<uint32_t>(kHsMaxSamples);
+        h.spl_key = c.take<unsigned long long>(kHsMaxBuckets);
+        h.spl_id = c.take<uint32_t>(kHsMaxBuckets);
+    }
+    h.count = c.take<uint32_t>(size_t(hs_counter_words(K)));
+    h.cursor = h.count ? h.count + nb : nullptr;
+    h.ticket = h.count ? h.count + 2 * nb : nullptr;
+    h.start = c.take<uint32_t>(nb + 1);
 }
+
+// Splitter u + 1 (the least pair of bucket u + 1).
+struct HsSampled {
+    const unsigned long long *key;
+    const uint32_t *id;
+    __device__ unsigned long long key_at(int u) const { return __ldg(&key[u]); }
+    __device__ uint32_t id_at(int u) const { return __ldg(&id[u]); }
+};
+struct HsPrevious {  // the sorted pairs of the previous iteration
+    const unsigned long long *key;
+    const uint32_t *id;
+    __device__ unsigned long long key_at(int u) const { return __ldg(&key[int64_t(u + 1) * kHsBucket]); }
+    __device__ uint32_t id_at(int u) const { return __ldg(&id[int64_t(u + 1) * kHsBucket]); }
+};
 
 // Buckets and samples per bucket for K pairs (nb = 1: no splitters).
 struct HsShape {
@@ -82,22 +109,13 @@ struct HsShape {
 };
 inline HsShape hs_shape(int64_t K) {
     HsShape h;
-    h.nb = int((K + kHsBucket - 1) / kHsBucket);
-    if (h.nb < 1) h.nb = 1;
+    h.nb = hs_buckets(K);
     h.s = kHsMaxSamples / h.nb;
     if (h.s > kHsMaxPerBucket) h.s = kHsMaxPerBucket;
     if (h.s < 1) h.s = 1;
     h.ns = h.nb > 1 ? h.nb * h.s : 0;  // nb > 1 means K > 1024 >= 8 nb, so ns < K
     return h;
 }
-
-// Extra words the first kernel clears (for the kernels after the sort).
-struct HsClears {
-    unsigned long long *u64 = nullptr;
-    int64_t n_u64 = 0;
-    uint32_t *u32 = nullptr;
-    int64_t n_u32 = 0;
-};
 
 // The kernels are private to each translation unit that includes this
 // header (each instantiates its own key source).
@@ -119,8 +137,8 @@ __device__ __forceinline__ uint32_t hs_id(const uint32_t *__restrict__ hint, int
 
 // 1a. Sample keys; clears the counters of the later kernels.
 template <class KeyOf>
-__global__ void __launch_bounds__(256) k_hs_sample(KeyOf key_of, const uint32_t *__restrict__ hint, int64_t K, int nb,
-                                                   int ns, HsBuffers h, HsClears clr, uint32_t *status) {
+__global__ void __launch_bounds__(256) k_hs_sample(KeyOf key_of, const uint32_t *__restrict__ hint, int64_t K,
+                                                   int64_t counter_words, int ns, HsBuffers h, uint32_t *status) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     const int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     for (int64_t t = t0; t < ns; t += stride) {
@@ -130,13 +148,7 @@ __global__ void __launch_bounds__(256) k_hs_sample(KeyOf key_of, const uint32_t 
         h.smp_id[t] = id;
         h.smp_rank[t] = 0u;
     }
-    for (int64_t t = t0; t < nb; t += stride) {
-        h.count[t] = 0u;
-        h.cursor[t] = 0u;
-    }
-    if (t0 < 2) h.ticket[t0] = 0u;
-    for (int64_t t = t0; t < clr.n_u64; t += stride) clr.u64[t] = 0ull;
-    for (int64_t t = t0; t < clr.n_u32; t += stride) clr.u32[t] = 0u;
+    for (int64_t t = t0; t < counter_words; t += stride) h.count[t] = 0u;
 }
 
 // 1b. Ranks of the samples by counting, one slice of the others per block
@@ -197,9 +209,9 @@ __global__ void __launch_bounds__(256) k_hs_rank(int ns, int s, HsBuffers h) {  
 
 // Bucket of pair x: the smallest u in [0, nb) with u == nb - 1 or
 // x < splitter(u + 1) (stored at u), searched outwards from the guess g.
-__device__ __forceinline__ int hs_bucket(unsigned long long xk, uint32_t xi, const unsigned long long *__restrict__ sk,
-                                         const uint32_t *__restrict__ si, int nb, int g) {
-    auto above = [&](int u) { return u >= nb - 1 || hs_less(xk, xi, __ldg(&sk[u]), __ldg(&si[u])); };
+template <class Split>
+__device__ __forceinline__ int hs_bucket(unsigned long long xk, uint32_t xi, const Split &split, int nb, int g) {
+    auto above = [&](int u) { return u >= nb - 1 || hs_less(xk, xi, split.key_at(u), split.id_at(u)); };
     int lo, hi;  // the answer is in [lo, hi]; above(hi); lo == 0 or !above(lo - 1)
     if (above(g)) {
         hi = g;
@@ -242,13 +254,14 @@ __device__ __forceinline__ int hs_bucket(unsigned long long xk, uint32_t xi, con
 
 // 2. Keys and buckets in hint order, counts per bucket; the last block
 // writes the bucket starts.
-template <class KeyOf>
-__global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, const uint32_t *__restrict__ hint, int64_t K, int nb,
-                                                  HsBuffers h, unsigned long long *__restrict__ tmp_key,
+template <class KeyOf, class Split>
+__global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, const uint32_t *__restrict__ hint,
+                                                  int64_t K, int nb, HsBuffers h,
+                                                  unsigned long long *__restrict__ tmp_key,
                                                   uint32_t *__restrict__ tmp_bucket, uint32_t *status) {
     __shared__ bool last;
-    __shared__ uint32_t part[256];
-    const int lane = threadIdx.x & 31;
+    __shared__ uint32_t part[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the bucket a hint place would have if the buckets split the hint
     // evenly: the search starts there
     const float g_scale = float(nb) / float(K);
@@ -260,7 +273,7 @@ __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, const uint32_t *
             const uint32_t id = hs_id(hint, p, K, status);
             const unsigned long long k = key_of(id);
             const int g = min(nb - 1, int(float(p) * g_scale));
-            u = nb > 1 ? hs_bucket(k, id, h.spl_key, h.spl_id, nb, g) : 0;
+            u = nb > 1 ? hs_bucket(k, id, split, nb, g) : 0;
             tmp_key[p] = k;
             tmp_bucket[p] = uint32_t(u);
         }
@@ -276,26 +289,36 @@ __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, const uint32_t *
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // exclusive scan of the counts: a contiguous chunk per thread
-    const int per = (nb + blockDim.x - 1) / blockDim.x;
-    const int b0 = threadIdx.x * per, b1 = min(nb, b0 + per);
-    uint32_t sum = 0;
-    for (int b = b0; b < b1; ++b) sum += __ldcg(&h.count[b]);
-    part[threadIdx.x] = sum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (int t = 0; t < int(blockDim.x); ++t) {
-            const uint32_t c = part[t];
-            part[t] = run;
-            run += c;
+    // exclusive scan of the counts, 1,024 at a time
+    uint32_t carry = 0u;
+    for (int b0 = 0; b0 < nb; b0 += 1024) {
+        const int b = b0 + 4 * int(threadIdx.x);
+        uint32_t c[4], sum = 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            c[q] = b + q < nb ? __ldcg(&h.count[b + q]) : 0u;
+            sum += c[q];
         }
-    }
-    __syncthreads();
-    uint32_t run = part[threadIdx.x];
-    for (int b = b0; b < b1; ++b) {
-        h.start[b] = run;
-        run += __ldcg(&h.count[b]);
+        uint32_t inc = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += y;
+        }
+        if (lane == 31) part[warp] = inc;
+        __syncthreads();
+        uint32_t run = carry + inc - sum, all = 0u;
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) run += part[w];
+            all += part[w];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (b + q < nb) h.start[b + q] = run;
+            run += c[q];
+        }
+        carry += all;
+        __syncthreads();
     }
     if (threadIdx.x == 0) h.start[nb] = uint32_t(K);
 }
@@ -550,34 +573,38 @@ __device__ void hs_pairs_chunked(unsigned long long *sk, uint32_t *sv, int64_t n
     }
 }
 
-// A bucket of n <= I * blockDim.x pairs: read coalesced through shared
-// memory; if its keys span less than 2^(63 - idbits), the words
-// (key - kmin) << idbits | id (ids < 2^idbits) order exactly as (key, id)
-// and are sorted as single words, then written back coalesced; otherwise
-// the pairs are sorted as pairs.  Every thread of the block calls it.
+// A bucket of n <= I * blockDim.x pairs.  If its keys span less than 2^(63 -
+// idbits), the words (key - kmin) << idbits | id (ids < 2^idbits) order exactly
+// as (key, id) and are sorted as single words: to kHsBins bins by the high bits
+// of the span, then ranked inside their bins and written to their places; with
+// a bin of more than kHsRankBin words, merged instead.  Otherwise the pairs are
+// sorted as pairs.  Every thread of the block calls it.
+// Bound by instruction issue.  The bins take about 140 instructions per pair,
+// the merge rounds 720 (155 us for 3.2 M bodies).
 template <int I>
 __device__ void hs_bucket_small(unsigned long long *sk, uint32_t *sv, int n, unsigned long long *dk,
                                 uint32_t *dv, int idbits, unsigned long long *shk, uint32_t *shv,
                                 unsigned long long *wmin, unsigned long long *wmax) {
-    const int t = threadIdx.x;
-    for (int q = t; q < n; q += blockDim.x) {
-        shk[hs_sw(q)] = sk[q];
-        shv[hs_sw(q)] = sv[q];
-    }
-    __syncthreads();
+    static_assert(kHsBins == 8 * kHsThreads && kHsBins <= kHsSmem, "eight bins a thread, in the ids' memory");
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    uint32_t *bins = shv;
     unsigned long long c[I];
+    uint32_t id[I];
     unsigned long long kmin = ~0ull, kmax = 0ull;
 #pragma unroll
     for (int j = 0; j < I; ++j) {
-        const int q = I * t + j;
-        c[j] = ~0ull;
-        if (q < n) {
-            const unsigned long long k = shk[hs_sw(q)];
-            c[j] = k;
-            kmin = k < kmin ? k : kmin;
-            kmax = k > kmax ? k : kmax;
+        const int q = j * kHsThreads + t;
+        c[j] = q < n ? __ldcg(&sk[q]) : 0ull;
+        id[j] = q < n ? __ldcg(&sv[q]) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < I; ++j) {
+        if (j * kHsThreads + t < n) {
+            kmin = c[j] < kmin ? c[j] : kmin;
+            kmax = c[j] > kmax ? c[j] : kmax;
         }
     }
+    for (int b = t; b < kHsBins; b += kHsThreads) bins[b] = 0u;
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
         const unsigned long long a = __shfl_xor_sync(0xFFFFFFFFu, kmin, d);
@@ -585,55 +612,108 @@ __device__ void hs_bucket_small(unsigned long long *sk, uint32_t *sv, int n, uns
         kmin = a < kmin ? a : kmin;
         kmax = b > kmax ? b : kmax;
     }
-    if ((t & 31) == 0) {
-        wmin[t >> 5] = kmin;
-        wmax[t >> 5] = kmax;
+    if (lane == 0) {
+        wmin[warp] = kmin;
+        wmax[warp] = kmax;
     }
     __syncthreads();
     kmin = wmin[0];
     kmax = wmax[0];
-    for (int w = 1; w < int(blockDim.x >> 5); ++w) {
+    for (int w = 1; w < kHsThreads / 32; ++w) {
         kmin = wmin[w] < kmin ? wmin[w] : kmin;
         kmax = wmax[w] > kmax ? wmax[w] : kmax;
     }
     if (((kmax - kmin) >> (63 - idbits)) != 0ull) {  // too wide for one word
         __syncthreads();
-        if (n <= kHsPairCap)
-            hs_block_sort(sk, sv, n, dk, dv, shk, shv);
-        else
-            hs_pairs_chunked(sk, sv, n, dk, dv, shk, shv);
+        hs_block_sort(sk, sv, n, dk, dv, shk, shv);
         return;
     }
+    const int bits = kmax > kmin ? 64 - __clzll(static_cast<long long>(kmax - kmin)) : 0;
+    const int sh = bits > 11 ? bits - 11 : 0;
+    uint32_t rank[I];
 #pragma unroll
     for (int j = 0; j < I; ++j) {
-        const int q = I * t + j;
-        if (q < n) c[j] = ((c[j] - kmin) << idbits) | shv[hs_sw(q)];
+        const bool in = j * kHsThreads + t < n;
+        rank[j] = in ? atomicAdd(&bins[uint32_t((c[j] - kmin) >> sh)], 1u) : 0u;
+        c[j] = in ? ((c[j] - kmin) << idbits) | id[j] : ~0ull;
     }
-    int P = I;
-    while (P < n) P <<= 1;
-    hs_sort_words<I>(c, P, shk);
-    __syncthreads();  // the last round's reads are done
+    __syncthreads();
+    // bins -> starts, eight bins per thread
+    uint4 *b4 = reinterpret_cast<uint4 *>(bins) + 2 * t;
+    uint4 x = b4[0], y = b4[1];
+    const uint32_t most = max(max(max(x.x, x.y), max(x.z, x.w)), max(max(y.x, y.y), max(y.z, y.w)));
+    const uint32_t sum = x.x + x.y + x.z + x.w + y.x + y.y + y.z + y.w;
+    uint32_t inc = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t z = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+        if (lane >= d) inc += z;
+    }
+    if (lane == 31) wmin[warp] = inc;  // kmin is in registers
+    if (__syncthreads_or(most > kHsRankBin)) {
+        // words crowded in few bins: sorted by merging
+#pragma unroll
+        for (int j = 0; j < I; ++j) {
+            const int q = j * kHsThreads + t;
+            if (q < n) shk[hs_sw(q)] = c[j];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < I; ++j) c[j] = I * t + j < n ? shk[hs_sw(I * t + j)] : ~0ull;
+        int P = I;
+        while (P < n) P <<= 1;
+        hs_sort_words<I>(c, P, shk);
+        __syncthreads();  // the last round's reads are done
+#pragma unroll
+        for (int j = 0; j < I; ++j)
+            if (I * t + j < n) shk[hs_sw(I * t + j)] = c[j];
+        __syncthreads();
+        const unsigned long long mask = (1ull << idbits) - 1ull;
+        for (int q = t; q < n; q += kHsThreads) {
+            const unsigned long long w = shk[hs_sw(q)];
+            dk[q] = (w >> idbits) + kmin;
+            dv[q] = uint32_t(w & mask);
+        }
+        return;
+    }
+    uint32_t run = inc - sum;
+    for (int w = 0; w < warp; ++w) run += uint32_t(wmin[w]);
+    const uint32_t r1 = run + x.x, r2 = r1 + x.y, r3 = r2 + x.z, r4 = r3 + x.w, r5 = r4 + y.x, r6 = r5 + y.y,
+                   r7 = r6 + y.z;
+    b4[0] = make_uint4(run, r1, r2, r3);
+    b4[1] = make_uint4(r4, r5, r6, r7);
+    __syncthreads();
 #pragma unroll
     for (int j = 0; j < I; ++j)
-        if (I * t + j < n) shk[hs_sw(I * t + j)] = c[j];
+        if (j * kHsThreads + t < n) shk[bins[uint32_t((c[j] >> idbits) >> sh)] + rank[j]] = c[j];
     __syncthreads();
     const unsigned long long mask = (1ull << idbits) - 1ull;
-    for (int q = t; q < n; q += blockDim.x) {
-        const unsigned long long w = shk[hs_sw(q)];
-        dk[q] = (w >> idbits) + kmin;
-        dv[q] = uint32_t(w & mask);
+    for (int q = t; q < n; q += kHsThreads) {
+        const unsigned long long w = shk[q], k = w >> idbits;
+        const uint32_t b = uint32_t(k >> sh);
+        const int lo = int(bins[b]), hi = b + 1 < uint32_t(kHsBins) ? int(bins[b + 1]) : n;
+        int at = lo;
+        for (int z = lo; z < hi; ++z) at += shk[z] < w ? 1 : 0;  // words differ by their ids
+        dk[at] = k + kmin;
+        dv[at] = uint32_t(w & mask);
     }
 }
 
-// One block per bucket: sorts its pairs from the slots into the output.
+// One block per bucket: sorts its pairs from the slots into the output, and
+// leaves the bucket's counters at zero for the next sort.
 __global__ void __launch_bounds__(kHsThreads) k_hs_bucket(HsBuffers h, unsigned long long *__restrict__ slot_key,
                                                           uint32_t *__restrict__ slot_id,
                                                           unsigned long long *__restrict__ out_key,
                                                           uint32_t *__restrict__ out_id, int idbits) {
     __shared__ unsigned long long shk[kHsSmem];
-    __shared__ uint32_t shv[kHsSmem];
+    __shared__ __align__(16) uint32_t shv[kHsSmem];
     __shared__ unsigned long long wmin[kHsThreads / 32], wmax[kHsThreads / 32];
     const int u = blockIdx.x;
+    if (threadIdx.x == 0) {
+        h.count[u] = 0u;
+        h.cursor[u] = 0u;
+        if (u == 0) h.ticket[0] = h.ticket[1] = 0u;
+    }
     const int64_t b0 = h.start[u];
     const int64_t n = int64_t(h.start[u + 1]) - b0;
     if (n <= 0) return;
@@ -649,48 +729,48 @@ __global__ void __launch_bounds__(kHsThreads) k_hs_bucket(HsBuffers h, unsigned 
 
 }  // namespace
 
-// The sort on stream `st`, in two halves (the first ends once the samples
-// are ranked, so a caller can time the two apart): K <= hs_max_keys()
-// pairs; key_of(id) gives the key of id.  tmp_key/tmp_bucket and
-// slot_key/slot_id hold K entries each and may not alias the hint or the
-// output; the output may not alias the hint.
-template <class KeyOf>
-int hinted_sort_samples(KeyOf key_of, const uint32_t *hint, int64_t K, const HsBuffers &h, uint32_t *status,
-                        cudaStream_t st, const HsClears &clr = HsClears()) {
+// The sort on stream `st`; key_of(id) gives the key of id.  tmp_key/tmp_bucket
+// and slot_key/slot_id hold K entries each and may not alias the hint, the
+// splitters or the output.  The counters of `h` are zero before it, and after.
+template <class KeyOf, class Split>
+int hinted_sort_place(KeyOf key_of, Split split, const uint32_t *hint, int64_t K, const HsBuffers &h,
+                      unsigned long long *tmp_key, uint32_t *tmp_bucket, unsigned long long *slot_key,
+                      uint32_t *slot_id, unsigned long long *out_key, uint32_t *out_id, uint32_t *status,
+                      cudaStream_t st) {
     if (K <= 0) return BGV_OK;
-    if (K > hs_max_keys()) return BGV_EINVAL;
-    const HsShape sh = hs_shape(K);
-    int64_t first_work = 2;
-    for (const int64_t w : {int64_t(sh.ns), int64_t(sh.nb), clr.n_u64, clr.n_u32})
-        if (w > first_work) first_work = w;
-    note_launch(), k_hs_sample<KeyOf><<<grid_for(first_work, 256, sm_count() * 4), 256, 0, st>>>(
-        key_of, hint, K, sh.nb, sh.ns, h, clr, status);
-    BGV_TRY(launch_status());
-    if (sh.ns > 0) {
-        const dim3 g((sh.ns + 255) / 256, kHsRankSlices);
-        note_launch(), k_hs_rank<<<g, 256, 0, st>>>(sh.ns, sh.s, h);
-        BGV_TRY(launch_status());
-    }
-    return BGV_OK;
-}
-
-template <class KeyOf>
-int hinted_sort_place(KeyOf key_of, const uint32_t *hint, int64_t K, const HsBuffers &h, unsigned long long *tmp_key,
-                      uint32_t *tmp_bucket, unsigned long long *slot_key, uint32_t *slot_id,
-                      unsigned long long *out_key, uint32_t *out_id, uint32_t *status, cudaStream_t st) {
-    if (K <= 0) return BGV_OK;
-    if (K > hs_max_keys()) return BGV_EINVAL;
-    const HsShape sh = hs_shape(K);
-    note_launch(), k_hs_count<KeyOf><<<grid_for(K, 256, sm_count() * 8), 256, 0, st>>>(key_of, hint, K, sh.nb, h,
-                                                                                      tmp_key, tmp_bucket, status);
+    const int nb = hs_buckets(K);
+    note_launch(), k_hs_count<KeyOf, Split><<<grid_for(K, 256, sm_count() * 8), 256, 0, st>>>(
+        key_of, split, hint, K, nb, h, tmp_key, tmp_bucket, status);
     BGV_TRY(launch_status());
     note_launch(), k_hs_scatter<<<grid_for(K, 256, sm_count() * 8), 256, 0, st>>>(hint, K, h, tmp_key, tmp_bucket,
                                                                                  slot_key, slot_id);
     BGV_TRY(launch_status());
     int idbits = 0;  // bits of the largest id
     while (idbits < 32 && (int64_t(1) << idbits) < K) ++idbits;
-    note_launch(), k_hs_bucket<<<sh.nb, kHsThreads, 0, st>>>(h, slot_key, slot_id, out_key, out_id, idbits);
+    note_launch(), k_hs_bucket<<<nb, kHsThreads, 0, st>>>(h, slot_key, slot_id, out_key, out_id, idbits);
     return launch_status();
+}
+
+// The same with splitters from samples of the hint, K <= hs_max_keys(); the
+// output may not alias the hint.
+template <class KeyOf>
+int hinted_sort_sampled(KeyOf key_of, const uint32_t *hint, int64_t K, const HsBuffers &h, unsigned long long *tmp_key,
+                        uint32_t *tmp_bucket, unsigned long long *slot_key, uint32_t *slot_id,
+                        unsigned long long *out_key, uint32_t *out_id, uint32_t *status, cudaStream_t st) {
+    if (K <= 0) return BGV_OK;
+    if (K > hs_max_keys()) return BGV_EINVAL;
+    const HsShape sh = hs_shape(K);
+    const int64_t words = hs_counter_words(K);
+    note_launch(), k_hs_sample<KeyOf><<<grid_for(words > sh.ns ? words : sh.ns, 256, sm_count() * 4), 256, 0, st>>>(
+        key_of, hint, K, words, sh.ns, h, status);
+    BGV_TRY(launch_status());
+    if (sh.ns > 0) {
+        const dim3 g((sh.ns + 255) / 256, kHsRankSlices);
+        note_launch(), k_hs_rank<<<g, 256, 0, st>>>(sh.ns, sh.s, h);
+        BGV_TRY(launch_status());
+    }
+    return hinted_sort_place(key_of, HsSampled{h.spl_key, h.spl_id}, hint, K, h, tmp_key, tmp_bucket, slot_key, slot_id,
+                             out_key, out_id, status, st);
 }
 
 }  // namespace bgv

@@ -638,10 +638,13 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_cross(int64_t K, int L, i
 //   cell [a, b]      -> a + S[a] + (its ancestors that also start at a: the cells
 //                                   that leave the tile, then the outer ones inside)
 //   skip(cell [a,b]) -> b + 1 + S[b + 1] (the element after its subtree)
-// Elements are float4 (x, y, mass, side^2), side^2 = -1 for a body.
+// Elements are float4 (x, y, mass, side^2), side^2 = -1 for a body.  Also leaves
+// the tiles' flags and the step's interaction counter at zero, for the next
+// step's k_tile and the traversal after this kernel.
 __global__ void __launch_bounds__(kTileThreads) k_tile_emit(int64_t K, const float4 *__restrict__ body, TileArrays T,
                                                             uint32_t *__restrict__ S, float4 *__restrict__ geo,
-                                                            int32_t *__restrict__ skip) {
+                                                            int32_t *__restrict__ skip,
+                                                            unsigned long long *interactions) {
     __shared__ uint32_t nst4[kTile / 4], loc4[kTile / 4];  // cells that start at each body: all, inside the tile
     __shared__ uint32_t pre[kTile + 1];  // cells starting before each body, in this tile
     __shared__ uint32_t wsum[kTileThreads / 32];
@@ -650,6 +653,15 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_emit(int64_t K, const flo
     const int64_t tile = blockIdx.x, t0 = tile * kTile;
     const int n = K - t0 < kTile ? int(K - t0) : kTile;
     nst4[tid] = loc4[tid] = 4 * tid < n ? reinterpret_cast<const uint32_t *>(T.starts + t0)[tid] : 0u;
+    if (tid == 0) {
+        const int64_t tiles = gridDim.x;
+        T.flags[tile] = 0u;
+        if (tile % kTileGroup == 0) T.flags[tiles + 2 + tile / kTileGroup] = 0u;
+        if (tile == 0) {
+            T.flags[tiles] = T.flags[tiles + 1] = 0u;
+            *interactions = 0ull;
+        }
+    }
     const uint32_t base = T.base[tile], cells = T.cells[tile], opens = T.open_n[tile];
     __syncthreads();
     if (tid < int(opens)) {  // one entry per first body
