@@ -184,22 +184,30 @@ __device__ __forceinline__ void xsum_warp(XSum &S, XSum &T) {
     }
 }
 
-// Block-wide merge of one (S, T) pair per thread in a fixed tree; thread 0
-// receives the result.
+// Block-wide merge of one (S, T) pair per thread; thread 0 receives the result.
 template <int kBlock>
 __device__ __forceinline__ void xsum_block(XSum &S, XSum &T) {
-    __shared__ XPart sS[kBlock / 32], sT[kBlock / 32];
+    constexpr int kWarps = kBlock / 32;
+    __shared__ XPart part[2][kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     xsum_warp(S, T);
     if (lane == 0) {
-        sS[warp] = xsum_pack(S);
-        sT[warp] = xsum_pack(T);
+        part[0][warp] = xsum_pack(S);
+        part[1][warp] = xsum_pack(T);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < kBlock / 32; ++k) {
-            S = xsum_merge(S, XSum{(u128(sS[k].hi) << 64) | sS[k].lo, sS[k].q0, sS[k].bad});
-            T = xsum_merge(T, XSum{(u128(sT[k].hi) << 64) | sT[k].lo, sT[k].q0, sT[k].bad});
+    if (warp == 0) {
+        auto get = [&](int k) {
+            const XPart &x = part[k][lane];
+            return lane < kWarps ? XSum{(u128(x.hi) << 64) | x.lo, x.q0, x.bad} : xsum_zero();
+        };
+        S = get(0);
+        T = get(1);
+#pragma unroll
+        for (int d = kWarps / 2; d > 0; d >>= 1) {
+            const XSum oS = xsum_shfl_down(S, d), oT = xsum_shfl_down(T, d);
+            S = xsum_merge(S, oS);
+            T = xsum_merge(T, oT);
         }
     }
     __syncthreads();

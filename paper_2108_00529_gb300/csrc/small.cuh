@@ -1,7 +1,8 @@
 // small.cuh -- whole ForceAtlas2 runs on graphs of up to kSmallMax bodies.
 //
 // With few bodies a step of the general path is a chain of a dozen kernels that
-// each last a few microseconds (72 us per step at 219 bodies, 94 at 1,764).
+// each last a few microseconds (72 us per step at 219 bodies, 94 at 1,764; here
+// 19.8 and 36).
 // Here one cluster of blocks keeps a graph in shared memory and takes every
 // step of the run in one launch: each block builds the whole quadtree for
 // itself (sorting 2,048 bodies costs less than fetching a tree from elsewhere),
@@ -27,7 +28,10 @@ constexpr int kSmallHalf = kSmallThreads / 2;
 constexpr int kSmallCluster = 8;         // blocks per cluster, at most
 constexpr int kSmallIdBits = 11;         // ids < kSmallMax
 constexpr int kSmallRank = 32;           // largest bin ranked by counting
-constexpr int kSmallCache = 8192;        // CSR entries a block keeps (weights below 2^21)
+// CSR entries a block keeps (weights below 2^21): what is left of its shared
+// memory.  200 steps at 1,764 bodies took 9,683 us with 8,192, and 7,239 with
+// 10,240, lighter moments and the sums merged by a warp.
+constexpr int kSmallCache = 10240;
 constexpr int64_t kSmallEntries = int64_t(1) << 19;  // CSR entries of a graph, at most
 constexpr int kSmallChunk = 256;         // steps per launch, at most
 static_assert(kSmallMax == 4 * kSmallThreads, "four bodies a thread");
@@ -216,6 +220,7 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
         small_sort(m, w, K);
     }
     // Morton order: bodies and the levels between neighbours
+    uint32_t heaviest = 0u;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const int s = r * kSmallThreads + tid;
@@ -233,13 +238,14 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
             d = 0u;
         }
         levels[s] = 0u;
+        heaviest = max(heaviest, mass);
         m.sm[s] = mass;
         m.sux[s] = U.x;
         m.suy[s] = U.y;
         D[s] = uint8_t(d);
     }
     if (tid < 4) D[kSmallMax + tid] = uint8_t(tid == 0 && K == kSmallMax ? 0u : 255u);
-    __syncthreads();
+    const bool light = !__syncthreads_or(heaviest >= kLightMass);
     {
         uint32_t c = m.D4[tid];
         c = __vminu4(c, c >> 16);
@@ -251,15 +257,17 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
     {
         const uint4 m4 = reinterpret_cast<const uint4 *>(m.sm)[tid];
         const uint4 x4 = reinterpret_cast<const uint4 *>(m.sux)[tid], y4 = reinterpret_cast<const uint4 *>(m.suy)[tid];
-        Mom acc = mom_body(m4.x, x4.x, y4.x);
-        acc = mom_add(acc, mom_body(m4.y, x4.y, y4.y));
-        acc = mom_add(acc, mom_body(m4.z, x4.z, y4.z));
-        acc = mom_add(acc, mom_body(m4.w, x4.w, y4.w));
-        Mom inc = acc;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const Mom o = mom_shfl_up(inc, d);
-            if (lane >= d) inc = mom_add(inc, o);
+        Mom acc, inc;
+        if (light) {
+            const Mom64 a = mom64_add(mom64_add(mom64_add(mom64_add(Mom64{0u, 0ull, 0ull}, m4.x, x4.x, y4.x), m4.y, x4.y,
+                                                          y4.y), m4.z, x4.z, y4.z), m4.w, x4.w, y4.w);
+            const Mom64 i = mom64_warp_scan(a);
+            acc = Mom{a.M, a.X, a.Y};
+            inc = Mom{i.M, i.X, i.Y};
+        } else {
+            acc = mom_add(mom_add(mom_body(m4.x, x4.x, y4.x), mom_body(m4.y, x4.y, y4.y)),
+                          mom_add(mom_body(m4.z, x4.z, y4.z), mom_body(m4.w, x4.w, y4.w)));
+            inc = mom_warp_scan(acc);
         }
         if (lane == 31) {
             m.red[warp][0] = inc.M;
@@ -316,8 +324,17 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
         const uint32_t c = m.list[q];
         const int a = int(c & 2047u), b = int((c >> 11) & 2047u), v = int(c >> 27);
         const int at = a + m.S[a] + int((c >> 22) & 31u);
-        m.u.tree.geo[at] = cell_element(mom_sub(before_place(b + 1), before_place(a)), v, max(int(D[a]), int(D[b + 1])),
-                                        b - a + 1, L, leaf_cap, fr);
+        const int pv = max(int(D[a]), int(D[b + 1]));
+        if (light) {
+            auto before = [&](int j) {
+                Mom64 x = mom64_load(&m.Pq[j >> 2]);
+                for (int k = j & ~3; k < j; ++k) x = mom64_add(x, m.sm[k], m.sux[k], m.suy[k]);
+                return x;
+            };
+            m.u.tree.geo[at] = cell_element(before(a), before(b + 1), v, pv, b - a + 1, L, leaf_cap, fr);
+        } else {
+            m.u.tree.geo[at] = cell_element(mom_sub(before_place(b + 1), before_place(a)), v, pv, b - a + 1, L, leaf_cap, fr);
+        }
         m.u.tree.skip[at] = uint16_t(b + 1 + m.S[b + 1]);
     }
     for (int s = tid; s < K; s += kSmallThreads) {
@@ -340,6 +357,7 @@ __device__ __forceinline__ float2 small_rows(const SmallMem &m, bool have, int64
     float ax = 0.0f, ay = 0.0f;
     const int64_t len = have ? e - b : 0;
     if (len <= att_short) {
+#pragma unroll 4
         for (int64_t x = b; x < b + len; ++x) {
             float wf;
             const float2 pj = entry(x, pi, &wf);

@@ -27,6 +27,9 @@
 // (gather and moment scan 110, candidates 21, range searches 143, scan 19, layout
 // 42).  500 steps at 1 M bodies and 16 M CSR entries: 224.6 ms with it, 211.2 with
 // the tiles.
+// k_tile is bound by instruction issue (34 warp instructions a body).  Moments of
+// light bodies in 32 and 64 bits, with the centre's division by an estimate: 500
+// steps of 1 M bodies 190.0 -> 188.7 ms, of 160 graphs 488.5 -> 484.4 ms.
 #pragma once
 
 #include "bgv_internal.cuh"
@@ -160,10 +163,27 @@ inline void carve_tiles(Carver &c, int64_t K, TileArrays &t) {
     t.cross_meta = c.take<uint2>(n * kTileLevels);
 }
 
+// floor(X / M) when it is below 2^32: an FP32 estimate (relative error below
+// 2^-21, so off by at most 2^11), corrected by its exact remainder, and once more
+// by one.
+__device__ __forceinline__ uint32_t mean_u32(unsigned long long X, uint32_t M) {
+    const float r = __frcp_rn(__uint2float_rn(M));
+    uint32_t q = __float2uint_rz(__fmul_rn(__ull2float_rn(X), r));  // saturates
+    long long R = static_cast<long long>(X - static_cast<unsigned long long>(q) * M);
+    const int dq = __float2int_rd(__fmul_rn(__ll2float_rn(R), r));
+    q += uint32_t(dq);
+    R -= static_cast<long long>(dq) * static_cast<long long>(static_cast<unsigned long long>(M));
+    if (R < 0) --q;
+    if (R >= static_cast<long long>(static_cast<unsigned long long>(M))) ++q;
+    return q;
+}
+
 // The element of one cell: FP32 centre from the exact moments, mass, and the
 // squared side of the opening test (+inf for a leaf that is never accepted).
 // v, pv: its level and its parent's, plus one; n bodies.
-__device__ __forceinline__ float4 cell_element(const Mom &mom, int v, int pv, int64_t n, int L, int leaf_cap, float4 fr) {
+// qx, qy: the centre in fixed point; Mf: the mass.
+__device__ __forceinline__ float4 cell_element(uint32_t qx, uint32_t qy, float Mf, int v, int pv, int64_t n, int L,
+                                               int leaf_cap, float4 fr) {
     const int lev = v - 1, par_lev = pv - 1;
     const bool leaf = n <= leaf_cap || lev >= L;
     // A leaf made by the depth limit (coincident keys, more than leaf_cap
@@ -171,22 +191,70 @@ __device__ __forceinline__ float4 cell_element(const Mom &mom, int v, int pv, in
     // parent's level and L; the deepest of them, at level L - 1, takes the
     // opening test for the whole chain.
     const bool testable = leaf && n > leaf_cap && par_lev + 1 <= L - 1;
-    uint32_t qx = 0u, qy = 0u;
-    if (mom.M) {
-        if (((mom.X | mom.Y) >> 64) == 0) {  // small cells: 64-bit division
-            qx = uint32_t(static_cast<unsigned long long>(mom.X) / mom.M);
-            qy = uint32_t(static_cast<unsigned long long>(mom.Y) / mom.M);
-        } else {
-            qx = uint32_t(mom.X / mom.M);
-            qy = uint32_t(mom.Y / mom.M);
-        }
-    }
     const float two_m32 = 2.3283064365386963e-10f;  // 2^-32
     const float cx = __fadd_rn(fr.x, __fmul_rn(fr.z, __fmul_rn(__uint2float_rn(qx), two_m32)));
     const float cy = __fadd_rn(fr.y, __fmul_rn(fr.z, __fmul_rn(__uint2float_rn(qy), two_m32)));
     const float sl = __fmul_rn(fr.z, pow2_neg(testable ? L - 1 : lev));
     const float side2 = (leaf && !testable) ? INFINITY : __fmul_rn(sl, sl);
-    return make_float4(cx, cy, __ull2float_rn(mom.M), side2);
+    return make_float4(cx, cy, Mf, side2);
+}
+__device__ __forceinline__ float4 cell_element(const Mom &mom, int v, int pv, int64_t n, int L, int leaf_cap, float4 fr) {
+    uint32_t qx = 0u, qy = 0u;
+    if (mom.M) {
+        qx = uint32_t(mom.X / mom.M);
+        qy = uint32_t(mom.Y / mom.M);
+    }
+    return cell_element(qx, qy, __ull2float_rn(mom.M), v, pv, n, L, leaf_cap, fr);
+}
+
+// Bodies lighter than this: the moments of kSmallMax or kTile of them fit in 32
+// (mass) and 64 bits (coordinates), a third of the work of the full width.
+constexpr uint32_t kLightMass = 1u << 21;
+struct Mom64 {
+    uint32_t M;
+    unsigned long long X, Y;
+};
+__device__ __forceinline__ Mom64 mom64_add(Mom64 a, uint32_t m, uint32_t ux, uint32_t uy) {
+    a.M += m;
+    a.X += static_cast<unsigned long long>(m) * ux;
+    a.Y += static_cast<unsigned long long>(m) * uy;
+    return a;
+}
+// A prefix stored by momp_store whose values fit.
+__device__ __forceinline__ Mom64 mom64_load(const MomP *p) {
+    const uint4 a = p->a;
+    const uint2 b = *reinterpret_cast<const uint2 *>(&p->b);
+    return Mom64{a.x, (static_cast<unsigned long long>(a.w) << 32) | a.z, (static_cast<unsigned long long>(b.y) << 32) | b.x};
+}
+__device__ __forceinline__ float4 cell_element(const Mom64 &lo, const Mom64 &hi, int v, int pv, int n, int L,
+                                               int leaf_cap, float4 fr) {
+    const uint32_t M = hi.M - lo.M;
+    return cell_element(M ? mean_u32(hi.X - lo.X, M) : 0u, M ? mean_u32(hi.Y - lo.Y, M) : 0u, __uint2float_rn(M), v, pv,
+                        n, L, leaf_cap, fr);
+}
+// Inclusive warp scan.
+__device__ __forceinline__ Mom64 mom64_warp_scan(Mom64 a) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t M = __shfl_up_sync(0xFFFFFFFFu, a.M, d);
+        const unsigned long long X = __shfl_up_sync(0xFFFFFFFFu, a.X, d), Y = __shfl_up_sync(0xFFFFFFFFu, a.Y, d);
+        if (lane >= d) {
+            a.M += M;
+            a.X += X;
+            a.Y += Y;
+        }
+    }
+    return a;
+}
+__device__ __forceinline__ Mom mom_warp_scan(Mom a) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const Mom o = mom_shfl_up(a, d);
+        if (lane >= d) a = mom_add(a, o);
+    }
+    return a;
 }
 
 // Level down to which two keys agree, plus one (the graph bits come first).
@@ -269,6 +337,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
     const int n = K - t0 < kTile ? int(K - t0) : kTile;
 
     // bodies and boundaries, neighbouring threads on neighbouring bodies
+    uint32_t heaviest = 0u;
 #pragma unroll
     for (int r = 0; r < kTileItems; ++r) {
         const int e = r * kTileThreads + tid;
@@ -286,6 +355,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
             d = s < K ? level_between(keys[s - 1], keys[s], L, gbits) : 0u;
         }
         levels[e] = 0u;
+        heaviest = max(heaviest, m);
         sm[e] = m;
         sux[e] = U.x;
         suy[e] = U.y;
@@ -296,7 +366,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
         if (tid == 0 && n == kTile) d = t0 + kTile < K ? level_between(keys[t0 + kTile - 1], keys[t0 + kTile], L, gbits) : 0u;
         D[kTile + tid] = uint8_t(d);
     }
-    __syncthreads();
+    const bool light = !__syncthreads_or(heaviest >= kLightMass);
 
     // minima of D: per 64 places, and over the tile's own boundaries 1 .. n
     {
@@ -320,15 +390,17 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
     const uint4 x4 = reinterpret_cast<const uint4 *>(sux)[tid], y4 = reinterpret_cast<const uint4 *>(suy)[tid];
     Mom total;
     {
-        Mom acc = mom_body(m4.x, x4.x, y4.x);
-        acc = mom_add(acc, mom_body(m4.y, x4.y, y4.y));
-        acc = mom_add(acc, mom_body(m4.z, x4.z, y4.z));
-        acc = mom_add(acc, mom_body(m4.w, x4.w, y4.w));
-        Mom inc = acc;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const Mom o = mom_shfl_up(inc, d);
-            if (lane >= d) inc = mom_add(inc, o);
+        Mom acc, inc;
+        if (light) {
+            const Mom64 a = mom64_add(mom64_add(mom64_add(mom64_add(Mom64{0u, 0ull, 0ull}, m4.x, x4.x, y4.x), m4.y, x4.y,
+                                                          y4.y), m4.z, x4.z, y4.z), m4.w, x4.w, y4.w);
+            const Mom64 i = mom64_warp_scan(a);
+            acc = Mom{a.M, a.X, a.Y};
+            inc = Mom{i.M, i.X, i.Y};
+        } else {
+            acc = mom_add(mom_add(mom_body(m4.x, x4.x, y4.x), mom_body(m4.y, x4.y, y4.y)),
+                          mom_add(mom_body(m4.z, x4.z, y4.z), mom_body(m4.w, x4.w, y4.w)));
+            inc = mom_warp_scan(acc);
         }
         if (lane == 31) {
             red_sh[warp][0] = inc.M;
@@ -425,11 +497,19 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
     for (uint32_t q = tid; q < cells; q += kTileThreads) {
         const uint32_t c = list[q];
         const int a = int(c & 1023u), b = int((c >> 10) & 1023u), v = int(c >> 20);
-        const Mom mom = mom_sub(before_place(b + 1), before_place(a));
         const int pv = max(int(D[a]), int(D[b + 1]));
         // positions of graph g in Morton order are its index range too
         const float4 fr = frames[bgraph ? bgraph[t0 + a] : 0];
-        T.cell[t0 + q] = cell_element(mom, v, pv, b - a + 1, L, leaf_cap, fr);
+        if (light) {
+            auto before = [&](int j) {
+                Mom64 x = mom64_load(&Pq[j >> 2]);
+                for (int k = j & ~3; k < j; ++k) x = mom64_add(x, sm[k], sux[k], suy[k]);
+                return x;
+            };
+            T.cell[t0 + q] = cell_element(before(a), before(b + 1), v, pv, b - a + 1, L, leaf_cap, fr);
+        } else {
+            T.cell[t0 + q] = cell_element(mom_sub(before_place(b + 1), before_place(a)), v, pv, b - a + 1, L, leaf_cap, fr);
+        }
         T.meta[t0 + q] = (c & 0xFFFFFu) | (uint32_t(__popc(levels[a] & ((1u << v) - 1u))) << 20);
     }
 
