@@ -2,7 +2,7 @@
 //
 // With few bodies a step of the general path is a chain of a dozen kernels that
 // each last a few microseconds (72 us per step at 219 bodies, 94 at 1,764; here
-// 19.8 and 36).
+// 18.0 and 30).
 // Here one cluster of blocks keeps a graph in shared memory and takes every
 // step of the run in one launch: each block builds the whole quadtree for
 // itself (sorting 2,048 bodies costs less than fetching a tree from elsewhere),
@@ -30,7 +30,8 @@ constexpr int kSmallIdBits = 11;         // ids < kSmallMax
 constexpr int kSmallRank = 32;           // largest bin ranked by counting
 // CSR entries a block keeps (weights below 2^21): what is left of its shared
 // memory.  200 steps at 1,764 bodies took 9,683 us with 8,192, and 7,239 with
-// 10,240, lighter moments and the sums merged by a warp.
+// 10,240, lighter moments and the sums merged by a warp (then 5,996 with the
+// cells found by LevelBits).
 constexpr int kSmallCache = 10240;
 constexpr int64_t kSmallEntries = int64_t(1) << 19;  // CSR entries of a graph, at most
 constexpr int kSmallChunk = 256;         // steps per launch, at most
@@ -58,7 +59,11 @@ struct SmallMem {
     float4 body[kSmallMax];              // Morton order: x, y, mass, id
     uint32_t mass[kSmallMax];            // by id
     uint32_t sm[kSmallMax], sux[kSmallMax], suy[kSmallMax];  // Morton order: mass, fixed-point position
-    MomP Pq[kSmallThreads + 1];          // moments before every fourth body
+    union {
+        LevelBits<kSmallMax / 32> bits;
+        MomP Pq[kSmallThreads + 1];      // then: moments before every fourth body
+    } w;
+    unsigned long long some[32];         // of the bits
     union {
         struct {
             unsigned long long a[kSmallMax], b[kSmallMax];  // key << kSmallIdBits | id
@@ -72,7 +77,6 @@ struct SmallMem {
     uint32_t list[kSmallMax];            // cells: first | last << 11 | outer cells from it << 22 | level << 27
     uint32_t D4[kSmallThreads + 1];
     uint16_t S[kSmallMax + 2];           // cells that start before each body
-    uint8_t chunk[kSmallMax / 64];
     uint32_t cache[kSmallCache];         // neighbour << 21 | weight
     float2 frep[kSmallHalf];             // repulsion of the block's nodes (written by the walkers of all blocks)
     XPart xpart[kSmallCluster][2];       // every block's S and T
@@ -80,7 +84,7 @@ struct SmallMem {
     float4 box[kSmallThreads / 32];
     unsigned long long kmin[kSmallThreads / 32], kmax[kSmallThreads / 32];
     uint32_t wsum[kSmallThreads / 32];
-    uint32_t cells;
+    uint32_t cells, greatest;
     double speed;
 };
 
@@ -203,7 +207,8 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
     for (int i = tid; i < K; i += kSmallThreads) box_add(box, m.pos[i]);
     box_warp(box);
     if (lane == 0) m.box[warp] = box;
-    if (tid == 0) m.cells = 0u;
+    if (tid == 0) m.cells = m.greatest = 0u;
+    if (tid < 32) m.some[tid] = 0ull;
     __syncthreads();
     box = m.box[0];
     for (int q = 1; q < kSmallThreads / 32; ++q) box_merge(box, m.box[q]);
@@ -220,7 +225,7 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
         small_sort(m, w, K);
     }
     // Morton order: bodies and the levels between neighbours
-    uint32_t heaviest = 0u;
+    uint32_t heaviest = 0u, greatest = 0u, ds = 0u;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const int s = r * kSmallThreads + tid;
@@ -243,17 +248,35 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
         m.sux[s] = U.x;
         m.suy[s] = U.y;
         D[s] = uint8_t(d);
+        ds |= d << (8 * r);
+        if (d != 255u) greatest = max(greatest, d);
     }
-    if (tid < 4) D[kSmallMax + tid] = uint8_t(tid == 0 && K == kSmallMax ? 0u : 255u);
+    if (tid == 0) D[kSmallMax] = K == kSmallMax ? 0u : 255u;
+    greatest = __reduce_max_sync(0xFFFFFFFFu, greatest);
+    if (lane == 0) atomicMax(&m.greatest, greatest);
     const bool light = !__syncthreads_or(heaviest >= kLightMass);
     {
-        uint32_t c = m.D4[tid];
-        c = __vminu4(c, c >> 16);
-        c = min(c & 0xFFu, (c >> 8) & 0xFFu);
+        const uint32_t hi = m.greatest;  // the least is 0, at place 0
 #pragma unroll
-        for (int d = 8; d > 0; d >>= 1) c = min(c, __shfl_xor_sync(0xFFFFFFFFu, c, d));
-        if ((lane & 15) == 0) m.chunk[tid >> 4] = uint8_t(c);
+        for (int r = 0; r < 4; ++r)
+            if (r * kSmallThreads + warp * 32 <= K)  // words past the end are not asked for
+                m.w.bits.add((ds >> (8 * r)) & 255u, r * (kSmallThreads / 32) + warp, 0u, hi, m.some);
     }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int j = r * kSmallThreads + tid + 1;
+        const uint32_t v = j < K ? D[j] : 0u;  // the end of all bodies closes every cell and stands for none
+        if (v == 0u) continue;
+        const int a = m.w.bits.last(int(v), m.some[v], j - 1);  // place 0 is not above any
+        if (D[a] == v) continue;
+        int e = m.w.bits.first(int(v) - 1, m.some[v - 1], j + 1 < kSmallMax ? j + 1 : kSmallMax - 1);
+        if (e <= j) e = kSmallMax;
+        m.list[atomicAdd(&m.cells, 1u)] = uint32_t(a) | (uint32_t(e - 1) << 11) | (v << 27);
+        atomicOr(&levels[a], 1u << v);
+    }
+    __syncthreads();  // the bits are done with: their memory takes the moments
+    const uint32_t cells = m.cells;
     {
         const uint4 m4 = reinterpret_cast<const uint4 *>(m.sm)[tid];
         const uint4 x4 = reinterpret_cast<const uint4 *>(m.sux)[tid], y4 = reinterpret_cast<const uint4 *>(m.suy)[tid];
@@ -276,38 +299,28 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
             m.red[warp][3] = static_cast<unsigned long long>(inc.Y);
             m.red[warp][4] = static_cast<unsigned long long>(inc.Y >> 64);
         }
-        __syncthreads();
-        Mom before = mom_zero();
-        for (int q = 0; q < warp; ++q)
-            before = mom_add(before, Mom{m.red[q][0], (u128(m.red[q][2]) << 64) | m.red[q][1],
-                                         (u128(m.red[q][4]) << 64) | m.red[q][3]});
-        before = mom_add(before, inc);
-        momp_store(&m.Pq[tid], mom_sub(before, acc));
-        if (tid == kSmallThreads - 1) momp_store(&m.Pq[kSmallThreads], before);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int j = r * kSmallThreads + tid + 1;
-        const uint32_t v = j < K ? D[j] : 0u;  // the end of all bodies closes every cell and stands for none
-        if (v == 0u) continue;
-        const int a = last_not_above(m.D4, m.chunk, j - 1, v);
-        if (a < 0 || D[a] == v) continue;
-        const int e = next_below<kSmallMax / 4>(m.D4, m.chunk, j + 1, v);
-        m.list[atomicAdd(&m.cells, 1u)] = uint32_t(a) | (uint32_t(e - 1) << 11) | (v << 27);
-        atomicOr(&levels[a], 1u << v);
-    }
-    __syncthreads();
-    const uint32_t cells = m.cells;
-    {
         const uint4 x = reinterpret_cast<const uint4 *>(levels)[tid];
         const uint32_t c0 = __popc(x.x), c1 = __popc(x.y), c2 = __popc(x.z), c3 = __popc(x.w);
-        const uint32_t run = small_scan(c0 + c1 + c2 + c3, m.wsum);
+        const uint32_t run = small_scan(c0 + c1 + c2 + c3, m.wsum);  // its barriers order m.red too
         m.S[4 * tid] = uint16_t(run);
         m.S[4 * tid + 1] = uint16_t(run + c0);
         m.S[4 * tid + 2] = uint16_t(run + c0 + c1);
         m.S[4 * tid + 3] = uint16_t(run + c0 + c1 + c2);
         if (tid == kSmallThreads - 1) m.S[kSmallMax] = uint16_t(run + c0 + c1 + c2 + c3);
+        Mom before = mom_zero();
+        if (light) {
+            Mom64 b{0u, 0ull, 0ull};
+            for (int q = 0; q < warp; ++q)
+                b = Mom64{b.M + uint32_t(m.red[q][0]), b.X + m.red[q][1], b.Y + m.red[q][3]};
+            before = Mom{b.M, b.X, b.Y};
+        } else {
+            for (int q = 0; q < warp; ++q)
+                before = mom_add(before, Mom{m.red[q][0], (u128(m.red[q][2]) << 64) | m.red[q][1],
+                                             (u128(m.red[q][4]) << 64) | m.red[q][3]});
+        }
+        before = mom_add(before, inc);
+        momp_store(&m.w.Pq[tid], mom_sub(before, acc));
+        if (tid == kSmallThreads - 1) momp_store(&m.w.Pq[kSmallThreads], before);
     }
     for (uint32_t q = tid; q < cells; q += kSmallThreads) {
         const uint32_t c = m.list[q];
@@ -315,7 +328,7 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
     }
     __syncthreads();
     auto before_place = [&](int j) {
-        Mom v = momp_load(&m.Pq[j >> 2]);
+        Mom v = momp_load(&m.w.Pq[j >> 2]);
         for (int q = j & ~3; q < j; ++q) v = mom_add(v, mom_body(m.sm[q], m.sux[q], m.suy[q]));
         return v;
     };
@@ -327,7 +340,7 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
         const int pv = max(int(D[a]), int(D[b + 1]));
         if (light) {
             auto before = [&](int j) {
-                Mom64 x = mom64_load(&m.Pq[j >> 2]);
+                Mom64 x = mom64_load(&m.w.Pq[j >> 2]);
                 for (int k = j & ~3; k < j; ++k) x = mom64_add(x, m.sm[k], m.sux[k], m.suy[k]);
                 return x;
             };

@@ -10,7 +10,7 @@
 // starts the cell, and the nearest after j with D < v ends it.  So every
 // boundary asks for itself, with two short searches, whether it stands for a
 // cell and for which; a tile of bodies finds nearly all of its cells in shared
-// memory (bytes of D, four per comparison, 64 per skip).  (Walking all the cells
+// memory (a bit row per level, LevelBits).  (Walking all the cells
 // that start at a body instead left most lanes waiting for the one with the
 // longest chain: 207 us for k_tile at 3.2 M bodies.)
 //   k_tile       gathers the bodies of a tile in Morton order, their levels D
@@ -27,10 +27,16 @@
 // (gather and moment scan 110, candidates 21, range searches 143, scan 19, layout
 // 42).  500 steps at 1 M bodies and 16 M CSR entries: 224.6 ms with it, 211.2 with
 // the tiles.
-// k_tile is bound by instruction issue (34 warp instructions a body).  Moments of
-// light bodies in 32 and 64 bits, with the centre's division by an estimate: 500
-// steps of 1 M bodies 190.0 -> 188.7 ms, of 160 graphs 488.5 -> 484.4 ms.
+// k_tile is bound by instruction issue.  Searching the bytes of D, four per
+// comparison and 64 per skip, it took 34 warp instructions a body with 18 lanes
+// active, as a warp waits for its longest search; with the bit rows (about one
+// ballot and one store per level and 32 bodies, then two words per search) 500
+// steps of 1 M bodies fell from 188.7 to 177.5 ms and 300 steps of 160 graphs
+// (5.7 M bodies) from 484.4 to 456.6 ms.  Before that, moments of light bodies in 32 and 64 bits,
+// with the centre's division by an estimate: 190.0 -> 188.7 and 488.5 -> 484.4 ms.
 #pragma once
+
+#include <type_traits>
 
 #include "bgv_internal.cuh"
 
@@ -264,40 +270,51 @@ __device__ __forceinline__ uint32_t level_between(unsigned long long a, unsigned
     return delta < gbits ? 0u : uint32_t((delta - gbits) >> 1) + 1u;
 }
 
-// Last place <= from with D <= v; -1 if there is none.
-__device__ __forceinline__ int last_not_above(const uint32_t *D4, const uint8_t *chunk, int from, uint32_t v) {
-    const uint32_t vv = v * 0x01010101u;
-    int w = from >> 2;
-    uint32_t x = D4[w] | ((from & 3) == 3 ? 0u : ~0u << (8 * ((from & 3) + 1)));  // the bytes after `from` never count
-    while (true) {
-        const uint32_t hit = __vcmpleu4(x, vv);
-        if (hit) return 4 * w + ((31 - __clz(int(hit))) >> 3);
-        if (w == 0) return -1;
-        --w;
-        while ((w & 15) == 15 && chunk[w >> 4] > v) {
-            if (w < 16) return -1;
-            w -= 16;
-        }
-        x = D4[w];
-    }
-}
-
-// First place >= from with D < v (D as bytes in kWords + 1 words, 255 past the
-// end; chunk: the minimum of every 64 bytes); past the words if there is none.
+// Where D <= v, a bit per place, for every level v between the least and the
+// greatest of a tile: a row of kWords words per level (kept kWords + 1 apart, as
+// neighbouring threads ask different rows for the same word) and a word that
+// tells which of them are not zero.  The nearest place before or after another
+// takes at most two words, however far it is.
 template <int kWords>
-__device__ __forceinline__ int next_below(const uint32_t *D4, const uint8_t *chunk, int from, uint32_t v) {
-    const uint32_t vv = v * 0x01010101u;
-    int w = from >> 2;
-    uint32_t x = D4[w] | ((1u << (8 * (from & 3))) - 1u);  // the bytes before `from` never count
-    while (true) {
-        const uint32_t hit = __vcmpltu4(x, vv);
-        if (hit) return 4 * w + ((__ffs(int(hit)) - 1) >> 3);
-        ++w;
-        while ((w & 15) == 0 && w < kWords && chunk[w >> 4] >= v) w += 16;
-        if (w > kWords) return 4 * (kWords + 1);
-        x = D4[w];
+struct LevelBits {
+    using Some = typename std::conditional<kWords == 32, uint32_t, unsigned long long>::type;
+    uint32_t row[32][kWords + 1];
+    // Every thread of a warp, with the value of its place of word w; lo <= hi, at most 32 levels.
+    __device__ __forceinline__ void add(uint32_t d, int w, uint32_t lo, uint32_t hi, Some *some) {
+        const uint32_t lane = threadIdx.x & 31;
+        uint32_t keep = 0u;
+        for (uint32_t v = lo; v <= hi; ++v) {
+            const uint32_t x = __ballot_sync(0xFFFFFFFFu, d <= v);
+            if (lane == v - lo) keep = x;
+        }
+        if (lane <= hi - lo) row[lane][w] = keep;
+        if (keep) atomicOr(&some[lane], Some(1) << w);
     }
-}
+    // Last place <= from in row r; -1 if there is none.
+    __device__ __forceinline__ int last(int r, Some some, int from) const {
+        int w = from >> 5;
+        uint32_t x = row[r][w] & (0xFFFFFFFFu >> (31 - (from & 31)));
+        if (!x) {
+            const Some s = some & ((Some(1) << w) - 1);
+            if (!s) return -1;
+            w = kWords == 32 ? 31 - __clz(int(s)) : 63 - __clzll(static_cast<long long>(s));
+            x = row[r][w];
+        }
+        return 32 * w + 31 - __clz(int(x));
+    }
+    // First place >= from (below 32 kWords) in row r; -1 if there is none.
+    __device__ __forceinline__ int first(int r, Some some, int from) const {
+        int w = from >> 5;
+        uint32_t x = row[r][w] & (0xFFFFFFFFu << (from & 31));
+        if (!x) {
+            const Some s = some & (~Some(1) << w);
+            if (!s) return -1;
+            w = (kWords == 32 ? __ffs(int(s)) : __ffsll(static_cast<long long>(s))) - 1;
+            x = row[r][w];
+        }
+        return 32 * w + __ffs(int(x)) - 1;
+    }
+};
 
 // Gather, levels, moments and the cells inside each tile of kTile bodies.  A
 // tile's blocks take tiles in order from a counter, so a tile's look-back waits
@@ -308,17 +325,20 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
     const int32_t *__restrict__ bgraph, int L, int gbits, int leaf_cap, float4 *__restrict__ body, TileArrays T,
     uint32_t *dev_status, int spin_limit) {
     __shared__ __align__(16) uint32_t sm[kTile], sux[kTile], suy[kTile];  // masses, fixed-point coordinates
-    __shared__ MomP Pq[kTileThreads + 1];                 // moments before every fourth body
+    __shared__ union {
+        LevelBits<kTile / 32> bits;
+        MomP Pq[kTileThreads + 1];                        // then: moments before every fourth body
+    } u;
+    __shared__ uint32_t some[32];                         // of the bits
     __shared__ uint32_t D4[kTile / 4 + 1];                // D of places 0 .. kTile (bytes)
     __shared__ uint32_t nst4[kTile / 4];                  // cells starting at each body (bytes)
     __shared__ uint16_t npre[kTileThreads + 1];           // cells starting before every fourth body
-    __shared__ uint8_t chunk[kTile / 64];
     __shared__ uint32_t list[kTile];                      // cells: first | last << 10 | level << 20
     __shared__ uint32_t levels[kTile];                    // levels of the cells that start at each body (bit mask)
     __shared__ uint32_t open_sh[kTileLevels + 6];
     __shared__ uint32_t wsum[kTileThreads / 32];
     __shared__ unsigned long long red_sh[kTileThreads / 32][5];
-    __shared__ uint32_t cells_sh, opens_sh, min_sh;
+    __shared__ uint32_t cells_sh, opens_sh, min_sh, max_sh;
     __shared__ unsigned tile_sh;
     __shared__ int near_sh;
     uint8_t *D = reinterpret_cast<uint8_t *>(D4), *nst = reinterpret_cast<uint8_t *>(nst4);
@@ -329,7 +349,9 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
         cells_sh = 0u;
         opens_sh = 0u;
         min_sh = 255u;
+        max_sh = 0u;
     }
+    if (tid < 32) some[tid] = 0u;
     __syncthreads();
     const int64_t tile = tile_sh;
     if (tile >= tiles) return;
@@ -337,7 +359,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
     const int n = K - t0 < kTile ? int(K - t0) : kTile;
 
     // bodies and boundaries, neighbouring threads on neighbouring bodies
-    uint32_t heaviest = 0u;
+    uint32_t heaviest = 0u, least = 255u, greatest = 0u, ds = 0u;
 #pragma unroll
     for (int r = 0; r < kTileItems; ++r) {
         const int e = r * kTileThreads + tid;
@@ -360,31 +382,58 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
         sux[e] = U.x;
         suy[e] = U.y;
         D[e] = uint8_t(d);
+        ds |= d << (8 * r);
+        if (e > 0) least = min(least, d);
+        if (d != 255u) greatest = max(greatest, d);
     }
-    if (tid < 4) {  // place kTile, and padding
+    if (tid == 0) {  // place kTile
         uint32_t d = 255u;
-        if (tid == 0 && n == kTile) d = t0 + kTile < K ? level_between(keys[t0 + kTile - 1], keys[t0 + kTile], L, gbits) : 0u;
-        D[kTile + tid] = uint8_t(d);
+        if (n == kTile) {
+            d = t0 + kTile < K ? level_between(keys[t0 + kTile - 1], keys[t0 + kTile], L, gbits) : 0u;
+            least = min(least, d);
+            greatest = max(greatest, d);
+        }
+        D[kTile] = uint8_t(d);
+    }
+    least = __reduce_min_sync(0xFFFFFFFFu, least);
+    greatest = __reduce_max_sync(0xFFFFFFFFu, greatest);
+    if (lane == 0) {
+        atomicMin(&min_sh, least);  // over the tile's own boundaries 1 .. n
+        atomicMax(&max_sh, greatest);
     }
     const bool light = !__syncthreads_or(heaviest >= kLightMass);
-
-    // minima of D: per 64 places, and over the tile's own boundaries 1 .. n
-    {
-        const uint32_t x = D4[tid];
-        uint32_t c = __vminu4(x, x >> 16);
-        c = min(c & 0xFFu, (c >> 8) & 0xFFu);
-        uint32_t own = tid ? c : min(min((x >> 8) & 0xFFu, (x >> 16) & 0xFFu), x >> 24);
-        if (tid == 0) own = min(own, D4[kTile / 4] & 0xFFu);
+    const uint32_t lo = min(min_sh, uint32_t(D[0])), top = max_sh;
 #pragma unroll
-        for (int d = 8; d > 0; d >>= 1) {
-            c = min(c, __shfl_xor_sync(0xFFFFFFFFu, c, d));
-            own = min(own, __shfl_xor_sync(0xFFFFFFFFu, own, d));
+    for (int r = 0; r < kTileItems; ++r) u.bits.add((ds >> (8 * r)) & 255u, r * (kTileThreads / 32) + warp, lo, top, some);
+    __syncthreads();
+
+    // the cells: boundary j stands for one if it is the first of its smallest
+    auto next_below = [&](int from, uint32_t v) {  // first place >= from with D < v
+        int e = -1;
+        if (v > lo && from < kTile) {
+            const int r = int(min(v - 1u, top) - lo);
+            e = u.bits.first(r, some[r], from);
         }
-        if ((lane & 15) == 0) {
-            chunk[tid >> 4] = uint8_t(c);
-            atomicMin(&min_sh, own);
+        return e >= 0 ? e : D[kTile] < v ? kTile : kTile + 1;
+    };
+#pragma unroll
+    for (int r = 0; r < kTileItems; ++r) {
+        const int j = r * kTileThreads + tid + 1;
+        const uint32_t v = j <= n ? D[j] : 0u;
+        if (v == 0u) continue;
+        const int a = u.bits.last(int(v - lo), some[v - lo], j - 1);
+        if (a < 0 || D[a] == v) continue;  // the cell starts before the tile, or an earlier boundary stands for it
+        const int e = next_below(j + 1, v);
+        if (e > n) {  // still open at the tile's end
+            open_sh[atomicAdd(&opens_sh, 1u)] = uint32_t(a) | (v << 10) | (uint32_t(D[a]) << 15);
+        } else {
+            list[atomicAdd(&cells_sh, 1u)] = uint32_t(a) | (uint32_t(e - 1) << 10) | (v << 20);
+            atomicOr(&levels[a], 1u << v);
         }
     }
+    const int first_below = warp == 0 && lane > 0 ? next_below(1, uint32_t(lane)) : kTile + 1;  // of level `lane`
+    __syncthreads();  // the bits are done with: their memory takes the moments
+
     // moment prefixes, a thread on four consecutive bodies
     const uint4 m4 = reinterpret_cast<const uint4 *>(sm)[tid];
     const uint4 x4 = reinterpret_cast<const uint4 *>(sux)[tid], y4 = reinterpret_cast<const uint4 *>(suy)[tid];
@@ -412,38 +461,27 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
         __syncthreads();
         Mom before = mom_zero();
         total = mom_zero();
-        for (int w = 0; w < kTileThreads / 32; ++w) {
+        if (light) {
+            Mom64 b{0u, 0ull, 0ull}, t = b;
+            for (int w = 0; w < kTileThreads / 32; ++w) {
+                if (w == warp) b = t;
+                t = Mom64{t.M + uint32_t(red_sh[w][0]), t.X + red_sh[w][1], t.Y + red_sh[w][3]};
+            }
+            before = Mom{b.M, b.X, b.Y};
+            total = Mom{t.M, t.X, t.Y};
+        } else for (int w = 0; w < kTileThreads / 32; ++w) {
             const Mom t{red_sh[w][0], (u128(red_sh[w][2]) << 64) | red_sh[w][1], (u128(red_sh[w][4]) << 64) | red_sh[w][3]};
             if (w < warp) before = mom_add(before, t);
             total = mom_add(total, t);
         }
-        momp_store(&Pq[tid], mom_sub(mom_add(before, inc), acc));
-        if (tid == 0) momp_store(&Pq[kTileThreads], total);
+        momp_store(&u.Pq[tid], mom_sub(mom_add(before, inc), acc));
+        if (tid == 0) momp_store(&u.Pq[kTileThreads], total);
     }
     if (tid == 0) {
         momp_store(tile == 0 ? &T.incl[0] : &T.agg[tile], total);
         __threadfence();
         atomicExch(&T.flags[tile], tile == 0 ? kMomIncl : kMomAgg);
     }
-    __syncthreads();
-
-    // the cells: boundary j stands for one if it is the first of its smallest
-#pragma unroll
-    for (int r = 0; r < kTileItems; ++r) {
-        const int j = r * kTileThreads + tid + 1;
-        const uint32_t v = j <= n ? D[j] : 0u;
-        if (v == 0u) continue;
-        const int a = last_not_above(D4, chunk, j - 1, v);
-        if (a < 0 || D[a] == v) continue;  // the cell starts before the tile, or an earlier boundary stands for it
-        const int e = next_below<kTile / 4>(D4, chunk, j + 1, v);
-        if (e > n) {  // still open at the tile's end
-            open_sh[atomicAdd(&opens_sh, 1u)] = uint32_t(a) | (v << 10) | (uint32_t(D[a]) << 15);
-        } else {
-            list[atomicAdd(&cells_sh, 1u)] = uint32_t(a) | (uint32_t(e - 1) << 10) | (v << 20);
-            atomicOr(&levels[a], 1u << v);
-        }
-    }
-    __syncthreads();
 #pragma unroll
     for (int r = 0; r < kTileItems; ++r) nst[r * kTileThreads + tid] = uint8_t(__popc(levels[r * kTileThreads + tid]));
     __syncthreads();
@@ -469,12 +507,12 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
     __syncthreads();
     // moments of the tile's bodies before place j
     auto before_place = [&](int j) {
-        Mom v = momp_load(&Pq[j >> 2]);
+        Mom v = momp_load(&u.Pq[j >> 2]);
         for (int q = j & ~3; q < j; ++q) v = mom_add(v, mom_body(sm[q], sux[q], suy[q]));
         return v;
     };
     if (warp == 0 && lane < kTileLevels) {  // the first boundary below each level
-        const int j = lane ? next_below<kTile / 4>(D4, chunk, 1, uint32_t(lane)) : kTile + 1;
+        const int j = first_below;
         uint32_t word = 0u;
         if (j <= n) {
             uint32_t c = npre[j >> 2];
@@ -502,7 +540,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
         const float4 fr = frames[bgraph ? bgraph[t0 + a] : 0];
         if (light) {
             auto before = [&](int j) {
-                Mom64 x = mom64_load(&Pq[j >> 2]);
+                Mom64 x = mom64_load(&u.Pq[j >> 2]);
                 for (int k = j & ~3; k < j; ++k) x = mom64_add(x, sm[k], sux[k], suy[k]);
                 return x;
             };
