@@ -24,8 +24,8 @@
 //      last block turns the counts into bucket starts.
 //   3. Scatter: every pair to its bucket (one atomic per bucket per warp).
 //   4. Bucket sort: one block per bucket.  Up to kHsCap pairs it sorts in
-//      shared memory, as single words (key - min key) << idbits | id when the
-//      bucket's keys span few enough bits: words go to bins by their high bits
+//      shared memory, as single words of its key above the least one and its id
+//      (or its place, when the keys span too many bits): words go to bins by their high bits
 //      (shared-memory atomics) and are ranked inside their bins, which hold a
 //      word or two; a bin too full for that (keys crowded in a corner of the
 //      bucket), or keys too far apart for one word, take a merge sort in
@@ -49,6 +49,8 @@ constexpr int kHsThreads = 256;         // bucket-sort block
 constexpr int kHsItems = 8;             // pairs (or words) per thread
 constexpr int kHsPairCap = kHsThreads * kHsItems;  // 2048: a chunk of the pair sort
 constexpr int kHsCap = kHsPairCap;      // larger buckets take the chunked path
+constexpr int kHsCapBits = 11;
+static_assert(kHsCap == 1 << kHsCapBits, "places of a bucket");
 constexpr int kHsRankSlices = 16;       // slices of the samples per ranking thread
 constexpr int kHsBins = 2048;           // bins of a bucket's words
 constexpr uint32_t kHsRankBin = 32;     // largest bin ranked by counting
@@ -573,14 +575,21 @@ __device__ void hs_pairs_chunked(unsigned long long *sk, uint32_t *sv, int64_t n
     }
 }
 
-// A bucket of n <= I * blockDim.x pairs.  If its keys span less than 2^(63 -
-// idbits), the words (key - kmin) << idbits | id (ids < 2^idbits) order exactly
-// as (key, id) and are sorted as single words: to kHsBins bins by the high bits
-// of the span, then ranked inside their bins and written to their places; with
-// a bin of more than kHsRankBin words, merged instead.  Otherwise the pairs are
-// sorted as pairs.  Every thread of the block calls it.
-// Bound by instruction issue.  The bins take about 140 instructions per pair,
-// the merge rounds 720 (155 us for 3.2 M bodies).
+// A bucket of n <= I * blockDim.x pairs, sorted as single words.  If its keys
+// span less than 2^(63 - idbits), the words (key - kmin) << idbits | id (ids <
+// 2^idbits) order exactly as (key, id).  Wider keys (up to 2^52: a batch's graph
+// ids and Morton bits) take the pair's place in the bucket instead of its id, and
+// equal keys look their ids up; that keeps the block at 8 bytes a pair, which
+// matters beside its own time (keys and ids apart, 34 KB for 26 a block, slowed
+// the attraction that shares the L1: 500 steps at 1 M bodies 191.4 for 188.7 ms).
+// Words go to kHsBins bins by the high bits of the span, are ranked inside their
+// bins and written to their places; with a bin of more than kHsRankBin words they
+// are merged instead, and words with places as pairs.  Every thread of the block
+// calls it.
+// Bound by instruction issue: about 140 instructions per pair, 720 with the
+// merge rounds (34 and 152 us for 3.2 M bodies).  Keys too wide for an id used to
+// be sorted as pairs by merging, 302 us a step for 160 graphs of 6.0 M bodies; 300
+// steps of them 456.6 -> 424.6 ms.
 template <int I>
 __device__ void hs_bucket_small(unsigned long long *sk, uint32_t *sv, int n, unsigned long long *dk,
                                 uint32_t *dv, int idbits, unsigned long long *shk, uint32_t *shv,
@@ -623,7 +632,9 @@ __device__ void hs_bucket_small(unsigned long long *sk, uint32_t *sv, int n, uns
         kmin = wmin[w] < kmin ? wmin[w] : kmin;
         kmax = wmax[w] > kmax ? wmax[w] : kmax;
     }
-    if (((kmax - kmin) >> (63 - idbits)) != 0ull) {  // too wide for one word
+    const bool local = ((kmax - kmin) >> (63 - idbits)) != 0ull;  // ids do not fit
+    const int low = local ? kHsCapBits : idbits;
+    if (((kmax - kmin) >> (63 - low)) != 0ull) {  // too wide for one word
         __syncthreads();
         hs_block_sort(sk, sv, n, dk, dv, shk, shv);
         return;
@@ -635,7 +646,7 @@ __device__ void hs_bucket_small(unsigned long long *sk, uint32_t *sv, int n, uns
     for (int j = 0; j < I; ++j) {
         const bool in = j * kHsThreads + t < n;
         rank[j] = in ? atomicAdd(&bins[uint32_t((c[j] - kmin) >> sh)], 1u) : 0u;
-        c[j] = in ? ((c[j] - kmin) << idbits) | id[j] : ~0ull;
+        c[j] = in ? ((c[j] - kmin) << low) | (local ? uint32_t(j * kHsThreads + t) : id[j]) : ~0ull;
     }
     __syncthreads();
     // bins -> starts, eight bins per thread
@@ -652,6 +663,10 @@ __device__ void hs_bucket_small(unsigned long long *sk, uint32_t *sv, int n, uns
     if (lane == 31) wmin[warp] = inc;  // kmin is in registers
     if (__syncthreads_or(most > kHsRankBin)) {
         // words crowded in few bins: sorted by merging
+        if (local) {
+            hs_block_sort(sk, sv, n, dk, dv, shk, shv);
+            return;
+        }
 #pragma unroll
         for (int j = 0; j < I; ++j) {
             const int q = j * kHsThreads + t;
@@ -685,17 +700,24 @@ __device__ void hs_bucket_small(unsigned long long *sk, uint32_t *sv, int n, uns
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < I; ++j)
-        if (j * kHsThreads + t < n) shk[bins[uint32_t((c[j] >> idbits) >> sh)] + rank[j]] = c[j];
+        if (j * kHsThreads + t < n) shk[bins[uint32_t((c[j] >> low) >> sh)] + rank[j]] = c[j];
     __syncthreads();
-    const unsigned long long mask = (1ull << idbits) - 1ull;
+    const unsigned long long mask = (1ull << low) - 1ull;
     for (int q = t; q < n; q += kHsThreads) {
-        const unsigned long long w = shk[q], k = w >> idbits;
+        const unsigned long long w = shk[q], k = w >> low;
         const uint32_t b = uint32_t(k >> sh);
         const int lo = int(bins[b]), hi = b + 1 < uint32_t(kHsBins) ? int(bins[b + 1]) : n;
+        const uint32_t i = local ? __ldcg(&sv[w & mask]) : uint32_t(w & mask);
         int at = lo;
-        for (int z = lo; z < hi; ++z) at += shk[z] < w ? 1 : 0;  // words differ by their ids
+        for (int z = lo; z < hi; ++z) at += shk[z] < w ? 1 : 0;
+        if (local)  // equal keys so far in the order of their places
+            for (int z = lo; z < hi; ++z) {
+                const unsigned long long o = shk[z];
+                if ((o >> low) != k || o == w) continue;
+                at += (__ldcg(&sv[o & mask]) < i ? 1 : 0) - (o < w ? 1 : 0);
+            }
         dk[at] = k + kmin;
-        dv[at] = uint32_t(w & mask);
+        dv[at] = i;
     }
 }
 

@@ -32,7 +32,7 @@
 // active, as a warp waits for its longest search; with the bit rows (about one
 // ballot and one store per level and 32 bodies, then two words per search) 500
 // steps of 1 M bodies fell from 188.7 to 177.5 ms and 300 steps of 160 graphs
-// (5.7 M bodies) from 484.4 to 456.6 ms.  Before that, moments of light bodies in 32 and 64 bits,
+// (6.0 M bodies) from 484.4 to 456.6 ms.  Before that, moments of light bodies in 32 and 64 bits,
 // with the centre's division by an estimate: 190.0 -> 188.7 and 488.5 -> 484.4 ms.
 #pragma once
 
