@@ -184,6 +184,35 @@ __device__ __forceinline__ void xsum_warp(XSum &S, XSum &T) {
     }
 }
 
+// The sum of one value below 2^104 per lane, in every lane: 26 bits per reduction.
+__device__ __forceinline__ u128 warp_sum_u104(u128 v) {
+    u128 sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        sum += u128(__reduce_add_sync(0xFFFFFFFFu, uint32_t(v >> (26 * k)) & 0x3FFFFFFu)) << (26 * k);
+    return sum;
+}
+// The sum of one term per lane, in every lane: at the scale of the largest term
+// they are integers below 2^96, so the whole warp takes six reductions.
+__device__ __forceinline__ XSum xsum_warp_terms(float x) {
+    const uint32_t b = __float_as_uint(x) & 0x7FFFFFFFu;
+    const int e = int(b >> 23);
+    const int bad = int(__reduce_or_sync(0xFFFFFFFFu, e == 255 ? (b & 0x7FFFFFu ? 2u : 1u) : 0u));
+    const uint32_t f = e == 255 ? 0u : e ? ((b & 0x7FFFFFu) | 0x800000u) : b;
+    const int q = (e ? e : 1) - 150;
+    const int top = __reduce_max_sync(0xFFFFFFFFu, f ? q : -1000);
+    if (top == -1000) return XSum{0, kXNoAnchor, bad};
+    const int q0 = top - kXHead, sh = q - q0;
+    return XSum{warp_sum_u104(sh >= 0 ? u128(f) << (f ? sh : 0) : sh > -24 ? u128(f >> -sh) : u128(0)), q0, bad};
+}
+// The merge of two accumulators of at most 2^6 terms per lane, in every lane.
+__device__ __forceinline__ XSum xsum_warp_merge(const XSum &a, const XSum &b) {
+    const int q0 = __reduce_max_sync(0xFFFFFFFFu, a.q0 > b.q0 ? a.q0 : b.q0);
+    const int bad = int(__reduce_or_sync(0xFFFFFFFFu, uint32_t(a.bad | b.bad)));
+    const u128 va = q0 - a.q0 < 128 ? a.V >> (q0 - a.q0) : u128(0), vb = q0 - b.q0 < 128 ? b.V >> (q0 - b.q0) : u128(0);
+    return XSum{warp_sum_u104(va + vb), q0, bad};
+}
+
 // Block-wide merge of one (S, T) pair per thread; thread 0 receives the result.
 template <int kBlock>
 __device__ __forceinline__ void xsum_block(XSum &S, XSum &T) {

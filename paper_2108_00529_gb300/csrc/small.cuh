@@ -25,6 +25,7 @@ namespace {
 constexpr int kSmallMax = 2048;
 constexpr int kSmallThreads = 512;
 constexpr int kSmallHalf = kSmallThreads / 2;
+constexpr int kSmallSums = kSmallHalf / 32;  // warps of nodes
 constexpr int kSmallCluster = 8;         // blocks per cluster, at most
 constexpr int kSmallIdBits = 11;         // ids < kSmallMax
 constexpr int kSmallRank = 32;           // largest bin ranked by counting
@@ -73,17 +74,16 @@ struct SmallMem {
             float4 geo[2 * kSmallMax];
             uint16_t skip[2 * kSmallMax];
         } tree;
+        XPart xpart[kSmallCluster * kSmallSums][2];  // after the walks: S and T of every block's node warps
     } u;
     uint32_t list[kSmallMax];            // cells: first | last << 11 | outer cells from it << 22 | level << 27
     uint32_t D4[kSmallThreads + 1];
     uint16_t S[kSmallMax + 2];           // cells that start before each body
     uint32_t cache[kSmallCache];         // neighbour << 21 | weight
     float2 frep[kSmallHalf];             // repulsion of the block's nodes (written by the walkers of all blocks)
-    XPart xpart[kSmallCluster][2];       // every block's S and T
     unsigned long long red[kSmallThreads / 32][5];
     float4 box[kSmallThreads / 32];
-    unsigned long long kmin[kSmallThreads / 32], kmax[kSmallThreads / 32];
-    uint32_t wsum[kSmallThreads / 32];
+    uint32_t wsum[2][kSmallThreads / 32];  // of the sort, of the cells
     uint32_t cells, greatest;
     double speed;
 };
@@ -99,61 +99,33 @@ __device__ __forceinline__ uint32_t small_scan(uint32_t x, uint32_t *wsum) {
     }
     if (lane == 31) wsum[warp] = inc;
     __syncthreads();
-    uint32_t before = 0u;
-    for (int q = 0; q < warp; ++q) before += wsum[q];
-    __syncthreads();
-    return before + inc - x;
+    return __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wsum[lane] : 0u) + inc - x;
 }
 
 // The words w (four per thread; item r of thread t is body r * kSmallThreads +
 // t) in ascending order into sort.a: binned by their high bits, then ranked
 // inside the bins; a bitonic network when a bin is too full.
-__device__ void small_sort(SmallMem &m, const unsigned long long (&w)[4], int K) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned long long lo = ~0ull, hi = 0ull;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        if (r * kSmallThreads + tid < K) {
-            lo = w[r] < lo ? w[r] : lo;
-            hi = w[r] > hi ? w[r] : hi;
-        }
-        m.u.sort.bins[r * kSmallThreads + tid] = 0u;
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        const unsigned long long a = __shfl_xor_sync(0xFFFFFFFFu, lo, d), b = __shfl_xor_sync(0xFFFFFFFFu, hi, d);
-        lo = a < lo ? a : lo;
-        hi = b > hi ? b : hi;
-    }
-    if (lane == 0) {
-        m.kmin[warp] = lo;
-        m.kmax[warp] = hi;
-    }
-    __syncthreads();
-    for (int q = 0; q < kSmallThreads / 32; ++q) {
-        lo = m.kmin[q] < lo ? m.kmin[q] : lo;
-        hi = m.kmax[q] > hi ? m.kmax[q] : hi;
-    }
-    const int bits = hi > lo ? 64 - __clzll(static_cast<long long>(hi - lo)) : 0;
-    const int sh = bits > kSmallIdBits ? bits - kSmallIdBits : 0;  // kSmallMax bins
+__device__ void small_sort(SmallMem &m, const unsigned long long (&w)[4], int K, int L) {
+    const int tid = threadIdx.x;
+    const int sh = 2 * L;  // kSmallMax bins over the keys, which fill their range (the frame is the bodies' box)
     uint32_t r4[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
-        r4[r] = r * kSmallThreads + tid < K ? atomicAdd(&m.u.sort.bins[uint32_t((w[r] - lo) >> sh)], 1u) : 0u;
+        r4[r] = r * kSmallThreads + tid < K ? atomicAdd(&m.u.sort.bins[uint32_t(w[r] >> sh)], 1u) : 0u;
     __syncthreads();
     uint4 c = reinterpret_cast<uint4 *>(m.u.sort.bins)[tid];
     const uint32_t most = max(max(c.x, c.y), max(c.z, c.w));
-    const uint32_t run = small_scan(c.x + c.y + c.z + c.w, m.wsum);
+    const uint32_t run = small_scan(c.x + c.y + c.z + c.w, m.wsum[0]);
     c = make_uint4(run, run + c.x, run + c.x + c.y, run + c.x + c.y + c.z);
     reinterpret_cast<uint4 *>(m.u.sort.bins)[tid] = c;
     if (!__syncthreads_or(most > kSmallRank)) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-            if (r * kSmallThreads + tid < K) m.u.sort.b[m.u.sort.bins[uint32_t((w[r] - lo) >> sh)] + r4[r]] = w[r];
+            if (r * kSmallThreads + tid < K) m.u.sort.b[m.u.sort.bins[uint32_t(w[r] >> sh)] + r4[r]] = w[r];
         __syncthreads();
         for (int s = tid; s < K; s += kSmallThreads) {
             const unsigned long long x = m.u.sort.b[s];
-            const uint32_t bin = uint32_t((x - lo) >> sh);
+            const uint32_t bin = uint32_t(x >> sh);
             const int b0 = int(m.u.sort.bins[bin]), b1 = bin + 1 < kSmallMax ? int(m.u.sort.bins[bin + 1]) : K;
             int at = b0;
             for (int t = b0; t < b1; ++t) at += m.u.sort.b[t] < x ? 1 : 0;  // words differ by their ids
@@ -205,6 +177,8 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
     uint32_t *levels = m.u.sort.bins;
     float4 box = box_empty();
     for (int i = tid; i < K; i += kSmallThreads) box_add(box, m.pos[i]);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) m.u.sort.bins[r * kSmallThreads + tid] = 0u;
     box_warp(box);
     if (lane == 0) m.box[warp] = box;
     if (tid == 0) m.cells = m.greatest = 0u;
@@ -222,7 +196,7 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
             const unsigned long long key = (spread_bits(U.x >> (32 - L)) << 1) | spread_bits(U.y >> (32 - L));
             w[r] = (key << kSmallIdBits) | unsigned(i);
         }
-        small_sort(m, w, K);
+        small_sort(m, w, K, L);
     }
     // Morton order: bodies and the levels between neighbours
     uint32_t heaviest = 0u, greatest = 0u, ds = 0u;
@@ -301,7 +275,7 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
         }
         const uint4 x = reinterpret_cast<const uint4 *>(levels)[tid];
         const uint32_t c0 = __popc(x.x), c1 = __popc(x.y), c2 = __popc(x.z), c3 = __popc(x.w);
-        const uint32_t run = small_scan(c0 + c1 + c2 + c3, m.wsum);  // its barriers order m.red too
+        const uint32_t run = small_scan(c0 + c1 + c2 + c3, m.wsum[1]);  // its barrier orders m.red too
         m.S[4 * tid] = uint16_t(run);
         m.S[4 * tid + 1] = uint16_t(run + c0);
         m.S[4 * tid + 2] = uint16_t(run + c0 + c1);
@@ -426,6 +400,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
     // Morton order (the other half's)
     const int per = (K + C - 1) / C;
     const int lo = min(rank * per, K), hi = min(lo + per, K);
+    const int warp = tid >> 5;
     const bool walker = tid >= kSmallHalf;
     const int mine = lo + (walker ? tid - kSmallHalf : tid);
     const bool have = mine < hi;
@@ -496,35 +471,33 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
                             : small_rows(m, node, rb, re, A.att_short, p, entry_global);
         }
         cluster.sync();  // the repulsions have arrived
-        XSum S = xsum_zero(), T = xsum_zero();
+        float2 st = make_float2(0.0f, 0.0f);
         if (node) {
             f = force_sum(fa, mass, p, m.frep[mine - lo], A.kg, A.strong);
-            const float2 st = swing_traction(mass, f.x, f.y, fp.x, fp.y);
-            xsum_add(S, st.x);
-            xsum_add(T, st.y);
+            st = swing_traction(mass, f.x, f.y, fp.x, fp.y);
         }
-        xsum_block<kSmallThreads>(S, T);
-        if (tid == 0)
-            for (int q = 0; q < C; ++q) {
-                XPart(*to)[2] = cluster.map_shared_rank(m.xpart, q);
-                to[rank][0] = xsum_pack(S);
-                to[rank][1] = xsum_pack(T);
+        if (!walker) {
+            const XSum S = xsum_warp_terms(st.x), T = xsum_warp_terms(st.y);
+            if (lane < C) {
+                XPart(*to)[2] = cluster.map_shared_rank(m.u.xpart, lane) + rank * kSmallSums + warp;
+                (*to)[0] = xsum_pack(S);
+                (*to)[1] = xsum_pack(T);
             }
+        }
         cluster.sync();  // every block's sums, and nobody reads positions any more
-        if (tid == 0) {
+        if (warp == 0) {
             auto part = [&](int q, int k) {
-                const XPart &x = m.xpart[q][k];
+                if (q >= C * kSmallSums) return xsum_zero();
+                const XPart &x = m.u.xpart[q][k];
                 return XSum{(u128(x.hi) << 64) | x.lo, x.q0, x.bad};
             };
-            S = part(0, 0);
-            T = part(0, 1);
-            for (int q = 1; q < C; ++q) {
-                S = xsum_merge(S, part(q, 0));
-                T = xsum_merge(T, part(q, 1));
-            }
+            const XSum S = xsum_warp_merge(part(lane, 0), part(lane + 32, 0));
+            const XSum T = xsum_warp_merge(part(lane, 1), part(lane + 32, 1));
             Ssum = xsum_value(S);
             Tsum = xsum_value(T);
-            m.speed = speed_update(m.speed, Ssum, Tsum, A.tau);
+            const double sp = speed_update(m.speed, Ssum, Tsum, A.tau);
+            __syncwarp();
+            if (lane == 0) m.speed = sp;
         }
         __syncthreads();
         if (node) {
