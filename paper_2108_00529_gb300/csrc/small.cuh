@@ -2,7 +2,7 @@
 //
 // With few bodies a step of the general path is a chain of a dozen kernels that
 // each last a few microseconds (72 us per step at 219 bodies, 94 at 1,764; here
-// 18.0 and 30).
+// 15.2 and 27).
 // Here one cluster of blocks keeps a graph in shared memory and takes every
 // step of the run in one launch: each block builds the whole quadtree for
 // itself (sorting 2,048 bodies costs less than fetching a tree from elsewhere),
@@ -10,6 +10,12 @@
 // other half sums the attraction of its share of the nodes; repulsions, sums of
 // swing and traction, and new positions go straight into the other blocks'
 // shared memory.  Three cluster barriers per step.
+// Bound by latency: at 1,764 bodies a step was 73,000 cycles, 20,500 of them the
+// search for cells, 14,600 the walk, 9,300 the sort, 9,000 the exact sums and the
+// speed, the rest short phases between barriers.  Cells found by LevelBits: 200
+// steps 7,239 -> 5,996 us (219 bodies: 3,975 -> 3,605); the sort binned by the
+// frame's own bits and sums by warp reductions of integers at one scale: 5,327
+// (3,037).
 // All arithmetic is that of the general path (forces.cuh, tree.cuh), and every
 // sum is taken in the same order or exactly, so the results are the same bits.
 #pragma once
@@ -31,8 +37,7 @@ constexpr int kSmallIdBits = 11;         // ids < kSmallMax
 constexpr int kSmallRank = 32;           // largest bin ranked by counting
 // CSR entries a block keeps (weights below 2^21): what is left of its shared
 // memory.  200 steps at 1,764 bodies took 9,683 us with 8,192, and 7,239 with
-// 10,240, lighter moments and the sums merged by a warp (then 5,996 with the
-// cells found by LevelBits).
+// 10,240, lighter moments and the sums merged by a warp.
 constexpr int kSmallCache = 10240;
 constexpr int64_t kSmallEntries = int64_t(1) << 19;  // CSR entries of a graph, at most
 constexpr int kSmallChunk = 256;         // steps per launch, at most
