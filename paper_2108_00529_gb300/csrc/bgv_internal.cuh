@@ -204,7 +204,7 @@ struct PsControl {
     uint32_t groups, buckets, over, guard, ticket, pad[3];
 };
 struct PairSortScratch {
-    uint32_t *total, *bstart, *bfine, *cursor;
+    uint32_t *total, *bstart, *bfine, *cursor, *run_cursor;
     uint16_t *bmap;
     PsControl *ctl;
     PsBucket *list, *over;

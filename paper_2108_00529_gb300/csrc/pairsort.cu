@@ -12,10 +12,10 @@
 //   2. k_ps_plan     groups neighbouring fine bins into buckets that one block
 //                    sorts in shared memory (at most kPsW keys and rows); a bin
 //                    larger than that is an oversize bucket of its own
-//   3. k_ps_scatter  reads the edges again and writes each key to its bucket: a
-//                    tile of 32,768 keys counts its keys per bucket, reserves
-//                    their places, and writes them, so that all blocks fill the
-//                    same few sectors of a bucket at a time
+//   3. k_ps_coarse   reads the edges again and writes each key to one of 256 runs
+//      k_ps_place    of neighbouring buckets, then from there to its bucket: a
+//                    tile of 8,192 keys orders its keys in shared memory first, so
+//                    that they leave in long pieces
 //   4. k_ps_split    one block per oversize bucket (the hubs of a skewed graph)
 //                    splits it by the next 15 bits of its keys
 //   5. k_ps_sort     one block per bucket: bins per row (and per part of a long
@@ -27,9 +27,10 @@
 // holds more than kPsGiant keys, or too many equal top bits are left, *guard is
 // set and the caller sorts the keys with the LSD sort instead; the decision
 // stays on the device.
-// Supergraph of 34 M R-MAT edges (68 M keys): 4.62 ms with the LSD sort, 3.16 with
+// Supergraph of 34 M R-MAT edges (68 M keys): 4.62 ms with the LSD sort, 2.47 with
 // this (and one pass less over the sorted keys); whole-graph CSR of 8 M edges 1.09
-// and 0.71 ms.
+// and 0.64 ms.  The 68 M keys: histogram 75 us, plan 56, moves 277 and 304, split
+// 185, sort 832 (instruction issue: about 260 thread instructions a key).
 #include "bgv_internal.cuh"
 
 namespace bgv {
@@ -227,11 +228,18 @@ __device__ __forceinline__ void ps_append_equal(PsBucket e, PsControl *ctl, PsBu
     }
 }
 
+constexpr int kCoarse = 256;  // runs of buckets, at most 128 buckets each
+// Groups of one run; run c holds groups [c * per, c * per + per).
+__device__ __forceinline__ uint32_t groups_per_run(uint32_t groups) {
+    return groups > uint32_t(kCoarse) ? (groups + kCoarse - 1) / kCoarse : 1u;
+}
+
 // One block.  ctl and list counters are zero before.
 __global__ void __launch_bounds__(kThreads, 1) k_ps_plan(const uint32_t *__restrict__ total, const int64_t *K_dev,
                                                       PsControl *ctl, uint32_t *__restrict__ bstart,
                                                       uint32_t *__restrict__ bfine, uint16_t *__restrict__ bmap,
-                                                      uint32_t *__restrict__ cursor, PsBucket *list, uint32_t list_cap,
+                                                      uint32_t *__restrict__ cursor, uint32_t *__restrict__ run_cursor,
+                                                      PsBucket *list, uint32_t list_cap,
                                                       PsBucket *over, uint32_t over_cap, unsigned long long *nkeys) {
     const int64_t K = *K_dev;
     const int b = key_bits(K), s1 = fine_shift(b);
@@ -259,6 +267,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_plan(const uint32_t *__restr
         *nkeys = all;
     }
     __syncthreads();
+    if (threadIdx.x < kCoarse) {
+        const uint32_t g = threadIdx.x * groups_per_run(groups);
+        run_cursor[threadIdx.x] = g < groups ? bstart[g] : all;
+    }
     for (uint32_t g = threadIdx.x; g < groups; g += kThreads) {
         const uint32_t f0 = bfine[g], f1 = g + 1 < groups ? bfine[g + 1] : uint32_t(NF);
         const uint32_t k0 = bstart[g], k1 = g + 1 < groups ? bstart[g + 1] : all;
@@ -282,25 +294,78 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_plan(const uint32_t *__restr
     }
 }
 
-// ------------------------------------------------------------ 3. scatter
-// Bound by the writes: a key is 8 bytes of a 32-byte sector, so a bucket's
-// sectors have to be filled while they are still in L2.  (With places reserved
-// once per block and bucket, 152 blocks kept a million sectors partly filled and
-// the kernel took 1,459 us for 68 M keys.)
-__global__ void __launch_bounds__(kThreads, 1) k_ps_scatter(const int32_t *__restrict__ edges, int64_t m, int32_t n,
+// -------------------------------------------------------------- 3. moves
+// A tile of kMoveKeys keys is ordered by destination in shared memory and written
+// in pieces: about 32 keys to a run of buckets, then about a hundred to a bucket.
+// (Written straight to thousands of buckets, a few keys each, the store requests
+// -- one 8-byte piece of a sector at a time -- and the phases that one large
+// block per SM cannot overlap took 1,215 us for 68 M keys; these two take 277 and 304.)
+constexpr int kMoveThreads = 512;
+constexpr int kMoveIn = 16;   // keys per thread
+constexpr int kMoveKeys = kMoveThreads * kMoveIn;
+static_assert(kFine / kCoarse <= kCoarse && kMoveKeys < 65536, "ranks in 16 bits");
+
+struct MoveBins {
+    uint32_t cnt[kCoarse + 32];   // keys per bin, then their first place in the tile; the last 32: no keys
+    uint32_t delta[kCoarse];      // from a place in the tile to the place in the output
+    uint32_t wsum[kMoveThreads / 32];
+    uint32_t total;
+};
+
+// Counts to places, and room in the output for every bin; ends in a barrier.
+__device__ void ps_move_plan(MoveBins &mb, int bins, uint32_t *cursor) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint32_t c = t < bins ? mb.cnt[t] : 0u;
+    const uint32_t room = c ? atomicAdd(&cursor[t], c) : 0u;
+    uint32_t inc = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+        if (lane >= d) inc += y;
+    }
+    if (lane == 31) mb.wsum[warp] = inc;
+    __syncthreads();
+    const uint32_t start = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? mb.wsum[lane] : 0u) + inc - c;
+    if (t < bins) {
+        mb.cnt[t] = start;
+        mb.delta[t] = room - start;
+    }
+    if (t == kMoveThreads - 1) mb.total = start + c;
+    __syncthreads();
+}
+
+// The tile's keys out of `stage`, which holds them by bin; ends in a barrier.
+template <class BinOf>
+__device__ void ps_move_out(const MoveBins &mb, const unsigned long long *stage, BinOf bin_of,
+                            unsigned long long *__restrict__ out, int64_t cap) {
+    const uint32_t total = mb.total;
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < total; i += kMoveThreads) {
+        const unsigned long long key = stage[i];
+        const uint32_t to = mb.delta[bin_of(key)] + i;
+        if (to < cap) out[to] = key;
+    }
+    __syncthreads();
+}
+
+constexpr size_t kCoarseSmem = size_t(kMoveKeys) * sizeof(unsigned long long) + kFine;
+constexpr size_t kPlaceSmem = size_t(kMoveKeys) * sizeof(unsigned long long);
+
+__global__ void __launch_bounds__(kMoveThreads, 2) k_ps_coarse(const int32_t *__restrict__ edges, int64_t m, int32_t n,
                                                             const int64_t *K_dev, const uint32_t *moved,
                                                             const int4 *__restrict__ mapped,
-                                                            const uint16_t *__restrict__ bmap_g, uint32_t *cursor,
+                                                            const uint16_t *__restrict__ bmap, uint32_t *run_cursor,
                                                             const PsControl *ctl,
                                                             unsigned long long *__restrict__ out, int64_t cap) {
     if (ctl->guard) return;
-    extern __shared__ uint32_t cnt[];  // [kFine] keys, then places, per group; then the bins' groups
-    uint16_t *bmap = reinterpret_cast<uint16_t *>(cnt + kFine);
+    extern __shared__ __align__(16) unsigned long long stage[];  // [kMoveKeys], then the fine bins' runs (bytes)
+    __shared__ MoveBins mb;
+    uint8_t *run_of = reinterpret_cast<uint8_t *>(stage + kMoveKeys);
     const int64_t K = *K_dev;
     const int b = key_bits(K), s1 = fine_shift(b);
     const int NF = K > 0 ? int((((static_cast<unsigned long long>(K) << b) - 1) >> s1) + 1) : 1;
-    const uint32_t groups = ctl->groups, padded = (groups + 1023u) & ~1023u;
-    for (int f = threadIdx.x; f < NF; f += kThreads) bmap[swz(f)] = bmap_g[f];
+    const uint32_t per = groups_per_run(ctl->groups);
+    for (int f = threadIdx.x; f < NF; f += kMoveThreads) run_of[f] = uint8_t(bmap[f] / per);
     const bool identity = *moved == 0u;
     const int4 *e2 = identity ? reinterpret_cast<const int4 *>(edges) : mapped;
     const int64_t full = identity ? m >> 1 : (m + 1) >> 1, pairs = (m + 1) >> 1;
@@ -312,51 +377,137 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_scatter(const int32_t *__res
     auto key_of = [&](int32_t a, int32_t c) {
         return (static_cast<unsigned long long>(uint32_t(a)) << b) | uint32_t(c);
     };
-    auto slot_of = [&](unsigned long long key) { return swz(bmap[swz(uint32_t(key >> s1))]); };
-    constexpr int kIn = 8;
-    constexpr int64_t kPairs = int64_t(kThreads) * kIn;  // int4 pairs per tile
-    for (int64_t p0 = int64_t(blockIdx.x) * kPairs; p0 < pairs; p0 += int64_t(gridDim.x) * kPairs) {
-        int4 e[kIn];
+    constexpr int kIn = kMoveIn / 4;  // two edges, four keys
+    int4 e[kIn];
+    auto load = [&](int64_t p0) {
 #pragma unroll
         for (int r = 0; r < kIn; ++r) {
-            const int64_t q = p0 + r * kThreads + threadIdx.x;
+            const int64_t q = p0 + r * kMoveThreads + threadIdx.x;
             e[r] = q < full ? __ldcs(e2 + q) : make_int4(0, 0, 0, 0);
             if (q >= full && q < pairs) e[r] = make_int4(edges[2 * (m - 1)], edges[2 * (m - 1) + 1], 0, 0);
         }
-        for (uint32_t g = threadIdx.x; g < padded; g += kThreads) cnt[g] = 0u;
+    };
+    constexpr int64_t kPairs = kMoveKeys / 4;  // int4 pairs per tile
+    int64_t p0 = int64_t(blockIdx.x) * kPairs;
+    if (p0 < pairs) load(p0);
+    while (p0 < pairs) {
+        if (threadIdx.x < kCoarse) mb.cnt[threadIdx.x] = 0u;
         __syncthreads();
-        auto count = [&](int32_t a, int32_t c) {
-            if (!has_keys(a, c)) return;
-            atomicAdd(&cnt[slot_of(key_of(a, c))], 1u);
-            atomicAdd(&cnt[slot_of(key_of(c, a))], 1u);
+        // every key's run (no keys: one of the last 32 counters) and its rank there
+        uint32_t at[kMoveIn];
+        const uint32_t none = kCoarse + (threadIdx.x & 31);
+#pragma unroll
+        for (int r = 0; r < kIn; ++r) {
+            const bool ok0 = has_keys(e[r].x, e[r].y), ok1 = has_keys(e[r].z, e[r].w);
+            at[4 * r] = ok0 ? run_of[uint32_t(key_of(e[r].x, e[r].y) >> s1)] : none;
+            at[4 * r + 1] = ok0 ? run_of[uint32_t(key_of(e[r].y, e[r].x) >> s1)] : none;
+            at[4 * r + 2] = ok1 ? run_of[uint32_t(key_of(e[r].z, e[r].w) >> s1)] : none;
+            at[4 * r + 3] = ok1 ? run_of[uint32_t(key_of(e[r].w, e[r].z) >> s1)] : none;
+        }
+#pragma unroll
+        for (int k = 0; k < kMoveIn; ++k) at[k] |= atomicAdd(&mb.cnt[at[k]], 1u) << 16;
+        __syncthreads();
+        ps_move_plan(mb, kCoarse, run_cursor);
+        auto put = [&](uint32_t x, int32_t a, int32_t c) {
+            const uint32_t r = x & 0xFFFFu;
+            if (r < kCoarse) stage[mb.cnt[r] + (x >> 16)] = key_of(a, c);
         };
 #pragma unroll
         for (int r = 0; r < kIn; ++r) {
-            count(e[r].x, e[r].y);
-            count(e[r].z, e[r].w);
+            put(at[4 * r], e[r].x, e[r].y);
+            put(at[4 * r + 1], e[r].y, e[r].x);
+            put(at[4 * r + 2], e[r].z, e[r].w);
+            put(at[4 * r + 3], e[r].w, e[r].z);
         }
+        p0 += int64_t(gridDim.x) * kPairs;
+        if (p0 < pairs) load(p0);  // in flight while this tile is written
         __syncthreads();
-        for (uint32_t g = threadIdx.x; g < groups; g += kThreads) {
-            const uint32_t c = cnt[swz(g)];
-            if (c) cnt[swz(g)] = atomicAdd(&cursor[g], c);
+        ps_move_out(mb, stage, [&](unsigned long long key) { return uint32_t(run_of[uint32_t(key >> s1)]); }, out, cap);
+    }
+}
+
+// run_cursor: the ends of the runs, as k_ps_coarse leaves it.
+__global__ void __launch_bounds__(kMoveThreads, 2) k_ps_place(const unsigned long long *__restrict__ in,
+                                                           const int64_t *K_dev, const uint16_t *__restrict__ bmap,
+                                                           const uint32_t *__restrict__ bstart,
+                                                           const uint32_t *__restrict__ run_cursor,
+                                                           const PsControl *ctl, uint32_t *cursor,
+                                                           unsigned long long *__restrict__ out, int64_t cap) {
+    if (ctl->guard) return;
+    extern __shared__ __align__(16) unsigned long long stage[];
+    __shared__ MoveBins mb;
+    __shared__ uint32_t tiles_before[kCoarse + 1], run_start[kCoarse], run_end[kCoarse];
+    const int s1 = fine_shift(key_bits(*K_dev));
+    const uint32_t groups = ctl->groups, per = groups_per_run(groups);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    {  // tiles of every run
+        uint32_t tiles = 0u;
+        if (t < kCoarse && uint32_t(t) * per < groups) {
+            run_start[t] = bstart[t * per];
+            run_end[t] = run_cursor[t];
+            tiles = (run_end[t] - run_start[t] + kMoveKeys - 1) / kMoveKeys;
         }
-        __syncthreads();
-        auto place = [&](unsigned long long key) {
-            const uint32_t pos = atomicAdd(&cnt[slot_of(key)], 1u);
-            if (pos < cap) out[pos] = key;
-        };
+        uint32_t inc = tiles;
 #pragma unroll
-        for (int r = 0; r < kIn; ++r) {
-            if (has_keys(e[r].x, e[r].y)) {
-                place(key_of(e[r].x, e[r].y));
-                place(key_of(e[r].y, e[r].x));
-            }
-            if (has_keys(e[r].z, e[r].w)) {
-                place(key_of(e[r].z, e[r].w));
-                place(key_of(e[r].w, e[r].z));
-            }
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += y;
+        }
+        if (lane == 31) mb.wsum[warp] = inc;
+        __syncthreads();
+        inc += __reduce_add_sync(0xFFFFFFFFu, lane < warp ? mb.wsum[lane] : 0u);
+        if (t < kCoarse) tiles_before[t + 1] = inc;
+        if (t == 0) tiles_before[0] = 0u;
+        __syncthreads();
+    }
+    const uint32_t all = tiles_before[kCoarse];
+    for (uint32_t tile = blockIdx.x; tile < all; tile += gridDim.x) {
+        int c = 0;  // the last run that starts at or before the tile
+#pragma unroll
+        for (int d = kCoarse / 2; d > 0; d >>= 1)
+            if (tiles_before[c + d] <= tile) c += d;
+        const uint32_t k0 = run_start[c] + (tile - tiles_before[c]) * kMoveKeys;
+        const uint32_t count = min(uint32_t(kMoveKeys), run_end[c] - k0);
+        const uint32_t g0 = uint32_t(c) * per;
+        const int bins = int(min(per, groups - g0));
+        if (t < kCoarse) mb.cnt[t] = 0u;
+        unsigned long long k[kMoveIn];
+#pragma unroll
+        for (int r = 0; r < kMoveIn; ++r) {
+            const uint32_t i = r * kMoveThreads + t;
+            k[r] = i < count ? __ldcs(in + k0 + i) : 0ull;
         }
         __syncthreads();
+        uint32_t at[kMoveIn];
+#pragma unroll
+        for (int r = 0; r < kMoveIn; ++r) {
+            const bool ok = uint32_t(r * kMoveThreads + t) < count;
+            at[r] = ok ? uint32_t(__ldg(bmap + uint32_t(k[r] >> s1))) - g0 : uint32_t(kCoarse + lane);
+        }
+#pragma unroll
+        for (int r = 0; r < kMoveIn; ++r) {
+            // a large bucket fills whole tiles: one add for a warp of its keys
+            const uint32_t first = __shfl_sync(0xFFFFFFFFu, at[r], 0);
+            uint32_t rank;
+            if (__all_sync(0xFFFFFFFFu, at[r] == first)) {
+                uint32_t base = 0u;
+                if (lane == 0) base = atomicAdd(&mb.cnt[first], 32u);
+                rank = __shfl_sync(0xFFFFFFFFu, base, 0) + lane;
+            } else {
+                rank = atomicAdd(&mb.cnt[at[r]], 1u);
+            }
+            at[r] |= rank << 16;
+        }
+        __syncthreads();
+        ps_move_plan(mb, bins, cursor + g0);
+#pragma unroll
+        for (int r = 0; r < kMoveIn; ++r) {
+            const uint32_t x = at[r] & 0xFFFFu;
+            if (x < kCoarse) stage[mb.cnt[x] + (at[r] >> 16)] = k[r];
+        }
+        __syncthreads();
+        ps_move_out(mb, stage, [&](unsigned long long key) { return uint32_t(__ldg(bmap + uint32_t(key >> s1))) - g0; }, out,
+                    cap);
     }
 }
 
@@ -675,7 +826,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf
 }
 
 constexpr size_t kHistSmem = size_t(kFine) * sizeof(uint32_t);
-constexpr size_t kScatterSmem = kHistSmem + size_t(kFine) * sizeof(uint16_t);
 // sec and prim (6 bytes a key), bins (2 bytes a key and 4 a primary), pcnt (4 a
 // primary, rounded up to 1,024): keys + primaries <= kPsW, or kPsMaxPrim
 // primaries besides kPsW keys
@@ -690,6 +840,7 @@ void carve_pair_sort(Carver &c, int64_t m, int32_t n, PairSortScratch &s) {
     s.bstart = c.take<uint32_t>(kFine);
     s.bfine = c.take<uint32_t>(kFine);
     s.cursor = c.take<uint32_t>(kFine);
+    s.run_cursor = c.take<uint32_t>(kCoarse);
     s.bmap = c.take<uint16_t>(kFine);
     s.ctl = c.take<PsControl>(1);
     s.over_cap = uint32_t(weight / kPsT + 64);
@@ -704,24 +855,28 @@ int pair_sort(const int32_t *edges, int64_t m, int32_t n, const int32_t *node_ma
               const uint32_t *moved, const PairSortScratch &s, unsigned long long *buf0, unsigned long long *buf1,
               unsigned long long *nkeys, uint32_t *status, cudaStream_t st) {
     const int64_t pairs = (m + 1) / 2;
-    const int sms = sm_count();  // one block per SM
+    const int sms = sm_count();  // one block per SM, two of the moves
     const int64_t cap = 2 * m;
     BGV_CUDA(cudaFuncSetAttribute(k_ps_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kHistSmem)));
     BGV_CUDA(cudaFuncSetAttribute(k_ps_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kHistSmem)));
-    BGV_CUDA(cudaFuncSetAttribute(k_ps_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kScatterSmem)));
+    BGV_CUDA(cudaFuncSetAttribute(k_ps_coarse, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCoarseSmem)));
+    BGV_CUDA(cudaFuncSetAttribute(k_ps_place, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kPlaceSmem)));
     BGV_CUDA(cudaFuncSetAttribute(k_ps_split, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kHistSmem)));
     BGV_CUDA(cudaFuncSetAttribute(k_ps_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSortSmem)));
     BGV_CUDA(cudaMemsetAsync(s.total, 0, sizeof(uint32_t) * kFine, st));
     BGV_CUDA(cudaMemsetAsync(s.ctl, 0, sizeof(PsControl), st));
-    int4 *mapped = reinterpret_cast<int4 *>(buf0);  // the mapped edges, until they are scattered
+    int4 *mapped = reinterpret_cast<int4 *>(buf1);  // the mapped edges, until their keys are in buf0
     note_launch(), k_ps_hist<<<grid_for(pairs, kThreads * 4, sms), kThreads, kHistSmem, st>>>(
         edges, m, n, node_map, K_dev, moved, mapped, s.total, status);
     BGV_TRY(launch_status());
-    note_launch(), k_ps_plan<<<1, kThreads, kHistSmem, st>>>(s.total, K_dev, s.ctl, s.bstart, s.bfine, s.bmap, s.cursor, s.list,
-                                                     s.list_cap, s.over, s.over_cap, nkeys);
+    note_launch(), k_ps_plan<<<1, kThreads, kHistSmem, st>>>(s.total, K_dev, s.ctl, s.bstart, s.bfine, s.bmap, s.cursor,
+                                                     s.run_cursor, s.list, s.list_cap, s.over, s.over_cap, nkeys);
     BGV_TRY(launch_status());
-    note_launch(), k_ps_scatter<<<grid_for(pairs, kThreads * 8, sms), kThreads, kScatterSmem, st>>>(
-        edges, m, n, K_dev, moved, mapped, s.bmap, s.cursor, s.ctl, buf1, cap);
+    note_launch(), k_ps_coarse<<<grid_for(pairs, kMoveKeys / 4, 2 * sms), kMoveThreads, kCoarseSmem, st>>>(
+        edges, m, n, K_dev, moved, mapped, s.bmap, s.run_cursor, s.ctl, buf0, cap);
+    BGV_TRY(launch_status());
+    note_launch(), k_ps_place<<<grid_for(2 * m, kMoveKeys, 2 * sms), kMoveThreads, kPlaceSmem, st>>>(
+        buf0, K_dev, s.bmap, s.bstart, s.run_cursor, s.ctl, s.cursor, buf1, cap);
     BGV_TRY(launch_status());
     note_launch(), k_ps_split<<<grid_for(2 * m, int(kPsW), sms), kThreads, kHistSmem, st>>>(buf1, buf0, K_dev, s.ctl, s.list, s.list_cap,
                                                                    s.over);
