@@ -178,6 +178,10 @@ __global__ void __launch_bounds__(kThreads) k_cut_pairs(const int32_t *__restric
 // the totals and the offsets of the rows after the last pair.  (Run starts and
 // superedge indices written here and turned into weights by a second pass cost
 // 16 more bytes per entry: 709 us for both passes at 68 M entries.)
+// Half of the warps wait for the look-back at any time (11.9 of 24 stall cycles per
+// instruction at the block's barriers), so as many blocks as fit: 8 per SM, 32
+// registers, for 6 at 40 (supergraph of 34 M edges 2,472 -> 2,461 us; a look-back
+// by all warps of the block: no faster).
 constexpr int kRedItems = 8;
 constexpr int kRedTile = kThreads * kRedItems;
 enum : uint32_t { kRedAgg = 1u, kRedIncl = 2u };
@@ -215,7 +219,7 @@ __device__ __forceinline__ unsigned long long block_exclusive_u64(unsigned long 
 
 constexpr int kRedGapList = 64;  // long runs of empty rows a tile fills with all its threads
 
-__global__ void __launch_bounds__(kThreads) k_csr_reduce(const unsigned long long *__restrict__ keys,
+__global__ void __launch_bounds__(kThreads, 8) k_csr_reduce(const unsigned long long *__restrict__ keys,
                                                          const unsigned long long *nkeys_dev, int64_t cap,
                                                          const int64_t *K_dev, int32_t *__restrict__ csr_off,
                                                          int32_t *__restrict__ csr_adj, uint32_t *__restrict__ csr_w,
