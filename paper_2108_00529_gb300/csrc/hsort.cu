@@ -18,7 +18,7 @@ struct HsWs {
 
 void carve_hs_ws(Carver &c, int64_t K, HsWs &w) {
     const size_t k = size_t(K > 0 ? K : 1);
-    carve_hs(c, K, true, w.h);
+    carve_hs(c, hs_buckets(K), true, w.h);
     w.tmp_key = c.take<unsigned long long>(k);
     w.tmp_bucket = c.take<uint32_t>(k);
     w.slot_key = c.take<unsigned long long>(k);
@@ -67,7 +67,7 @@ int bgv_sort_hinted(const uint64_t *keys, const uint32_t *hint, int64_t K, uint6
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     uint32_t *status = status_ptr(ws);
     const KeyArray key_of{reinterpret_cast<const unsigned long long *>(keys)};
-    BGV_TRY(hinted_sort_sampled(key_of, hint, K, w.h, w.tmp_key, w.tmp_bucket, w.slot_key, w.slot_id,
+    BGV_TRY(hinted_sort_sampled(key_of, hint, K, hs_buckets(K), w.h, w.tmp_key, w.tmp_bucket, w.slot_key, w.slot_id,
                                 reinterpret_cast<unsigned long long *>(out_keys), out_ids, status, st));
     uint32_t dev_status = 0;
     BGV_CUDA(cudaMemcpyAsync(&dev_status, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));

@@ -13,8 +13,9 @@
 //   1. Splitters.  ForceAtlas2 still holds the previous iteration's sorted
 //      (key, id) pairs: every kHsBucket-th of them is a splitter (HsPrevious), in
 //      order already, with about as many new pairs between two as old ones.
-//      The public entry point has no earlier keys: it takes the ids at ns evenly
-//      spaced places of the hint and their keys, ranks them among themselves by
+//      The public entry point has no earlier keys, and a first or single step of
+//      up to kHsFirstMax bodies not even a hint (it takes id order for one): they
+//      take the ids at ns evenly spaced places of the hint and their keys, rank them among themselves by
 //      counting (equal pairs by sample index), and every s-th is a splitter
 //      (HsSampled).  Bucket u holds the pairs x with splitter(u) <= x <
 //      splitter(u+1), splitter(0) = -inf, splitter(nb) = +inf.
@@ -72,11 +73,17 @@ struct HsBuffers {
 };
 
 inline int hs_buckets(int64_t K) { return K > kHsBucket ? int((K + kHsBucket - 1) / kHsBucket) : 1; }
-// Words from `count` on that are zero before a sort (and after it).
-inline int64_t hs_counter_words(int64_t K) { return 2 * int64_t(hs_buckets(K)) + 2; }
+// Without a hint (bodies in id order) only the samples tell where the keys lie,
+// and a bucket between sampled splitters may hold twice its share: half the
+// share keeps it in shared memory.  For as many pairs as the samples serve with
+// kHsMaxPerBucket a bucket.
+constexpr int kHsFirstBucket = kHsBucket / 2;
+constexpr int64_t kHsFirstMax = int64_t(kHsMaxSamples) / kHsMaxPerBucket * kHsFirstBucket;  // 262,144
+inline int hs_first_buckets(int64_t K) { return K > kHsFirstBucket ? int((K + kHsFirstBucket - 1) / kHsFirstBucket) : 1; }
+// Words from `count` on that are zero before a sort into nb buckets (and after it).
+inline int64_t hs_counter_words(int nb) { return 2 * int64_t(nb) + 2; }
 
-inline void carve_hs(Carver &c, int64_t K, bool sampled, HsBuffers &h) {
-    const size_t nb = size_t(hs_buckets(K));
+inline void carve_hs(Carver &c, int nb, bool sampled, HsBuffers &h) {
     h = HsBuffers{};
     if (sampled) {
         h.smp_key = c.take<unsigned long long>(kHsMaxSamples);
@@ -85,10 +92,14 @@ inline void carve_hs(Carver &c, int64_t K, bool sampled, HsBuffers &h) {
         h.spl_key = c.take<unsigned long long>(kHsMaxBuckets);
         h.spl_id = c.take<uint32_t>(kHsMaxBuckets);
     }
-    h.count = c.take<uint32_t>(size_t(hs_counter_words(K)));
-    h.cursor = h.count ? h.count + nb : nullptr;
-    h.ticket = h.count ? h.count + 2 * nb : nullptr;
-    h.start = c.take<uint32_t>(nb + 1);
+    h.count = c.take<uint32_t>(size_t(hs_counter_words(nb)));
+    h.start = c.take<uint32_t>(size_t(nb) + 1);
+}
+// The same buffers for a sort into nb buckets (no more than they were carved for).
+inline HsBuffers hs_for(HsBuffers h, int nb) {
+    h.cursor = h.count + nb;
+    h.ticket = h.count + 2 * size_t(nb);
+    return h;
 }
 
 // Splitter u + 1 (the least pair of bucket u + 1).
@@ -105,19 +116,24 @@ struct HsPrevious {  // the sorted pairs of the previous iteration
     __device__ uint32_t id_at(int u) const { return __ldg(&id[int64_t(u + 1) * kHsBucket]); }
 };
 
-// Buckets and samples per bucket for K pairs (nb = 1: no splitters).
+// Samples per bucket for K pairs in nb buckets (ns = 0: no splitters).
 struct HsShape {
-    int nb, s, ns;
+    int s, ns;
 };
-inline HsShape hs_shape(int64_t K) {
+inline HsShape hs_shape(int64_t K, int nb) {
     HsShape h;
-    h.nb = hs_buckets(K);
-    h.s = kHsMaxSamples / h.nb;
+    h.s = kHsMaxSamples / nb;
     if (h.s > kHsMaxPerBucket) h.s = kHsMaxPerBucket;
     if (h.s < 1) h.s = 1;
-    h.ns = h.nb > 1 ? h.nb * h.s : 0;  // nb > 1 means K > 1024 >= 8 nb, so ns < K
+    h.ns = nb > 1 ? nb * h.s : 0;  // nb > 1 means K > 512 (nb - 1) >= 8 nb, so ns < K
     return h;
 }
+
+// Extra words the first kernel clears (for the kernels after the sort).
+struct HsClears {
+    uint32_t *u32 = nullptr;
+    int64_t n_u32 = 0;
+};
 
 // The kernels are private to each translation unit that includes this
 // header (each instantiates its own key source).
@@ -129,7 +145,7 @@ __device__ __forceinline__ bool hs_less(unsigned long long ak, uint32_t ai, unsi
 
 __device__ __forceinline__ uint32_t hs_id(const uint32_t *__restrict__ hint, int64_t p, int64_t K,
                                           uint32_t *status) {
-    uint32_t id = hint[p];
+    uint32_t id = hint ? hint[p] : uint32_t(p);  // no hint: id order
     if (id >= uint64_t(K)) {
         raise_status(status, BGV_DEV_BADHINT);
         id = 0u;
@@ -140,7 +156,8 @@ __device__ __forceinline__ uint32_t hs_id(const uint32_t *__restrict__ hint, int
 // 1a. Sample keys; clears the counters of the later kernels.
 template <class KeyOf>
 __global__ void __launch_bounds__(256) k_hs_sample(KeyOf key_of, const uint32_t *__restrict__ hint, int64_t K,
-                                                   int64_t counter_words, int ns, HsBuffers h, uint32_t *status) {
+                                                   int64_t counter_words, int ns, HsBuffers h, HsClears clr,
+                                                   uint32_t *status) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     const int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     for (int64_t t = t0; t < ns; t += stride) {
@@ -151,6 +168,7 @@ __global__ void __launch_bounds__(256) k_hs_sample(KeyOf key_of, const uint32_t 
         h.smp_rank[t] = 0u;
     }
     for (int64_t t = t0; t < counter_words; t += stride) h.count[t] = 0u;
+    for (int64_t t = t0; t < clr.n_u32; t += stride) clr.u32[t] = 0u;
 }
 
 // 1b. Ranks of the samples by counting, one slice of the others per block
@@ -342,7 +360,7 @@ __global__ void __launch_bounds__(256) k_hs_scatter(const uint32_t *__restrict__
         if (p < K) {
             u = int(tmp_bucket[p]);
             k = tmp_key[p];
-            id = hint[p];
+            id = hint ? hint[p] : uint32_t(p);
             if (id >= uint64_t(K)) id = 0u;  // reported by the count kernel
         }
         const unsigned peers = __match_any_sync(0xFFFFFFFFu, u);
@@ -751,16 +769,17 @@ __global__ void __launch_bounds__(kHsThreads) k_hs_bucket(HsBuffers h, unsigned 
 
 }  // namespace
 
-// The sort on stream `st`; key_of(id) gives the key of id.  tmp_key/tmp_bucket
-// and slot_key/slot_id hold K entries each and may not alias the hint, the
-// splitters or the output.  The counters of `h` are zero before it, and after.
+// The sort into nb buckets on stream `st`; key_of(id) gives the key of id, a null
+// hint is id order.  tmp_key/tmp_bucket and slot_key/slot_id hold K entries each
+// and may not alias the hint, the splitters or the output.  The counters of `h`
+// are zero before it, and after.
 template <class KeyOf, class Split>
-int hinted_sort_place(KeyOf key_of, Split split, const uint32_t *hint, int64_t K, const HsBuffers &h,
+int hinted_sort_place(KeyOf key_of, Split split, const uint32_t *hint, int64_t K, int nb, const HsBuffers &buffers,
                       unsigned long long *tmp_key, uint32_t *tmp_bucket, unsigned long long *slot_key,
                       uint32_t *slot_id, unsigned long long *out_key, uint32_t *out_id, uint32_t *status,
                       cudaStream_t st) {
     if (K <= 0) return BGV_OK;
-    const int nb = hs_buckets(K);
+    const HsBuffers h = hs_for(buffers, nb);
     note_launch(), k_hs_count<KeyOf, Split><<<grid_for(K, 256, sm_count() * 8), 256, 0, st>>>(
         key_of, split, hint, K, nb, h, tmp_key, tmp_bucket, status);
     BGV_TRY(launch_status());
@@ -773,26 +792,31 @@ int hinted_sort_place(KeyOf key_of, Split split, const uint32_t *hint, int64_t K
     return launch_status();
 }
 
-// The same with splitters from samples of the hint, K <= hs_max_keys(); the
-// output may not alias the hint.
+// The same with splitters from samples of the hint, nb <= kHsMaxBuckets; clears
+// the counters first.
 template <class KeyOf>
-int hinted_sort_sampled(KeyOf key_of, const uint32_t *hint, int64_t K, const HsBuffers &h, unsigned long long *tmp_key,
-                        uint32_t *tmp_bucket, unsigned long long *slot_key, uint32_t *slot_id,
-                        unsigned long long *out_key, uint32_t *out_id, uint32_t *status, cudaStream_t st) {
+int hinted_sort_sampled(KeyOf key_of, const uint32_t *hint, int64_t K, int nb, const HsBuffers &buffers,
+                        unsigned long long *tmp_key, uint32_t *tmp_bucket, unsigned long long *slot_key,
+                        uint32_t *slot_id, unsigned long long *out_key, uint32_t *out_id, uint32_t *status,
+                        cudaStream_t st, const HsClears &clr = HsClears()) {
     if (K <= 0) return BGV_OK;
-    if (K > hs_max_keys()) return BGV_EINVAL;
-    const HsShape sh = hs_shape(K);
-    const int64_t words = hs_counter_words(K);
-    note_launch(), k_hs_sample<KeyOf><<<grid_for(words > sh.ns ? words : sh.ns, 256, sm_count() * 4), 256, 0, st>>>(
-        key_of, hint, K, words, sh.ns, h, status);
+    if (nb > kHsMaxBuckets) return BGV_EINVAL;
+    const HsBuffers h = hs_for(buffers, nb);
+    const HsShape sh = hs_shape(K, nb);
+    const int64_t words = hs_counter_words(nb);
+    int64_t work = sh.ns;
+    for (const int64_t w : {words, clr.n_u32})
+        if (w > work) work = w;
+    note_launch(), k_hs_sample<KeyOf><<<grid_for(work, 256, sm_count() * 4), 256, 0, st>>>(key_of, hint, K, words,
+                                                                                          sh.ns, h, clr, status);
     BGV_TRY(launch_status());
     if (sh.ns > 0) {
         const dim3 g((sh.ns + 255) / 256, kHsRankSlices);
         note_launch(), k_hs_rank<<<g, 256, 0, st>>>(sh.ns, sh.s, h);
         BGV_TRY(launch_status());
     }
-    return hinted_sort_place(key_of, HsSampled{h.spl_key, h.spl_id}, hint, K, h, tmp_key, tmp_bucket, slot_key, slot_id,
-                             out_key, out_id, status, st);
+    return hinted_sort_place(key_of, HsSampled{h.spl_key, h.spl_id}, hint, K, nb, h, tmp_key, tmp_bucket, slot_key,
+                             slot_id, out_key, out_id, status, st);
 }
 
 }  // namespace bgv
