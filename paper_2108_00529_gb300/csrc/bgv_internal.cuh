@@ -78,6 +78,28 @@ inline int launch_status() { return cudaGetLastError() == cudaSuccess ? BGV_OK :
 // Process-wide count of kernel launches issued by the library (every launch
 // site calls note_launch; graph replays are added by the replay loop).
 void note_launch();
+// A kernel that follows another one of its chain: its blocks may take their place
+// on the SMs while the last blocks of the one before still run, and wait there
+// (chain_wait, first thing in both kernels) until it has finished and its writes
+// are seen.  Saves the launch and most of the drain between two kernels.
+template <class... P, class... A>
+int launch_chained(bool early, void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    note_launch();
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? launch_status() : BGV_ECUDA;
+}
+__device__ __forceinline__ void chain_wait() {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
 void add_launches(unsigned long long n);
 unsigned long long launches_issued();
 

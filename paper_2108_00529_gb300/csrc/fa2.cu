@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kRT) k_repulse(const float4 *__restrict__ geo,
                                                       float theta2, float2 *__restrict__ Frep,
                                                       unsigned long long *inter_step,
                                                       unsigned long long *inter_total) {
+    chain_wait();
     const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     unsigned inter = 0;
     if (s < K) {
@@ -1019,33 +1020,21 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
     BGV_TRY(mark(2));
     if (K >= 2) {
         const unsigned tiles = unsigned(tile_count(K));
-        note_launch(), k_tile<<<tiles, kTileThreads, 0, st>>>(s.sort.keys[res], s.sort.vals[res], K, pos, mass, s.frame,
-                                                              s.bgraph, L, gbits, p.leaf_cap, s.body, s.tree,
-                                                              &hdr->status, spin_limit());
-        BGV_TRY(launch_status());
+        BGV_TRY(launch_chained(hs_early(K), k_tile, tiles, kTileThreads, st, s.sort.keys[res], s.sort.vals[res], K, pos, mass, s.frame,
+                               s.bgraph, L, gbits, p.leaf_cap, s.body, s.tree, &hdr->status, spin_limit()));
         BGV_TRY(mark(3));
         const unsigned per = kTileThreads / 32;  // tiles per block
-        note_launch(), k_tile_cross<<<(tiles + per - 1) / per, kTileThreads, 0, st>>>(K, L, p.leaf_cap, s.frame,
-                                                                                    s.bgraph, s.tree, &hdr->tree_nodes);
-        BGV_TRY(launch_status());
+        BGV_TRY(launch_chained(hs_early(K), k_tile_cross, (tiles + per - 1) / per, kTileThreads, st, K, L, p.leaf_cap, s.frame,
+                               s.bgraph, s.tree, &hdr->tree_nodes));
         BGV_TRY(mark(4));
-        note_launch(), k_tile_emit<<<tiles, kTileThreads, 0, st>>>(K, s.body, s.tree, s.T, s.geo, s.skip,
-                                                                   &hdr->interactions);
-        BGV_TRY(launch_status());
+        BGV_TRY(launch_chained(hs_early(K), k_tile_emit, tiles, kTileThreads, st, K, s.body, s.tree, s.T, s.geo, s.skip,
+                               &hdr->interactions));
         BGV_TRY(mark(5));
         const float theta2 = p.theta * p.theta;
-        if (tune.repulse_threads == 128) {
-            const unsigned gr = unsigned((K + 127) / 128);
-            note_launch(), k_repulse<128><<<gr, 128, 0, st>>>(s.geo, s.skip, s.T, koff, s.bgraph, s.body, K, p.kr,
-                                                              theta2, s.Frep, &hdr->interactions,
-                                                              &hdr->interactions_total);
-        } else {
-            const unsigned gr = unsigned((K + kThreads - 1) / kThreads);
-            note_launch(), k_repulse<kThreads><<<gr, kThreads, 0, st>>>(s.geo, s.skip, s.T, koff, s.bgraph, s.body, K,
-                                                                        p.kr, theta2, s.Frep, &hdr->interactions,
-                                                                        &hdr->interactions_total);
-        }
-        BGV_TRY(launch_status());
+        const unsigned rt = tune.repulse_threads == 128 ? 128u : unsigned(kThreads);
+        BGV_TRY(launch_chained(hs_early(K), rt == 128 ? k_repulse<128> : k_repulse<kThreads>, unsigned((K + rt - 1) / rt), rt, st, s.geo,
+                               s.skip, s.T, koff, s.bgraph, s.body, K, p.kr, theta2, s.Frep, &hdr->interactions,
+                               &hdr->interactions_total));
     } else {
         BGV_CUDA(cudaMemsetAsync(s.Frep, 0, sizeof(float2), st));
         BGV_TRY(mark(3));

@@ -324,6 +324,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
     const float2 *__restrict__ pos, const uint32_t *__restrict__ mass, const float4 *__restrict__ frames,
     const int32_t *__restrict__ bgraph, int L, int gbits, int leaf_cap, float4 *__restrict__ body, TileArrays T,
     uint32_t *dev_status, int spin_limit) {
+    chain_wait();
     __shared__ __align__(16) uint32_t sm[kTile], sux[kTile], suy[kTile];  // masses, fixed-point coordinates
     __shared__ union {
         LevelBits<kTile / 32> bits;
@@ -661,6 +662,7 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_cross(int64_t K, int L, i
                                                              const float4 *__restrict__ frames,
                                                              const int32_t *__restrict__ bgraph, TileArrays T,
                                                              unsigned long long *tree_nodes) {
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int64_t tiles = (K + kTile - 1) / kTile;
     const int64_t tile = (int64_t(blockIdx.x) * kTileThreads + threadIdx.x) >> 5;
@@ -763,6 +765,7 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_emit(int64_t K, const flo
                                                             uint32_t *__restrict__ S, float4 *__restrict__ geo,
                                                             int32_t *__restrict__ skip,
                                                             unsigned long long *interactions) {
+    chain_wait();
     __shared__ uint32_t nst4[kTile / 4], loc4[kTile / 4];  // cells that start at each body: all, inside the tile
     __shared__ uint32_t pre[kTile + 1];  // cells starting before each body, in this tile
     __shared__ uint32_t wsum[kTileThreads / 32];
