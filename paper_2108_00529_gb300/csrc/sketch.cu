@@ -19,7 +19,7 @@
 //                  out of shared memory)
 //   k_deg_count    lists counted with shared-memory atomics, one range's
 //                  counters per block, and added to the degrees
-// Degree sketch of 34 M edges on 3.2 M nodes: 608 us before, 437 with the ranges.
+// Degree sketch of 34 M edges on 3.2 M nodes: 608 us before, 431 with the ranges.
 #include <mutex>
 
 #include "bgv_internal.cuh"
@@ -103,7 +103,8 @@ constexpr int kRange = 1 << kRangeBits;
 constexpr int kMaxRanges = 512;                    // n <= 16,777,216
 constexpr int64_t kDegSplitMin = int64_t(1) << 19; // edges; below, one kernel is shorter than three
 constexpr int kDegIn = 4;                          // int4 loads per thread and tile
-constexpr int kDegTile = kDegThreads * kDegIn * 4; // endpoints per tile
+constexpr int kPlaceThreads = 512;  // of k_deg_place, two blocks per SM: their phases overlap (437 us with one of 1,024)
+constexpr int kDegTile = kPlaceThreads * kDegIn * 4; // endpoints per tile
 constexpr uint32_t kDegPiece = 1u << 18;           // endpoints a block counts at a time
 
 inline int deg_ranges(int32_t n) { return (n + kRange - 1) / kRange; }
@@ -175,20 +176,20 @@ __device__ __forceinline__ void scan_ranges(uint32_t v, uint32_t *out) {
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kDegThreads, 1) k_deg_place(const int32_t *__restrict__ edges, int64_t m, int32_t n,
+__global__ void __launch_bounds__(kPlaceThreads, 2) k_deg_place(const int32_t *__restrict__ edges, int64_t m, int32_t n,
                                                               int ranges, const uint32_t *__restrict__ count,
                                                               uint32_t *cursor, uint16_t *__restrict__ local) {
     __shared__ uint16_t stage[kDegTile];
     __shared__ uint32_t cnt[kMaxRanges], lstart[kMaxRanges + 1], start[kMaxRanges + 1], gbase[kMaxRanges];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     scan_ranges(t < ranges ? count[t] : 0u, start);
-    const int64_t pairs = (m + 1) >> 1, tile_pairs = kDegThreads * kDegIn;
+    const int64_t pairs = (m + 1) >> 1, tile_pairs = kPlaceThreads * kDegIn;
     for (int64_t p0 = int64_t(blockIdx.x) * tile_pairs; p0 < pairs; p0 += int64_t(gridDim.x) * tile_pairs) {
         if (t < kMaxRanges) cnt[t] = 0u;
         int4 e[kDegIn];
         int have[kDegIn];
 #pragma unroll
-        for (int r = 0; r < kDegIn; ++r) e[r] = load_pair(edges, m, p0 + r * kDegThreads + t, &have[r]);
+        for (int r = 0; r < kDegIn; ++r) e[r] = load_pair(edges, m, p0 + r * kPlaceThreads + t, &have[r]);
         __syncthreads();
         uint32_t rank[kDegIn * 4];
 #pragma unroll
@@ -211,7 +212,7 @@ __global__ void __launch_bounds__(kDegThreads, 1) k_deg_place(const int32_t *__r
                     stage[lstart[x >> kRangeBits] + rank[4 * r + j]] = uint16_t(x & (kRange - 1));
             }
         __syncthreads();
-        for (int b = warp; b < ranges; b += kDegThreads / 32) {  // a warp per run
+        for (int b = warp; b < ranges; b += kPlaceThreads / 32) {  // a warp per run
             const uint32_t s = lstart[b], k = lstart[b + 1] - s;
             uint16_t *dst = local + (k ? gbase[b] : 0u);
             for (uint32_t i = lane; i < k; i += 32) dst[i] = stage[s + i];
@@ -336,7 +337,7 @@ int run_sketch(const int32_t *edges, int64_t m, int32_t n, const HashFamily &h, 
         note_launch(), k_deg_ranges<<<grid_for(pairs, kDegThreads * kDegIn, sm_count() * 2), kDegThreads, hist, st>>>(
             edges, m, n, R, count, status);
         BGV_TRY(launch_status());
-        note_launch(), k_deg_place<<<grid_for(pairs, kDegThreads * kDegIn, sm_count() * 2), kDegThreads, 0, st>>>(
+        note_launch(), k_deg_place<<<grid_for(pairs, kPlaceThreads * kDegIn, sm_count() * 2), kPlaceThreads, 0, st>>>(
             edges, m, n, R, count, cursor, s.local);
         BGV_TRY(launch_status());
         note_launch(), k_deg_count<<<grid_for(2 * m / kDegPiece + R, 1, sm_count()), kDegThreads, counters, st>>>(
