@@ -27,9 +27,9 @@
 // holds more than kPsGiant keys, or too many equal top bits are left, *guard is
 // set and the caller sorts the keys with the LSD sort instead; the decision
 // stays on the device.
-// Supergraph of 34 M R-MAT edges (68 M keys): 4.62 ms with the LSD sort, 2.47 with
+// Supergraph of 34 M R-MAT edges (68 M keys): 4.62 ms with the LSD sort, 2.44 with
 // this (and one pass less over the sorted keys); whole-graph CSR of 8 M edges 1.09
-// and 0.64 ms.  The 68 M keys: histogram 75 us, plan 56, moves 277 and 304, split
+// and 0.62 ms.  The 68 M keys: histogram 75 us, plan 36, moves 277 and 304, split
 // 185, sort 832 (instruction issue: about 260 thread instructions a key).
 #include "bgv_internal.cuh"
 
@@ -234,7 +234,9 @@ __device__ __forceinline__ uint32_t groups_per_run(uint32_t groups) {
     return groups > uint32_t(kCoarse) ? (groups + kCoarse - 1) / kCoarse : 1u;
 }
 
-// One block.  ctl and list counters are zero before.
+// One block.  ctl and list counters are zero before.  Bound by the latency of its
+// passes (the bins' groups go out through shared memory: written by the threads
+// that walk the bins, 32 apart, they took 20 us more).
 __global__ void __launch_bounds__(kThreads, 1) k_ps_plan(const uint32_t *__restrict__ total, const int64_t *K_dev,
                                                       PsControl *ctl, uint32_t *__restrict__ bstart,
                                                       uint32_t *__restrict__ bfine, uint16_t *__restrict__ bmap,
@@ -256,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_plan(const uint32_t *__restr
     ps_scan<uint32_t>(mine, &all);
     const uint32_t groups = ps_groups(
         NF, rows_per_bin, 0u, [&](int f) { return c_sh[swz(f)]; },
-        [&](int f, uint32_t, uint32_t g) { bmap[f] = uint16_t(g); },
+        [&](int f, uint32_t, uint32_t g) { c_sh[swz(f)] = g; },  // its count has been read for the last time
         [&](uint32_t g, int f, uint32_t k) {
             bstart[g] = k;
             bfine[g] = uint32_t(f);
@@ -267,6 +269,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_plan(const uint32_t *__restr
         *nkeys = all;
     }
     __syncthreads();
+    for (int f = threadIdx.x; f < NF; f += kThreads) bmap[f] = uint16_t(c_sh[swz(f)]);
     if (threadIdx.x < kCoarse) {
         const uint32_t g = threadIdx.x * groups_per_run(groups);
         run_cursor[threadIdx.x] = g < groups ? bstart[g] : all;
