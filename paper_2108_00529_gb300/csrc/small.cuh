@@ -2,7 +2,7 @@
 //
 // With few bodies a step of the general path is a chain of a dozen kernels that
 // each last a few microseconds (72 us per step at 219 bodies, 94 at 1,764; here
-// 15.2 and 27).
+// 15.1 and 26).
 // Here one cluster of blocks keeps a graph in shared memory and takes every
 // step of the run in one launch: each block builds the whole quadtree for
 // itself (sorting 2,048 bodies costs less than fetching a tree from elsewhere),
@@ -15,7 +15,9 @@
 // speed, the rest short phases between barriers.  Cells found by LevelBits: 200
 // steps 7,239 -> 5,996 us (219 bodies: 3,975 -> 3,605); the sort binned by the
 // frame's own bits and sums by warp reductions of integers at one scale: 5,327
-// (3,037).
+// (3,037); the bits' summary words set by 32-bit atomics, as 64-bit ones loop:
+// 5,184 (3,020).  A step at 1,764 bodies is then about 52,000 cycles, the walk
+// 14,400, cells 7,900, sort 6,000, no other phase more than 4,000.
 // All arithmetic is that of the general path (forces.cuh, tree.cuh), and every
 // sum is taken in the same order or exactly, so the results are the same bits.
 #pragma once
@@ -239,7 +241,8 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
             if (r * kSmallThreads + warp * 32 <= K)  // words past the end are not asked for
-                m.w.bits.add((ds >> (8 * r)) & 255u, r * (kSmallThreads / 32) + warp, 0u, hi, m.some);
+                m.w.bits.add((ds >> (8 * r)) & 255u, r * (kSmallThreads / 32) + warp, 0u, hi,
+                             reinterpret_cast<uint32_t *>(m.some));
     }
     __syncthreads();
 #pragma unroll

@@ -280,7 +280,7 @@ struct LevelBits {
     using Some = typename std::conditional<kWords == 32, uint32_t, unsigned long long>::type;
     uint32_t row[32][kWords + 1];
     // Every thread of a warp, with the value of its place of word w; lo <= hi, at most 32 levels.
-    __device__ __forceinline__ void add(uint32_t d, int w, uint32_t lo, uint32_t hi, Some *some) {
+    __device__ __forceinline__ void add(uint32_t d, int w, uint32_t lo, uint32_t hi, uint32_t *some) {
         const uint32_t lane = threadIdx.x & 31;
         uint32_t keep = 0u;
         for (uint32_t v = lo; v <= hi; ++v) {
@@ -288,7 +288,7 @@ struct LevelBits {
             if (lane == v - lo) keep = x;
         }
         if (lane <= hi - lo) row[lane][w] = keep;
-        if (keep) atomicOr(&some[lane], Some(1) << w);
+        if (keep) atomicOr(&some[lane * (kWords / 32) + (w >> 5)], 1u << (w & 31));  // 32 bits: a native operation
     }
     // Last place <= from in row r; -1 if there is none.
     __device__ __forceinline__ int last(int r, Some some, int from) const {
