@@ -223,7 +223,8 @@ struct PsBucket {
     uint32_t flags, pad;
 };
 struct PsControl {
-    uint32_t groups, buckets, over, guard, ticket, pad[3];
+    // buckets: listed, the first `planned` of them before any split
+    uint32_t groups, buckets, over, guard, ticket, planned, split_ticket, pad;
 };
 struct PairSortScratch {
     uint32_t *total, *bstart, *bfine, *cursor, *run_cursor;

@@ -16,9 +16,10 @@
 //      k_ps_place    of neighbouring buckets, then from there to its bucket: a
 //                    tile of 8,192 keys orders its keys in shared memory first, so
 //                    that they leave in long pieces
-//   4. k_ps_split    one block per oversize bucket (the hubs of a skewed graph)
-//                    splits it by the next 15 bits of its keys
-//   5. k_ps_sort     one block per bucket: bins per row (and per part of a long
+//   4. k_ps_sort     one block per oversize bucket (the hubs of a skewed graph)
+//                    splits it by the next 15 bits of its keys (ps_split), beside
+//                    the other buckets; the pieces take a second launch
+//                    One block per bucket sorts it: bins per row (and per part of a long
 //                    row) by shared-memory atomics, then every key's rank inside
 //                    its bin, which holds a few keys; bins that hold many keys
 //                    go through a bitonic network
@@ -27,7 +28,7 @@
 // holds more than kPsGiant keys, or too many equal top bits are left, *guard is
 // set and the caller sorts the keys with the LSD sort instead; the decision
 // stays on the device.
-// Supergraph of 34 M R-MAT edges (68 M keys): 4.62 ms with the LSD sort, 2.44 with
+// Supergraph of 34 M R-MAT edges (68 M keys): 4.62 ms with the LSD sort, 2.36 with
 // this (and one pass less over the sorted keys); whole-graph CSR of 8 M edges 1.09
 // and 0.62 ms.  The 68 M keys: histogram 75 us, plan 36, moves 277 and 304, split
 // 185, sort 832 (instruction issue: about 260 thread instructions a key).
@@ -295,6 +296,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_plan(const uint32_t *__restr
                 ctl->guard = 1u;
         }
     }
+    __syncthreads();
+    if (threadIdx.x == 0) ctl->planned = atomicAdd(&ctl->buckets, 0u);
 }
 
 // -------------------------------------------------------------- 3. moves
@@ -519,81 +522,76 @@ __global__ void __launch_bounds__(kMoveThreads, 2) k_ps_place(const unsigned lon
 // keys, grouped as above, and moved bin by bin from `in` to the same range of
 // `out`.  One block per bucket; a bucket has at most kPsGiant keys.
 constexpr int kSplitGroups = 2048;  // of one bucket: at most 3 kPsGiant / kPsT + 4
-__global__ void __launch_bounds__(kThreads, 1) k_ps_split(const unsigned long long *__restrict__ in,
-                                                       unsigned long long *__restrict__ out, const int64_t *K_dev,
-                                                       PsControl *ctl, PsBucket *list, uint32_t list_cap,
-                                                       const PsBucket *__restrict__ over) {
-    if (ctl->guard) return;
-    extern __shared__ uint32_t h[];  // [kFine] counts, then cursors
-    __shared__ uint32_t gstart[kSplitGroups], gfine[kSplitGroups];
-    const int b = key_bits(*K_dev), s1 = fine_shift(b), s2 = s1 > kFineBits ? s1 - kFineBits : 0;
+// h: [kFine] counts, then cursors; after them [2 * kSplitGroups].  Every thread of
+// the block calls it; ends in a barrier.
+__device__ void ps_split(const PsBucket &o, int b, const unsigned long long *__restrict__ in,
+                         unsigned long long *__restrict__ out, PsControl *ctl, PsBucket *list, uint32_t list_cap,
+                         uint32_t *h) {
+    uint32_t *gstart = h + kFine, *gfine = gstart + kSplitGroups;
+    const int s1 = fine_shift(b), s2 = s1 > kFineBits ? s1 - kFineBits : 0;
     const uint32_t rows_per_bin = s2 >= b ? 1u << (s2 - b) : 0u;
-    const uint32_t count = ctl->over;
-    for (uint32_t q = blockIdx.x; q < count; q += gridDim.x) {
-        const PsBucket o = over[q];
-        const int NF = int(o.span >> s2);  // a power of two up to kFine
-        for (int f = threadIdx.x; f < kFine; f += kThreads) h[f] = 0u;
-        __syncthreads();
-        const unsigned long long *src = in + o.start;
-        constexpr int kIn = 8;
-        for (uint32_t i0 = threadIdx.x; i0 < o.count; i0 += kThreads * kIn) {
-            unsigned long long k[kIn];
+    const int NF = int(o.span >> s2);  // a power of two up to kFine
+    for (int f = threadIdx.x; f < kFine; f += kThreads) h[f] = 0u;
+    __syncthreads();
+    const unsigned long long *src = in + o.start;
+    constexpr int kIn = 8;
+    for (uint32_t i0 = threadIdx.x; i0 < o.count; i0 += kThreads * kIn) {
+        unsigned long long k[kIn];
 #pragma unroll
-            for (int r = 0; r < kIn; ++r) k[r] = i0 + r * kThreads < o.count ? src[i0 + r * kThreads] : o.lo;
+        for (int r = 0; r < kIn; ++r) k[r] = i0 + r * kThreads < o.count ? src[i0 + r * kThreads] : o.lo;
 #pragma unroll
-            for (int r = 0; r < kIn; ++r)
-                if (i0 + r * kThreads < o.count) atomicAdd(&h[swz(uint32_t((k[r] - o.lo) >> s2) & (kFine - 1))], 1u);
-        }
-        __syncthreads();
-        const uint32_t groups = ps_groups(
-            NF, rows_per_bin, 0u, [&](int f) { return h[swz(f)]; }, [&](int, uint32_t, uint32_t) {},
-            [&](uint32_t g, int f, uint32_t k) {
-                if (g < kSplitGroups) {
-                    gstart[g] = k;
-                    gfine[g] = uint32_t(f);
-                }
-            });
-        if (groups > kSplitGroups) {  // cannot happen, see kSplitGroups
-            if (threadIdx.x == 0) ctl->guard = 1u;
-            return;
-        }
-        for (uint32_t g = threadIdx.x; g < groups; g += kThreads) {
-            const uint32_t f0 = gfine[g], f1 = g + 1 < groups ? gfine[g + 1] : uint32_t(NF);
-            const uint32_t k0 = gstart[g], k1 = g + 1 < groups ? gstart[g + 1] : o.count;
-            if (k1 == k0) continue;
-            PsBucket e{o.start + k0, k1 - k0, o.lo + (static_cast<unsigned long long>(f0) << s2),
-                       static_cast<unsigned long long>(f1 - f0) << s2, kSrcSplit, 0u};
-            if (f1 - f0 == 1 && s2 == 0) continue;  // equal keys, in their place already
-            if (e.count > kPsW && s2 > kFineBits && (1 << (s2 - kFineBits)) > kPsMaxSlices) ctl->guard = 1u;
-            ps_append(e, ctl, list, list_cap);
-        }
-        __syncthreads();
-        // counts -> exclusive prefix (a cursor per bin), then every key to its bin
-        constexpr int kPer = kFine / kThreads;
-        uint32_t sum = 0, all;
-        for (int f = 0; f < kPer; ++f) sum += h[swz(threadIdx.x * kPer + f)];
-        uint32_t run = ps_scan<uint32_t>(sum, &all);
-        for (int f = 0; f < kPer; ++f) {
-            uint32_t &x = h[swz(threadIdx.x * kPer + f)];
-            const uint32_t c = x;
-            x = run;
-            run += c;
-        }
-        __syncthreads();
-        unsigned long long *dst = out + o.start;
-        for (uint32_t i0 = threadIdx.x; i0 < o.count; i0 += kThreads * kIn) {
-            unsigned long long k[kIn];
-#pragma unroll
-            for (int r = 0; r < kIn; ++r) k[r] = i0 + r * kThreads < o.count ? src[i0 + r * kThreads] : o.lo;
-#pragma unroll
-            for (int r = 0; r < kIn; ++r)
-                if (i0 + r * kThreads < o.count) {
-                    const uint32_t pos = atomicAdd(&h[swz(uint32_t((k[r] - o.lo) >> s2) & (kFine - 1))], 1u);
-                    if (pos < o.count) dst[pos] = k[r];
-                }
-        }
-        __syncthreads();
+        for (int r = 0; r < kIn; ++r)
+            if (i0 + r * kThreads < o.count) atomicAdd(&h[swz(uint32_t((k[r] - o.lo) >> s2) & (kFine - 1))], 1u);
     }
+    __syncthreads();
+    const uint32_t groups = ps_groups(
+        NF, rows_per_bin, 0u, [&](int f) { return h[swz(f)]; }, [&](int, uint32_t, uint32_t) {},
+        [&](uint32_t g, int f, uint32_t k) {
+            if (g < kSplitGroups) {
+                gstart[g] = k;
+                gfine[g] = uint32_t(f);
+            }
+        });
+    if (groups > kSplitGroups) {  // cannot happen, see kSplitGroups
+        if (threadIdx.x == 0) ctl->guard = 1u;
+        return;
+    }
+    for (uint32_t g = threadIdx.x; g < groups; g += kThreads) {
+        const uint32_t f0 = gfine[g], f1 = g + 1 < groups ? gfine[g + 1] : uint32_t(NF);
+        const uint32_t k0 = gstart[g], k1 = g + 1 < groups ? gstart[g + 1] : o.count;
+        if (k1 == k0) continue;
+        PsBucket e{o.start + k0, k1 - k0, o.lo + (static_cast<unsigned long long>(f0) << s2),
+                   static_cast<unsigned long long>(f1 - f0) << s2, kSrcSplit, 0u};
+        if (f1 - f0 == 1 && s2 == 0) continue;  // equal keys, in their place already
+        if (e.count > kPsW && s2 > kFineBits && (1 << (s2 - kFineBits)) > kPsMaxSlices) ctl->guard = 1u;
+        ps_append(e, ctl, list, list_cap);
+    }
+    __syncthreads();
+    // counts -> exclusive prefix (a cursor per bin), then every key to its bin
+    constexpr int kPer = kFine / kThreads;
+    uint32_t sum = 0, all;
+    for (int f = 0; f < kPer; ++f) sum += h[swz(threadIdx.x * kPer + f)];
+    uint32_t run = ps_scan<uint32_t>(sum, &all);
+    for (int f = 0; f < kPer; ++f) {
+        uint32_t &x = h[swz(threadIdx.x * kPer + f)];
+        const uint32_t c = x;
+        x = run;
+        run += c;
+    }
+    __syncthreads();
+    unsigned long long *dst = out + o.start;
+    for (uint32_t i0 = threadIdx.x; i0 < o.count; i0 += kThreads * kIn) {
+        unsigned long long k[kIn];
+#pragma unroll
+        for (int r = 0; r < kIn; ++r) k[r] = i0 + r * kThreads < o.count ? src[i0 + r * kThreads] : o.lo;
+#pragma unroll
+        for (int r = 0; r < kIn; ++r)
+            if (i0 + r * kThreads < o.count) {
+                const uint32_t pos = atomicAdd(&h[swz(uint32_t((k[r] - o.lo) >> s2) & (kFine - 1))], 1u);
+                if (pos < o.count) dst[pos] = k[r];
+            }
+    }
+    __syncthreads();
 }
 
 // --------------------------------------------------------------- 5. sort
@@ -674,23 +672,35 @@ __device__ void ps_count_out(const PsBucket &e, unsigned long long *buf, unsigne
     __syncthreads();
 }
 
+// kSplit: the splits of the oversize buckets first, then the buckets listed before
+// them; else the buckets that the splits have listed.  The largest hub takes one
+// block as long as hundreds of small buckets, which the other blocks sort
+// meanwhile; nothing waits for anything inside a launch.  (As a kernel of its own
+// the split of a 34 M-edge R-MAT graph took 185 us, nearly all of it one hub.)
+template <bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf0, unsigned long long *buf1,
-                                                      const int64_t *K_dev, PsControl *ctl,
-                                                      const PsBucket *__restrict__ list, uint32_t list_cap) {
+                                                      const int64_t *K_dev, PsControl *ctl, PsBucket *list,
+                                                      uint32_t list_cap, const PsBucket *__restrict__ over) {
     if (ctl->guard) return;
     extern __shared__ uint32_t smem[];
     __shared__ uint32_t big[kPsW / (kPsRank + 1) + 1];  // bins too large to rank: start | size << 16
     __shared__ uint32_t bigs, next_sh;
     const int b = key_bits(*K_dev), s1 = fine_shift(b);
-    const uint32_t count = min(ctl->buckets, list_cap);
+    const uint32_t splits = kSplit ? ctl->over : 0u, planned = ctl->planned;
+    const uint32_t count = kSplit ? splits + min(planned, list_cap) : min(ctl->buckets, list_cap) - min(planned, list_cap);
     while (true) {
         if (threadIdx.x == 0) {
-            next_sh = atomicAdd(&ctl->ticket, 1u);
+            next_sh = atomicAdd(kSplit ? &ctl->split_ticket : &ctl->ticket, 1u);
             bigs = 0u;
         }
         __syncthreads();
-        const uint32_t q = next_sh;
+        uint32_t q = next_sh;
         if (q >= count) return;
+        if (kSplit && q < splits) {
+            ps_split(over[q], b, buf1, buf0, ctl, list, list_cap, smem);
+            continue;
+        }
+        q = kSplit ? q - splits : q + planned;
         const PsBucket e = list[q];
         const unsigned long long *in = ((e.flags & kSrcSplit) ? buf0 : buf1) + e.start;
         unsigned long long *out = buf0 + e.start;
@@ -834,7 +844,7 @@ constexpr size_t kHistSmem = size_t(kFine) * sizeof(uint32_t);
 // primaries besides kPsW keys
 constexpr size_t kSortSmem = size_t(kPsW) * 8 + size_t(kPsMaxPrim) * 8 + 4096 + 64;
 static_assert(kPsW <= 65536 / 2, "bin starts and sizes in 16 bits");
-static_assert(kSortSmem >= kHistSmem, "ps_count_out counts in the same memory");
+static_assert(kSortSmem >= kHistSmem + 2 * kSplitGroups * sizeof(uint32_t), "splits and ps_count_out work in the same memory");
 }  // namespace
 
 void carve_pair_sort(Carver &c, int64_t m, int32_t n, PairSortScratch &s) {
@@ -864,8 +874,8 @@ int pair_sort(const int32_t *edges, int64_t m, int32_t n, const int32_t *node_ma
     BGV_CUDA(cudaFuncSetAttribute(k_ps_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kHistSmem)));
     BGV_CUDA(cudaFuncSetAttribute(k_ps_coarse, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCoarseSmem)));
     BGV_CUDA(cudaFuncSetAttribute(k_ps_place, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kPlaceSmem)));
-    BGV_CUDA(cudaFuncSetAttribute(k_ps_split, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kHistSmem)));
-    BGV_CUDA(cudaFuncSetAttribute(k_ps_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSortSmem)));
+    BGV_CUDA(cudaFuncSetAttribute(k_ps_sort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSortSmem)));
+    BGV_CUDA(cudaFuncSetAttribute(k_ps_sort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSortSmem)));
     BGV_CUDA(cudaMemsetAsync(s.total, 0, sizeof(uint32_t) * kFine, st));
     BGV_CUDA(cudaMemsetAsync(s.ctl, 0, sizeof(PsControl), st));
     int4 *mapped = reinterpret_cast<int4 *>(buf1);  // the mapped edges, until their keys are in buf0
@@ -881,10 +891,10 @@ int pair_sort(const int32_t *edges, int64_t m, int32_t n, const int32_t *node_ma
     note_launch(), k_ps_place<<<grid_for(2 * m, kMoveKeys, 2 * sms), kMoveThreads, kPlaceSmem, st>>>(
         buf0, K_dev, s.bmap, s.bstart, s.run_cursor, s.ctl, s.cursor, buf1, cap);
     BGV_TRY(launch_status());
-    note_launch(), k_ps_split<<<grid_for(2 * m, int(kPsW), sms), kThreads, kHistSmem, st>>>(buf1, buf0, K_dev, s.ctl, s.list, s.list_cap,
-                                                                   s.over);
+    const int blocks = grid_for(2 * m, int(kPsT), sms);
+    note_launch(), k_ps_sort<true><<<blocks, kThreads, kSortSmem, st>>>(buf0, buf1, K_dev, s.ctl, s.list, s.list_cap, s.over);
     BGV_TRY(launch_status());
-    note_launch(), k_ps_sort<<<grid_for(2 * m, int(kPsT), sms), kThreads, kSortSmem, st>>>(buf0, buf1, K_dev, s.ctl, s.list, s.list_cap);
+    note_launch(), k_ps_sort<false><<<blocks, kThreads, kSortSmem, st>>>(buf0, buf1, K_dev, s.ctl, s.list, s.list_cap, s.over);
     return launch_status();
 }
 
