@@ -30,6 +30,8 @@
  *             streams are made by the first such call of a host thread on a
  *             device (make it outside any stream capture) and live until the
  *             process ends; each step makes and destroys four CUDA events.
+ *             (Steps and runs on graphs of up to 2,048 bodies and 524,288 CSR
+ *             entries are one kernel on `stream` itself.)
  * Scratch.    The library allocates no memory.  Each stage takes a caller
  *             workspace `ws` of `ws_bytes` bytes (256-byte aligned), sized by
  *             the matching *_ws_size query.  The first 256 bytes of every
@@ -339,11 +341,12 @@ int bgv_fa2_run(int64_t K, int64_t nnz, const int32_t *csr_off, const int32_t *c
  * BGV_FA2_STAGES stages of each step (on the library stream that runs the
  * main chain); synchronises `stream` and returns in stage_ms[BGV_FA2_STAGES]
  * the summed milliseconds per stage:
- *   0 frame + Morton keys (from the second step on: frame + the hinted
- *   sort's samples), 1 sort (the radix sort in the first step, the rest of
- *   the hinted sort in the others), 2 gather into Morton order and moment
- *   prefix sums, 3 radix tree and quadtree cells, 4 pre-order layout,
- *   5 Barnes-Hut repulsion, 6 the wait for the attraction (which runs beside
+ *   0 frame (from the second step on the step before left it), and the Morton
+ *   keys when the radix sort follows, 1 sort (the hinted sort; in a first step
+ *   of more than 262,144 bodies the radix sort), 2 gather into Morton order,
+ *   moments and the quadtree cells inside tiles of bodies, 3 cells across
+ *   tiles, 4 pre-order layout, 5 Barnes-Hut repulsion, 6 the wait for the
+ *   attraction (which runs beside
  *   stages 0-5), 7 total force, swing/traction, speed and displacement (one
  *   persistent kernel).
  * Creates and destroys (BGV_FA2_STAGES + 1) * iterations CUDA events. */
@@ -452,8 +455,10 @@ int bgv_fa2_run_batched(int32_t G, const int64_t *koff, int64_t nnz, const int32
                         float *Fprev, double *speed, void *ws, size_t ws_bytes, void *stream);
 
 /* ------------------------------------------------------------------------
- * 7. Autotuners.  The radix sort of the supergraph and ForceAtlas2 stages
- *    runs either as one onesweep kernel per pass with decoupled look-back
+ * 7. Autotuners.  The radix sort (of the supergraph's pairs below 131,072
+ *    edges, of Morton keys in a first step of more than 262,144 bodies, and of
+ *    degrees and sizes) runs either as one onesweep kernel per pass with
+ *    decoupled look-back
  *    (method 0), 8 keys per thread up to a size cutoff and 16 above it, or
  *    as one cooperative kernel for all its passes (method 1: per pass, digit
  *    counts per block chunk, a scan over the chunks, a stable scatter; no
@@ -520,13 +525,13 @@ int64_t bgv_set_sort_cutoff(int64_t cutoff);
 int32_t bgv_set_sort_method(int32_t method);
 
 /* ------------------------------------------------------------------------
- * Hinted sort.  The radix tree of the Barnes-Hut repulsion (§3.1, the
- * quadtree of ForceAtlas2's repulsion) is built over the bodies in Morton
- * order.  A body moves little between two steps, so from the second step of
- * a run on (bgv_fa2_run, bgv_layout*) the library finds that order with a
- * sample sort whose buckets follow the previous step's order, instead of a
- * full radix sort; both give the same order, (key, id).  The paper has no
- * counterpart.
+ * Hinted sort.  The quadtree of the Barnes-Hut repulsion (Section 3.1) is built
+ * over the bodies in Morton order.  A body moves little between two steps, so
+ * from the second step of a run on (bgv_fa2_run, bgv_layout*) the library finds
+ * that order with a bucket sort whose buckets follow the previous step's order;
+ * a first or single step of up to 262,144 bodies takes buckets between sampled
+ * keys, a larger one the full radix sort.  All give the same order, (key, id).
+ * The paper has no counterpart.
  *
  * bgv_sort_hinted sorts the pairs (keys[id], id), id in [0, K), into (key, id)
  * order and writes them to out_keys and out_ids.  `hint` is an order of the
@@ -542,11 +547,11 @@ int32_t bgv_set_sort_method(int32_t method);
  * `stream`.  ws: bgv_sort_hinted_ws_size(K) bytes (0 for a K out of range),
  * header zeroed by bgv_ws_init.
  *
- * bgv_set_fa2_order(1) (the default) makes ForceAtlas2 runs use the hinted
- * sort from their second step on (for K up to the same limit); 0 makes every
- * step use the full radix sort.  Process wide; returns the previous value
- * (-1 and no change for other values).  A CUDA graph captured earlier keeps
- * the method it was captured with.
+ * bgv_set_fa2_order(1) (the default) makes ForceAtlas2 steps use these bucket
+ * sorts; 0 makes every step use the full radix sort.  Process wide; returns the
+ * previous value (-1 and no change for other values).  A CUDA graph captured
+ * earlier keeps the method it was captured with.  (Runs on up to 2,048 bodies
+ * sort inside one cluster of blocks whatever the method.)
  * ---------------------------------------------------------------------- */
 int64_t bgv_sort_hinted_max_keys(void);
 size_t bgv_sort_hinted_ws_size(int64_t K);
