@@ -101,7 +101,10 @@ constexpr int kDegThreads = 1024;
 constexpr int kRangeBits = 15;
 constexpr int kRange = 1 << kRangeBits;
 constexpr int kMaxRanges = 512;                    // n <= 16,777,216
-constexpr int64_t kDegSplitMin = int64_t(1) << 19; // edges; below, one kernel is shorter than three
+// Edges; below, one kernel is shorter than three.  The sketch takes 81 us at 2^20
+// R-MAT edges with the ranges and 67 without, 89 and 89 at 2^21, 110 and 129 at
+// 2^22; with uniform endpoints 87 and 75 at 2.2 M edges.
+constexpr int64_t kDegSplitMin = int64_t(1) << 22;
 constexpr int kDegIn = 4;                          // int4 loads per thread and tile
 constexpr int kPlaceThreads = 512;  // of k_deg_place, two blocks per SM: their phases overlap (437 us with one of 1,024)
 constexpr int kDegTile = kPlaceThreads * kDegIn * 4; // endpoints per tile

@@ -1,4 +1,4 @@
-"""Degrees counted by node ranges (from 524,288 edges up, to 16,777,216 nodes)
+"""Degrees counted by node ranges (from 4,194,304 edges up, to 16,777,216 nodes)
 against NumPy, around the ranges of 32,768 nodes and the smallest edge count."""
 import numpy as np
 import pytest
@@ -16,7 +16,7 @@ import gpu_pipeline as G  # noqa: E402
 B = G.B
 
 
-@pytest.mark.parametrize("m", [(1 << 19) - 1, 1 << 19, (1 << 19) + 1, 1_234_567])
+@pytest.mark.parametrize("m", [(1 << 22) - 1, 1 << 22, (1 << 22) + 1, 5_234_567])
 @pytest.mark.parametrize("n,skew", [(1, 1.0), (32_767, 1.0), (32_768, 5.0), (32_769, 1.0), (400_001, 3.0),
                                     (16_777_216, 1.0), (16_777_217, 1.0)])
 def test_sketch_over_node_ranges(n, m, skew):
@@ -28,7 +28,7 @@ def test_sketch_over_node_ranges(n, m, skew):
 
 
 def test_one_node_takes_every_endpoint_and_bad_ones_are_reported():
-    n, m = 100_000, 700_001
+    n, m = 100_000, 4_700_001
     e = np.full((m, 2), 65_536, np.int32)
     S, d, st = G.sketch(e, n, 1, 4096, 3)
     assert st == 0 and np.array_equal(S, oracle.sketch_degrees(e, n, 1, 4096, 3)[0])
