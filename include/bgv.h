@@ -455,7 +455,7 @@ int bgv_fa2_run_batched(int32_t G, const int64_t *koff, int64_t nnz, const int32
                         float *Fprev, double *speed, void *ws, size_t ws_bytes, void *stream);
 
 /* ------------------------------------------------------------------------
- * 7. Autotuners.  The radix sort (of the supergraph's pairs below 131,072
+ * 7. Autotuners.  The radix sort (of the supergraph's pairs below 1,048,576
  *    edges, of Morton keys in a first step of more than 262,144 bodies, and of
  *    degrees and sizes) runs either as one onesweep kernel per pass with
  *    decoupled look-back
