@@ -85,6 +85,14 @@ __device__ __forceinline__ void propose_edge(int32_t u, int32_t v, uint32_t e, u
     if (w >= 0) offer(best, w, e, lab);
 }
 
+// Edges from which a round filters them by the map.  Below, the map's way through
+// L2 costs more than the gathers it saves: ten rounds over 11,000 edges 160 us with
+// it and 136 without, four over 180,000 109 and 108, eight over 247,000 of an R-MAT
+// graph 132 and 159.  Where nearly every node passes, as on an even graph whose
+// threshold is the usual degree, the map saves nothing and a round is up to 8 %
+// longer than without (nine rounds over 1.08 M edges 240 us against 223).
+constexpr int64_t kMapMin = int64_t(1) << 17;
+
 // All rounds in one persistent kernel (cooperative launch, every block
 // resident): initial state and bit map, then per round the map into shared
 // memory, the proposals over the edge list, a grid barrier, the winning
@@ -100,11 +108,11 @@ __global__ void __launch_bounds__(kRoundThreads, 1) k_comm_rounds(
     const int32_t *__restrict__ edges, int64_t m, int32_t n, const uint32_t *__restrict__ deg_est,
     const int32_t *__restrict__ node_graph, const uint32_t *__restrict__ D0, int32_t passes, uint32_t threshold,
     uint32_t growth, int tie_mode, int32_t jumps, uint2 *state, uint4 *bstate, unsigned long long *best, uint32_t *jump,
-    uint32_t *map, int shift, int words, uint32_t *any, int32_t *__restrict__ labels, uint32_t *__restrict__ deg_out,
+    uint32_t *map, int shift, int words, int filter, uint32_t *any, int32_t *__restrict__ labels, uint32_t *__restrict__ deg_out,
     uint32_t *status, WsHeader *hdr, int spin_limit) {
     extern __shared__ uint4 map_sh4[];
     const uint32_t *map_sh = reinterpret_cast<const uint32_t *>(map_sh4);
-    constexpr int kLoads = kB ? 1 : 2;  // int4 (two edges each) per thread in flight: 64 registers
+    constexpr int kLoads = kB ? 1 : 3;  // int4 (two edges each) per thread in flight: 64 registers
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     const int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
@@ -117,6 +125,7 @@ __global__ void __launch_bounds__(kRoundThreads, 1) k_comm_rounds(
             bool ok = false;
             const int64_t v0 = q << shift, v1 = (q + 1) << shift;
             for (int64_t v = v0; v < v1 && v < n; ++v) ok |= pass(v);
+            if (!filter) continue;
             const uint32_t word = __ballot_sync(0xFFFFFFFFu, ok);
             if (lane == 0) {
                 map[q >> 5] = word;
@@ -140,17 +149,19 @@ __global__ void __launch_bounds__(kRoundThreads, 1) k_comm_rounds(
     const int64_t pairs = m >> 1;
     auto passes_map = [&](int32_t x) {
         const uint32_t b = uint32_t(x) >> shift;
-        return ((map_sh[b >> 5] >> (b & 31u)) & 1u) != 0u;
+        return !filter || ((map_sh[b >> 5] >> (b & 31u)) & 1u) != 0u;
     };
     // both endpoints in range (else reported), not a loop, and both on the map
     auto wanted = [&](int32_t u, int32_t v) { return endpoints_ok(u, v, n, status) && passes_map(u) && passes_map(v); };
     unsigned long long D = threshold;
     const unsigned long long factor = growth ? growth : threshold;
     for (int32_t p = 0; p < passes; ++p) {
-        if (p == 0 || __ldcg(&any[p & 1]) != 0u) {
+        if (!filter || p == 0 || __ldcg(&any[p & 1]) != 0u) {
             const uint4 *src = reinterpret_cast<const uint4 *>(map);
-            for (int i = threadIdx.x; i < words / 4; i += kRoundThreads) map_sh4[i] = __ldcg(src + i);
-            __syncthreads();
+            if (filter) {
+                for (int i = threadIdx.x; i < words / 4; i += kRoundThreads) map_sh4[i] = __ldcg(src + i);
+                __syncthreads();
+            }
             for (int64_t q0 = t0; q0 < pairs; q0 += stride * kLoads) {
                 int4 e[kLoads];
                 bool go[2 * kLoads];
@@ -329,15 +340,18 @@ int run_communities(const int32_t *edges, int64_t m, int32_t n, const uint32_t *
     int tmode = tie_mode, limit = spin_limit();
     uint32_t *map = s.map, *any = s.any;
     int shift = map_shift(n), words = int(map_words(n, shift));
+    int filter = m >= kMapMin ? 1 : 0;
     BGV_CUDA(cudaMemsetAsync(any, 0, 2 * sizeof(uint32_t), st));
     void *args[] = {&edges, &m, &n, &deg_est, &node_graph, &D0, &passes, &threshold, &growth, &tmode, &jumps,
-                    &state, &bstate, &best, &jump, &map, &shift, &words, &any, &labels, &deg_out, &status, &hdr, &limit};
+                    &state, &bstate, &best, &jump, &map, &shift, &words, &filter, &any, &labels, &deg_out, &status, &hdr, &limit};
     const void *kernel = batch ? reinterpret_cast<const void *>(k_comm_rounds<true>)
                                : reinterpret_cast<const void *>(k_comm_rounds<false>);
     const size_t smem = size_t(words) * sizeof(uint32_t);
     BGV_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMapBytes));
-    // no more blocks than there is work for: a barrier over few blocks is shorter
-    const int64_t work = int64_t(n) > m / 4 ? int64_t(n) : m / 4;
+    // no more blocks than there is work for (two edges a thread): a barrier over
+    // few blocks is shorter; with four a thread ten rounds over 11,000 edges took 136
+    // us, with two 110
+    const int64_t work = int64_t(n) > m / 2 ? int64_t(n) : m / 2;
     const int blocks = coop_blocks(kernel, kRoundThreads, grid_for(work, kRoundThreads, sm_count()), smem);
     return launch_coop(kernel, blocks, kRoundThreads, args, st, smem);
 }

@@ -1,5 +1,5 @@
 """Community rounds behind the bit map of nodes that pass the threshold: one
-id per bit, several ids per bit (more ids than the map has bits), rounds that
+id per bit (from 131,072 edges up; without the map below), several ids per bit (more ids than the map has bits), rounds that
 no node passes before rounds that some do, and bad endpoints when no node passes."""
 import numpy as np
 import pytest
@@ -20,7 +20,8 @@ B = G.B
 MAP_BITS = 208 * 1024 * 8
 
 
-@pytest.mark.parametrize("n,m", [(1, 0), (31, 60), (33, 61), (128, 400), (1025, 4001), (40_000, 160_001),
+@pytest.mark.parametrize("n,m", [(1, 0), (31, 60), (33, 61), (128, 400), (1025, 4001), (40_000, 160_001), (33, 1 << 17), (1025, (1 << 17) + 1),
+                                 (40_000, (1 << 17) - 1), (40_000, 300_001),
                                  (MAP_BITS, 800_000), (MAP_BITS + 1, 800_001), (4 * MAP_BITS + 5, 2_000_001)])
 @pytest.mark.parametrize("threshold,tie", [(0, 1), (1, 0), (6, 1)])
 def test_rounds_match_oracle(n, m, threshold, tie):
@@ -34,9 +35,11 @@ def test_rounds_match_oracle(n, m, threshold, tie):
     assert np.array_equal(lab, lab0) and np.array_equal(d, d0)
 
 
-def test_rounds_that_nothing_passes_come_before_rounds_that_move():
+@pytest.mark.parametrize("copies", [1, 7])  # 7: enough edges for the map
+def test_rounds_that_nothing_passes_come_before_rounds_that_move(copies):
     n, e, _ = graphgen.load("sbm16")
     deg = np.bincount(e.reshape(-1), minlength=n).astype(np.uint32) + 50
+    e = np.tile(e, (copies, 1))
     lab, d, st = G.communities(e, n, deg, 8, 1, 2, 0)  # thresholds 1, 2, 4, ..., 128: degrees start at 50
     lab0, d0 = oracle.communities(e, n, deg, 8, 1, 2, 0)
     assert st == 0 and (lab0 != np.arange(n)).any()
