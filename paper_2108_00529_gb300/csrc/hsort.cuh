@@ -181,6 +181,7 @@ __global__ void __launch_bounds__(256) k_hs_sample(KeyOf key_of, const uint32_t 
 // 1b. Ranks of the samples by counting, one slice of the others per block
 // row; the last block places every s-th one as a splitter.
 __global__ void __launch_bounds__(256) k_hs_rank(int ns, int s, HsBuffers h) {  // 256 threads
+    chain_wait();  // with no samples in a block's slice too: its tickets are the samples' kernel's to clear
     __shared__ unsigned long long sk[(kHsMaxSamples + kHsRankSlices - 1) / kHsRankSlices];
     __shared__ uint32_t si[(kHsMaxSamples + kHsRankSlices - 1) / kHsRankSlices];
     __shared__ bool last;
@@ -188,7 +189,6 @@ __global__ void __launch_bounds__(256) k_hs_rank(int ns, int s, HsBuffers h) {  
     const int j0 = blockIdx.y * per;
     const int j1 = min(ns, j0 + per);
     for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-    chain_wait();
         sk[j - j0] = h.smp_key[j];
         si[j - j0] = h.smp_id[j];
     }
