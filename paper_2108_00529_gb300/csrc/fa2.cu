@@ -914,8 +914,9 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
         return BGV_OK;
     };
 
-    // The per-step counters are cleared by k_keys; S and T are written whole
-    // by the node kernels; the last-block tickets are reset by their last
+    // Of the per-step counters, k_tile_cross writes tree_nodes whole and k_tile_emit
+    // clears the interactions before the traversal counts them; S and T are
+    // written whole by the tail; the last-block tickets are reset by their last
     // blocks (the header starts zeroed, see bgv_ws_init).
     BGV_TRY(mark(0));
     ForkJoin ev;
@@ -1044,7 +1045,9 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
                                s.skip, s.T, koff, s.bgraph, s.body, K, p.kr, theta2, s.Frep, &hdr->interactions,
                                &hdr->interactions_total));
     } else {
+        // no tree kernels, which leave the step's counters (interactions, tree_nodes)
         BGV_CUDA(cudaMemsetAsync(s.Frep, 0, sizeof(float2), st));
+        BGV_CUDA(cudaMemsetAsync(&hdr->interactions, 0, 2 * sizeof(unsigned long long), st));
         BGV_TRY(mark(3));
         BGV_TRY(mark(4));
         BGV_TRY(mark(5));
