@@ -681,7 +681,6 @@ template <bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf0, unsigned long long *buf1,
                                                       const int64_t *K_dev, PsControl *ctl, PsBucket *list,
                                                       uint32_t list_cap, const PsBucket *__restrict__ over) {
-    if (ctl->guard) return;
     extern __shared__ uint32_t smem[];
     __shared__ uint32_t big[kPsW / (kPsRank + 1) + 1];  // bins too large to rank: start | size << 16
     __shared__ uint32_t bigs, next_sh;
@@ -690,7 +689,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf
     const uint32_t count = kSplit ? splits + min(planned, list_cap) : min(ctl->buckets, list_cap) - min(planned, list_cap);
     while (true) {
         if (threadIdx.x == 0) {
-            next_sh = atomicAdd(kSplit ? &ctl->split_ticket : &ctl->ticket, 1u);
+            // a split in another block may set the guard at any time: one thread
+            // reads it, so that a block goes on or ends as a whole
+            const bool off = *static_cast<volatile uint32_t *>(&ctl->guard) != 0u;
+            next_sh = off ? 0xFFFFFFFFu : atomicAdd(kSplit ? &ctl->split_ticket : &ctl->ticket, 1u);
             bigs = 0u;
         }
         __syncthreads();
