@@ -343,7 +343,7 @@ int bgv_fa2_run(int64_t K, int64_t nnz, const int32_t *csr_off, const int32_t *c
  * the summed milliseconds per stage:
  *   0 frame (from the second step on the step before left it), and the Morton
  *   keys when the radix sort follows, 1 sort (the hinted sort; in a first step
- *   of more than 262,144 bodies the radix sort), 2 gather into Morton order,
+ *   of more than 65,536 bodies the radix sort), 2 gather into Morton order,
  *   moments and the quadtree cells inside tiles of bodies, 3 cells across
  *   tiles, 4 pre-order layout, 5 Barnes-Hut repulsion, 6 the wait for the
  *   attraction (which runs beside
@@ -456,7 +456,7 @@ int bgv_fa2_run_batched(int32_t G, const int64_t *koff, int64_t nnz, const int32
 
 /* ------------------------------------------------------------------------
  * 7. Autotuners.  The radix sort (of the supergraph's pairs below 1,048,576
- *    edges, of Morton keys in a first step of more than 262,144 bodies, and of
+ *    edges, of Morton keys in a first step of more than 65,536 bodies, and of
  *    degrees and sizes) runs either as one onesweep kernel per pass with
  *    decoupled look-back
  *    (method 0), 8 keys per thread up to a size cutoff and 16 above it, or
@@ -529,7 +529,7 @@ int32_t bgv_set_sort_method(int32_t method);
  * over the bodies in Morton order.  A body moves little between two steps, so
  * from the second step of a run on (bgv_fa2_run, bgv_layout*) the library finds
  * that order with a bucket sort whose buckets follow the previous step's order;
- * a first or single step of up to 262,144 bodies takes buckets between sampled
+ * a first or single step of up to 65,536 bodies takes buckets between sampled
  * keys, a larger one the full radix sort.  All give the same order, (key, id).
  * The paper has no counterpart.
  *

@@ -1029,19 +1029,20 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
     BGV_TRY(mark(2));
     if (K >= 2) {
         const unsigned tiles = unsigned(tile_count(K));
-        BGV_TRY(launch_chained(hs_early(K), k_tile, tiles, kTileThreads, st, s.sort.keys[res], s.sort.vals[res], K, pos, mass, s.frame,
+        const bool early = hs_early(K, !hinted);
+        BGV_TRY(launch_chained(early, k_tile, tiles, kTileThreads, st, s.sort.keys[res], s.sort.vals[res], K, pos, mass, s.frame,
                                s.bgraph, L, gbits, p.leaf_cap, s.body, s.tree, &hdr->status, spin_limit()));
         BGV_TRY(mark(3));
         const unsigned per = kTileThreads / 32;  // tiles per block
-        BGV_TRY(launch_chained(hs_early(K), k_tile_cross, (tiles + per - 1) / per, kTileThreads, st, K, L, p.leaf_cap, s.frame,
+        BGV_TRY(launch_chained(early, k_tile_cross, (tiles + per - 1) / per, kTileThreads, st, K, L, p.leaf_cap, s.frame,
                                s.bgraph, s.tree, &hdr->tree_nodes));
         BGV_TRY(mark(4));
-        BGV_TRY(launch_chained(hs_early(K), k_tile_emit, tiles, kTileThreads, st, K, s.body, s.tree, s.T, s.geo, s.skip,
+        BGV_TRY(launch_chained(early, k_tile_emit, tiles, kTileThreads, st, K, s.body, s.tree, s.T, s.geo, s.skip,
                                &hdr->interactions));
         BGV_TRY(mark(5));
         const float theta2 = p.theta * p.theta;
         const unsigned rt = tune.repulse_threads == 128 ? 128u : unsigned(kThreads);
-        BGV_TRY(launch_chained(hs_early(K), rt == 128 ? k_repulse<128> : k_repulse<kThreads>, unsigned((K + rt - 1) / rt), rt, st, s.geo,
+        BGV_TRY(launch_chained(early, rt == 128 ? k_repulse<128> : k_repulse<kThreads>, unsigned((K + rt - 1) / rt), rt, st, s.geo,
                                s.skip, s.T, koff, s.bgraph, s.body, K, p.kr, theta2, s.Frep, &hdr->interactions,
                                &hdr->interactions_total));
     } else {

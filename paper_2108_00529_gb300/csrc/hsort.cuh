@@ -73,18 +73,25 @@ struct HsBuffers {
 };
 
 // Up to this many bodies the kernels of a step are short, and each may take its
-// place while the one before drains (launch_chained): a single step of 60,000
-// bodies 149.9 -> 133.9 us.  Above, the waiting blocks keep the attraction's off
-// the SMs: 500 steps of 1 M bodies of an R-MAT graph 190 ms without, 214 with it.
-// (The line lies where the first step's sort changes; sizes between not measured.)
-inline bool hs_early(int64_t K) { return K <= int64_t(1) << 18; }
+// place while the one before drains (launch_chained): single steps of 60,000,
+// 100,000 and 130,000 bodies 141, 158 and 163 us without and 127, 143 and 150 with
+// it.  In the later steps of a run, beside a longer attraction, the waiting blocks
+// keep the attraction's off the SMs: 30 steps of 60,000 bodies 2,993 us without and
+// 2,952 with it, of 130,000 equal, of 145,000 3,367 and 3,473, of 240,000 4,093 and
+// 4,211, 500 steps of 1 M bodies 190 and 214 ms.  A first or single step is shorter
+// with it up to its line (145,000 bodies 162 and 155 us, 240,000 184 and 178).
+inline bool hs_early(int64_t K, bool first) { return K <= int64_t(1) << (first ? 18 : 17); }
 inline int hs_buckets(int64_t K) { return K > kHsBucket ? int((K + kHsBucket - 1) / kHsBucket) : 1; }
 // Without a hint (bodies in id order) only the samples tell where the keys lie,
 // and a bucket between sampled splitters may hold twice its share: half the
-// share keeps it in shared memory.  For as many pairs as the samples serve with
-// kHsMaxPerBucket a bucket.
+// share keeps it in shared memory.  A bucket may also span far-apart clusters
+// of keys, crowded in few of its bins, and is merged then, 30 us more for the
+// whole sort.  Single steps with the radix sort and with this: 30,000 bodies 132 us
+// and 114, 60,000 140 and 127 (crowded 156), 80,000 143 and 142, 100,000 145 and
+// 143, 115,000 (crowded) 146 and 173, 160,000 158 and 199.
 constexpr int kHsFirstBucket = kHsBucket / 2;
-constexpr int64_t kHsFirstMax = int64_t(kHsMaxSamples) / kHsMaxPerBucket * kHsFirstBucket;  // 262,144
+constexpr int64_t kHsFirstMax = int64_t(1) << 16;
+static_assert(kHsFirstMax / kHsFirstBucket * kHsMaxPerBucket <= kHsMaxSamples, "eight samples a bucket");
 inline int hs_first_buckets(int64_t K) { return K > kHsFirstBucket ? int((K + kHsFirstBucket - 1) / kHsFirstBucket) : 1; }
 // Words from `count` on that are zero before a sort into nb buckets (and after it).
 inline int64_t hs_counter_words(int nb) { return 2 * int64_t(nb) + 2; }
@@ -791,15 +798,17 @@ int hinted_sort_place(KeyOf key_of, Split split, const uint32_t *hint, int64_t K
                       cudaStream_t st) {
     if (K <= 0) return BGV_OK;
     const HsBuffers h = hs_for(buffers, nb);
+    constexpr bool kSampled = std::is_same<Split, HsSampled>::value;
+    const bool early = hs_early(K, kSampled);
     // after the samples' kernels it follows in the chain; else an event precedes it
-    BGV_TRY(launch_chained(std::is_same<Split, HsSampled>::value && hs_early(K), k_hs_count<KeyOf, Split>,
+    BGV_TRY(launch_chained(kSampled && early, k_hs_count<KeyOf, Split>,
                            grid_for(K, 256, sm_count() * 8), 256, st, key_of, split, hint, K, nb, h, tmp_key, tmp_bucket,
                            status));
-    BGV_TRY(launch_chained(hs_early(K), k_hs_scatter, grid_for(K, 256, sm_count() * 8), 256, st, hint, K, h, tmp_key, tmp_bucket,
+    BGV_TRY(launch_chained(early, k_hs_scatter, grid_for(K, 256, sm_count() * 8), 256, st, hint, K, h, tmp_key, tmp_bucket,
                            slot_key, slot_id));
     int idbits = 0;  // bits of the largest id
     while (idbits < 32 && (int64_t(1) << idbits) < K) ++idbits;
-    return launch_chained(hs_early(K), k_hs_bucket, nb, kHsThreads, st, h, slot_key, slot_id, out_key, out_id, idbits);
+    return launch_chained(early, k_hs_bucket, nb, kHsThreads, st, h, slot_key, slot_id, out_key, out_id, idbits);
 }
 
 // The same with splitters from samples of the hint, nb <= kHsMaxBuckets; clears
@@ -822,7 +831,7 @@ int hinted_sort_sampled(KeyOf key_of, const uint32_t *hint, int64_t K, int nb, c
     BGV_TRY(launch_status());
     if (sh.ns > 0) {
         const dim3 g((sh.ns + 255) / 256, kHsRankSlices);
-        BGV_TRY(launch_chained(hs_early(K), k_hs_rank, g, 256, st, sh.ns, sh.s, h));
+        BGV_TRY(launch_chained(hs_early(K, true), k_hs_rank, g, 256, st, sh.ns, sh.s, h));
     }
     return hinted_sort_place(key_of, HsSampled{h.spl_key, h.spl_id}, hint, K, nb, h, tmp_key, tmp_bucket, slot_key,
                              slot_id, out_key, out_id, status, st);
