@@ -22,7 +22,12 @@
 //   2. Count: every pair's key and bucket (the search starts at the bucket
 //      its place in the hint would have, so a good hint needs one or two
 //      probes), counted per bucket with one atomic per bucket per warp; the
-//      last block turns the counts into bucket starts.
+//      last block turns the counts into bucket starts.  When the keys have
+//      moved as a whole (a caller's own start that expands, a frame that a few
+//      bodies stretch), many of them lie between two of the previous splitters:
+//      with a bucket of more than kHsPoor pairs the step takes samples of its
+//      own keys after all and counts again.  Those two kernels follow every count
+//      and return at once as a rule.
 //   3. Scatter: every pair to its bucket (one atomic per bucket per warp).
 //   4. Bucket sort: one block per bucket.  Up to kHsCap pairs it sorts in
 //      shared memory, as single words of its key above the least one and its id
@@ -52,23 +57,25 @@ constexpr int kHsPairCap = kHsThreads * kHsItems;  // 2048: a chunk of the pair 
 constexpr int kHsCap = kHsPairCap;      // larger buckets take the chunked path
 constexpr int kHsCapBits = 11;
 static_assert(kHsCap == 1 << kHsCapBits, "places of a bucket");
-constexpr int kHsRankSlices = 16;       // slices of the samples per ranking thread
+constexpr int kHsRankSlices = 8;       // slices of the samples per ranking thread
 constexpr int kHsBins = 2048;           // bins of a bucket's words
 constexpr uint32_t kHsRankBin = 32;     // largest bin ranked by counting
 constexpr int kHsSmem = kHsCap + kHsCap / 16;  // skewed shared-memory slots
+constexpr uint32_t kHsPoor = 2 * kHsCap;  // a larger bucket and the sort counts again
 
 inline int64_t hs_max_keys() { return int64_t(kHsMaxBuckets) * kHsBucket; }
 
 // Small device arrays of the sort (the large ones are the caller's).
 struct HsBuffers {
-    unsigned long long *smp_key;  // [kHsMaxSamples] samples in hint order (public entry point only)
+    unsigned long long *smp_key;  // [kHsMaxSamples] samples in hint order (sampled splitters only)
     uint32_t *smp_id;             // [kHsMaxSamples]
-    uint32_t *smp_rank;           // [kHsMaxSamples]
-    unsigned long long *spl_key;  // [kHsMaxBuckets] splitter u at u - 1
-    uint32_t *spl_id;             // [kHsMaxBuckets]
+    unsigned long long *spl_key;  // [nb] splitter u at u - 1
+    uint32_t *spl_id;             // [nb]
     uint32_t *count;              // [nb] pairs per bucket; zero between sorts, with all that follows:
     uint32_t *cursor;             // [nb] scatter cursors
-    uint32_t *ticket;             // [2] last-block tickets
+    uint32_t *ticket;             // [3] last-block tickets of the ranking, the count and the second count
+    uint32_t *poor;               // [1] the sort counts again
+    uint32_t *smp_rank;           // [hs_shape(nb).ns] ranks of the samples
     uint32_t *start;              // [nb + 1] bucket starts
 };
 
@@ -93,25 +100,48 @@ constexpr int kHsFirstBucket = kHsBucket / 2;
 constexpr int64_t kHsFirstMax = int64_t(1) << 16;
 static_assert(kHsFirstMax / kHsFirstBucket * kHsMaxPerBucket <= kHsMaxSamples, "eight samples a bucket");
 inline int hs_first_buckets(int64_t K) { return K > kHsFirstBucket ? int((K + kHsFirstBucket - 1) / kHsFirstBucket) : 1; }
+// Samples per bucket for K pairs in nb buckets (ns = 0: no splitters).  The ranking
+// compares all pairs of samples: 8 a bucket up to 512 buckets, 4 up to 2,048 and 2
+// above keep it shorter than the count.
+struct HsShape {
+    int s, ns;
+};
+inline HsShape hs_shape(int nb) {
+    HsShape h;
+    h.s = nb <= 512 ? kHsMaxPerBucket : nb <= 2048 ? kHsMaxPerBucket / 2 : kHsMaxPerBucket / 4;
+    h.ns = nb > 1 ? nb * h.s : 0;  // nb > 1 means K > 512 (nb - 1) >= 8 nb, so ns < K
+    return h;
+}
+// The shape of a sort whose splitters are always samples.
+inline HsShape hs_shape_sampled(int nb) {
+    HsShape h;
+    h.s = kHsMaxSamples / nb;
+    if (h.s > kHsMaxPerBucket) h.s = kHsMaxPerBucket;
+    if (h.s < 1) h.s = 1;
+    h.ns = nb > 1 ? nb * h.s : 0;
+    return h;
+}
+
 // Words from `count` on that are zero before a sort into nb buckets (and after it).
-inline int64_t hs_counter_words(int nb) { return 2 * int64_t(nb) + 2; }
+inline int64_t hs_counter_words(int nb) { return 2 * int64_t(nb) + 4 + hs_shape(nb).ns; }
 
 inline void carve_hs(Carver &c, int nb, bool sampled, HsBuffers &h) {
     h = HsBuffers{};
     if (sampled) {
         h.smp_key = c.take<unsigned long long>(kHsMaxSamples);
         h.smp_id = c.take<uint32_t>(kHsMaxSamples);
-        h.smp_rank = c.take<uint32_t>(kHsMaxSamples);
-        h.spl_key = c.take<unsigned long long>(kHsMaxBuckets);
-        h.spl_id = c.take<uint32_t>(kHsMaxBuckets);
     }
+    h.spl_key = c.take<unsigned long long>(size_t(nb));
+    h.spl_id = c.take<uint32_t>(size_t(nb));
     h.count = c.take<uint32_t>(size_t(hs_counter_words(nb)));
     h.start = c.take<uint32_t>(size_t(nb) + 1);
 }
 // The same buffers for a sort into nb buckets (no more than they were carved for).
 inline HsBuffers hs_for(HsBuffers h, int nb) {
     h.cursor = h.count + nb;
-    h.ticket = h.count + 2 * size_t(nb);
+    h.ticket = h.cursor + nb;
+    h.poor = h.ticket + 3;
+    h.smp_rank = h.poor + 1;
     return h;
 }
 
@@ -128,19 +158,6 @@ struct HsPrevious {  // the sorted pairs of the previous iteration
     __device__ unsigned long long key_at(int u) const { return __ldg(&key[int64_t(u + 1) * kHsBucket]); }
     __device__ uint32_t id_at(int u) const { return __ldg(&id[int64_t(u + 1) * kHsBucket]); }
 };
-
-// Samples per bucket for K pairs in nb buckets (ns = 0: no splitters).
-struct HsShape {
-    int s, ns;
-};
-inline HsShape hs_shape(int64_t K, int nb) {
-    HsShape h;
-    h.s = kHsMaxSamples / nb;
-    if (h.s > kHsMaxPerBucket) h.s = kHsMaxPerBucket;
-    if (h.s < 1) h.s = 1;
-    h.ns = nb > 1 ? nb * h.s : 0;  // nb > 1 means K > 512 (nb - 1) >= 8 nb, so ns < K
-    return h;
-}
 
 // Extra words the first kernel clears (for the kernels after the sort).
 struct HsClears {
@@ -179,39 +196,65 @@ __global__ void __launch_bounds__(256) k_hs_sample(KeyOf key_of, const uint32_t 
         const uint32_t id = hs_id(hint, p, K, status);
         h.smp_key[t] = key_of(id);
         h.smp_id[t] = id;
-        h.smp_rank[t] = 0u;
     }
     for (int64_t t = t0; t < counter_words; t += stride) h.count[t] = 0u;
     for (int64_t t = t0; t < clr.n_u32; t += stride) clr.u32[t] = 0u;
 }
 
+// The samples that k_hs_sample left.
+struct HsStored {
+    static constexpr bool kAgain = false;
+    const unsigned long long *key_;
+    const uint32_t *id_;
+    __device__ void get(int t, unsigned long long *key, uint32_t *id) const {
+        *key = key_[t];
+        *id = id_[t];
+    }
+};
+// Samples of the keys that the first count left, in hint order.
+struct HsCounted {
+    static constexpr bool kAgain = true;
+    const unsigned long long *key_;
+    const uint32_t *hint;
+    int64_t K;
+    int ns;
+    __device__ void get(int t, unsigned long long *key, uint32_t *id) const {
+        const int64_t p = ((2 * int64_t(t) + 1) * K) / (2 * int64_t(ns));
+        const uint32_t i = hint ? hint[p] : uint32_t(p);
+        *key = key_[p];
+        *id = i < uint64_t(K) ? i : 0u;  // reported by the count kernel
+    }
+};
+
 // 1b. Ranks of the samples by counting, one slice of the others per block
-// row; the last block places every s-th one as a splitter.
-__global__ void __launch_bounds__(256) k_hs_rank(int ns, int s, HsBuffers h) {  // 256 threads
-    chain_wait();  // with no samples in a block's slice too: its tickets are the samples' kernel's to clear
-    __shared__ unsigned long long sk[(kHsMaxSamples + kHsRankSlices - 1) / kHsRankSlices];
-    __shared__ uint32_t si[(kHsMaxSamples + kHsRankSlices - 1) / kHsRankSlices];
+// row; the last block places every s-th one as a splitter, and leaves the ranks
+// at zero.
+template <class Samples>
+__global__ void __launch_bounds__(256) k_hs_rank(Samples samples, int ns, int s, HsBuffers h) {  // 256 threads
+    chain_wait();  // with no samples in a block's slice too: its tickets are the kernel's before to clear
+    if (Samples::kAgain && *h.poor == 0u) return;
+    __shared__ unsigned long long sk[256];
+    __shared__ uint32_t si[256];
     __shared__ bool last;
     const int per = (ns + kHsRankSlices - 1) / kHsRankSlices;
     const int j0 = blockIdx.y * per;
     const int j1 = min(ns, j0 + per);
-    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-        sk[j - j0] = h.smp_key[j];
-        si[j - j0] = h.smp_id[j];
-    }
-    __syncthreads();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < ns) {
-        const unsigned long long ki = h.smp_key[i];
-        const uint32_t ii = h.smp_id[i];
-        uint32_t c = 0;
-        for (int j = j0; j < j1; ++j) {
-            const unsigned long long kj = sk[j - j0];
-            const uint32_t ij = si[j - j0];
-            c += (hs_less(kj, ij, ki, ii) || (kj == ki && ij == ii && j < i)) ? 1u : 0u;
+    unsigned long long ki = 0ull;
+    uint32_t ii = 0u, c = 0u;
+    if (i < ns) samples.get(i, &ki, &ii);
+    for (int b0 = j0; b0 < j1; b0 += 256) {
+        const int n = min(256, j1 - b0);
+        if (int(threadIdx.x) < n) samples.get(b0 + threadIdx.x, &sk[threadIdx.x], &si[threadIdx.x]);
+        __syncthreads();
+        for (int j = 0; j < n; ++j) {
+            const unsigned long long kj = sk[j];
+            const uint32_t ij = si[j];
+            c += (hs_less(kj, ij, ki, ii) || (kj == ki && ij == ii && b0 + j < i)) ? 1u : 0u;
         }
-        if (c) atomicAdd(&h.smp_rank[i], c);
+        __syncthreads();
     }
+    if (i < ns && c) atomicAdd(&h.smp_rank[i], c);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -221,23 +264,29 @@ __global__ void __launch_bounds__(256) k_hs_rank(int ns, int s, HsBuffers h) {  
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // every load first (one round trip to L2), then the placements
-    constexpr int kPer = kHsMaxSamples / 256;
-    uint32_t r[kPer], id[kPer];
-    unsigned long long key[kPer];
+    // every load of a round first (one round trip to L2), then the placements
+    constexpr int kPer = 16;
+    for (int t0 = threadIdx.x; t0 < ns; t0 += 256 * kPer) {
+        uint32_t r[kPer], id[kPer];
+        unsigned long long key[kPer];
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-        const int t = threadIdx.x + 256 * q;
-        r[q] = t < ns ? __ldcg(&h.smp_rank[t]) : 0u;
-        key[q] = t < ns ? __ldcg(&h.smp_key[t]) : 0ull;
-        id[q] = t < ns ? __ldcg(&h.smp_id[t]) : 0u;
-    }
+        for (int q = 0; q < kPer; ++q) {
+            const int t = t0 + 256 * q;
+            r[q] = id[q] = 0u;
+            key[q] = 0ull;
+            if (t < ns) {
+                r[q] = __ldcg(&h.smp_rank[t]);
+                samples.get(t, &key[q], &id[q]);
+            }
+        }
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-        if (r[q] >= uint32_t(s) && r[q] % uint32_t(s) == 0u && r[q] < uint32_t(ns)) {
-            const uint32_t u = r[q] / uint32_t(s);
-            h.spl_key[u - 1] = key[q];
-            h.spl_id[u - 1] = id[q];
+        for (int q = 0; q < kPer; ++q) {
+            if (t0 + 256 * q < ns) h.smp_rank[t0 + 256 * q] = 0u;
+            if (r[q] >= uint32_t(s) && r[q] % uint32_t(s) == 0u && r[q] < uint32_t(ns)) {
+                const uint32_t u = r[q] / uint32_t(s);
+                h.spl_key[u - 1] = key[q];
+                h.spl_id[u - 1] = id[q];
+            }
         }
     }
 }
@@ -287,14 +336,19 @@ __device__ __forceinline__ int hs_bucket(unsigned long long xk, uint32_t xi, con
     return lo;
 }
 
+// The keys of the second count: by place in the hint, as the first one left them.
+struct HsAgain {};
+
 // 2. Keys and buckets in hint order, counts per bucket; the last block
-// writes the bucket starts.
+// writes the bucket starts, or, with previous splitters and a bucket of more than
+// kHsPoor pairs, asks for the second count (KeyOf = HsAgain).
 template <class KeyOf, class Split>
 __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, const uint32_t *__restrict__ hint,
-                                                  int64_t K, int nb, HsBuffers h,
-                                                  unsigned long long *__restrict__ tmp_key,
+                                                  int64_t K, int nb, HsBuffers h, unsigned long long *tmp_key,
                                                   uint32_t *__restrict__ tmp_bucket, uint32_t *status) {
     chain_wait();
+    constexpr bool kAgain = std::is_same<KeyOf, HsAgain>::value, kWatch = std::is_same<Split, HsPrevious>::value;
+    if (kAgain && *h.poor == 0u) return;
     __shared__ bool last;
     __shared__ uint32_t part[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -307,10 +361,15 @@ __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, con
         int u = -1;
         if (p < K) {
             const uint32_t id = hs_id(hint, p, K, status);
-            const unsigned long long k = key_of(id);
+            unsigned long long k;
+            if constexpr (kAgain) {
+                k = tmp_key[p];
+            } else {
+                k = key_of(id);
+                tmp_key[p] = k;
+            }
             const int g = min(nb - 1, int(float(p) * g_scale));
             u = nb > 1 ? hs_bucket(k, id, split, nb, g) : 0;
-            tmp_key[p] = k;
             tmp_bucket[p] = uint32_t(u);
         }
         const unsigned peers = __match_any_sync(0xFFFFFFFFu, u);
@@ -320,13 +379,13 @@ __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, con
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        last = atomicAdd(&h.ticket[1], 1u) == gridDim.x - 1;
+        last = atomicAdd(&h.ticket[kAgain ? 2 : 1], 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
     // exclusive scan of the counts, 1,024 at a time
-    uint32_t carry = 0u;
+    uint32_t carry = 0u, most = 0u;
     for (int b0 = 0; b0 < nb; b0 += 1024) {
         const int b = b0 + 4 * int(threadIdx.x);
         uint32_t c[4], sum = 0u;
@@ -334,6 +393,7 @@ __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, con
         for (int q = 0; q < 4; ++q) {
             c[q] = b + q < nb ? __ldcg(&h.count[b + q]) : 0u;
             sum += c[q];
+            most = max(most, c[q]);
         }
         uint32_t inc = sum;
 #pragma unroll
@@ -357,6 +417,11 @@ __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, con
         __syncthreads();
     }
     if (threadIdx.x == 0) h.start[nb] = uint32_t(K);
+    if (kAgain && threadIdx.x == 0) *h.poor = 0u;
+    if (kWatch && __syncthreads_or(most > kHsPoor)) {
+        for (int b = threadIdx.x; b < nb; b += blockDim.x) h.count[b] = 0u;
+        if (threadIdx.x == 0) *h.poor = 1u;
+    }
 }
 
 // 3. Every pair to its bucket.
@@ -770,7 +835,7 @@ __global__ void __launch_bounds__(kHsThreads) k_hs_bucket(HsBuffers h, unsigned 
     if (threadIdx.x == 0) {
         h.count[u] = 0u;
         h.cursor[u] = 0u;
-        if (u == 0) h.ticket[0] = h.ticket[1] = 0u;
+        if (u == 0) h.ticket[0] = h.ticket[1] = h.ticket[2] = 0u;
     }
     const int64_t b0 = h.start[u];
     const int64_t n = int64_t(h.start[u + 1]) - b0;
@@ -804,7 +869,21 @@ int hinted_sort_place(KeyOf key_of, Split split, const uint32_t *hint, int64_t K
     BGV_TRY(launch_chained(kSampled && early, k_hs_count<KeyOf, Split>,
                            grid_for(K, 256, sm_count() * 8), 256, st, key_of, split, hint, K, nb, h, tmp_key, tmp_bucket,
                            status));
-    BGV_TRY(launch_chained(early, k_hs_scatter, grid_for(K, 256, sm_count() * 8), 256, st, hint, K, h, tmp_key, tmp_bucket,
+    // The second count, which returns at once as a rule: few blocks, launched beside
+    // the ranking, as the scatter is beside them (500 steps of 1 M bodies 171.2 ms
+    // without the two kernels, 172.8 so, 174.8 with 16 slices, 4 blocks an SM and
+    // plain launches).  What it is for: 20 steps of 1 M bodies, ten of them far off,
+    // 65 ms without and 9.1 with it; three steps from a tight start 12.3 and 1.5.
+    const bool again = !kSampled && nb > 1;
+    if (again) {
+        const HsShape sh = hs_shape(nb);
+        const dim3 g((sh.ns + 255) / 256, kHsRankSlices);
+        BGV_TRY(launch_chained(early, k_hs_rank<HsCounted>, g, 256, st, HsCounted{tmp_key, hint, K, sh.ns}, sh.ns, sh.s,
+                               h));
+        BGV_TRY(launch_chained(true, k_hs_count<HsAgain, HsSampled>, grid_for(K, 256, sm_count() * 2), 256, st,
+                               HsAgain{}, HsSampled{h.spl_key, h.spl_id}, hint, K, nb, h, tmp_key, tmp_bucket, status));
+    }
+    BGV_TRY(launch_chained(early || again, k_hs_scatter, grid_for(K, 256, sm_count() * 8), 256, st, hint, K, h, tmp_key, tmp_bucket,
                            slot_key, slot_id));
     int idbits = 0;  // bits of the largest id
     while (idbits < 32 && (int64_t(1) << idbits) < K) ++idbits;
@@ -821,7 +900,7 @@ int hinted_sort_sampled(KeyOf key_of, const uint32_t *hint, int64_t K, int nb, c
     if (K <= 0) return BGV_OK;
     if (nb > kHsMaxBuckets) return BGV_EINVAL;
     const HsBuffers h = hs_for(buffers, nb);
-    const HsShape sh = hs_shape(K, nb);
+    const HsShape sh = hs_shape_sampled(nb);
     const int64_t words = hs_counter_words(nb);
     int64_t work = sh.ns;
     for (const int64_t w : {words, clr.n_u32})
@@ -831,7 +910,8 @@ int hinted_sort_sampled(KeyOf key_of, const uint32_t *hint, int64_t K, int nb, c
     BGV_TRY(launch_status());
     if (sh.ns > 0) {
         const dim3 g((sh.ns + 255) / 256, kHsRankSlices);
-        BGV_TRY(launch_chained(hs_early(K, true), k_hs_rank, g, 256, st, sh.ns, sh.s, h));
+        BGV_TRY(launch_chained(hs_early(K, true), k_hs_rank<HsStored>, g, 256, st, HsStored{h.smp_key, h.smp_id},
+                               sh.ns, sh.s, h));
     }
     return hinted_sort_place(key_of, HsSampled{h.spl_key, h.spl_id}, hint, K, nb, h, tmp_key, tmp_bucket, slot_key,
                              slot_id, out_key, out_id, status, st);
