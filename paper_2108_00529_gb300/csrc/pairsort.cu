@@ -33,6 +33,7 @@
 // and 0.62 ms.  The 68 M keys: histogram 75 us, plan 36, moves 277 and 304, split
 // 185, sort 832 (instruction issue: about 260 thread instructions a key).
 #include "bgv_internal.cuh"
+#include "pieces.cuh"
 
 namespace bgv {
 namespace {
@@ -221,10 +222,11 @@ __device__ __forceinline__ void ps_append(const PsBucket &e, PsControl *ctl, PsB
 }
 // Equal keys need no sorting, only a place: shared out in pieces.
 __device__ __forceinline__ void ps_append_equal(PsBucket e, PsControl *ctl, PsBucket *list, uint32_t cap) {
-    const uint32_t end = e.start + e.count;
+    const uint32_t start = e.start, end = e.start + e.count, pieces = pieces_of(e.count, kPsW);
     e.flags |= kEqual;
-    for (; e.start < end; e.start += kPsW) {
-        e.count = min(kPsW, end - e.start);
+    for (uint32_t p = 0; p < pieces; ++p) {
+        e.start = start + p * kPsW;
+        e.count = piece_size(e.start, end, kPsW);
         ps_append(e, ctl, list, cap);
     }
 }
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(kMoveThreads, 2) k_ps_place(const unsigned lon
         if (t < kCoarse && uint32_t(t) * per < groups) {
             run_start[t] = bstart[t * per];
             run_end[t] = run_cursor[t];
-            tiles = (run_end[t] - run_start[t] + kMoveKeys - 1) / kMoveKeys;
+            tiles = pieces_of(run_end[t] - run_start[t], kMoveKeys);
         }
         uint32_t inc = tiles;
 #pragma unroll

@@ -23,6 +23,7 @@
 #include <mutex>
 
 #include "bgv_internal.cuh"
+#include "pieces.cuh"
 
 namespace bgv {
 
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(kDegThreads, 1) k_deg_count(const uint16_t *__
     const int t = threadIdx.x;
     const uint32_t c = t < ranges ? count[t] : 0u;
     scan_ranges(c, start);
-    scan_ranges((c + kDegPiece - 1) / kDegPiece, pieces);
+    scan_ranges(pieces_of(c, kDegPiece), pieces);
     const uint32_t total = pieces[kMaxRanges];
     for (uint32_t q = blockIdx.x; q < total; q += gridDim.x) {
         int lo = 0, hi = kMaxRanges;  // the range whose pieces hold q
@@ -243,9 +244,9 @@ __global__ void __launch_bounds__(kDegThreads, 1) k_deg_count(const uint16_t *__
         for (int i = t; i < kRange; i += kDegThreads) h[i] = 0u;
         __syncthreads();
         const uint32_t a = start[lo] + (q - pieces[lo]) * kDegPiece;
-        const uint32_t b = min(a + kDegPiece, start[lo + 1]);
+        const uint32_t b = a + piece_size(a, start[lo + 1], kDegPiece);
         // whole 16-byte words between the ragged ends
-        const uint32_t a8 = min((a + 7u) & ~7u, b), b8 = max(b & ~7u, a8);
+        const uint32_t a8 = a + ragged_head(a, b, 8u), b8 = max(b & ~7u, a8);
         if (t < a8 - a) atomicAdd(&h[swz(local[a + t] & (kRange - 1))], 1u);
         if (t < b - b8) atomicAdd(&h[swz(local[b8 + t] & (kRange - 1))], 1u);
         const uint4 *words = reinterpret_cast<const uint4 *>(local);
