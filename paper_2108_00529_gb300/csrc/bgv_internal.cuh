@@ -81,7 +81,10 @@ void note_launch();
 // A kernel that follows another one of its chain: its blocks may take their place
 // on the SMs while the last blocks of the one before still run, and wait there
 // (chain_wait, first thing in both kernels) until it has finished and its writes
-// are seen.  Saves the launch and most of the drain between two kernels.
+// are seen.  Saves the launch and most of the drain between two kernels.  What the
+// kernel before writes changes while the follower already runs: it is read with plain
+// loads, not as const __restrict__ or by __ldg, which promise data that stays as it is
+// for the kernel's whole life.
 template <class... P, class... A>
 int launch_chained(bool early, void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};

@@ -216,8 +216,7 @@ __global__ void __launch_bounds__(kThreads) k_keys(const float2 *__restrict__ po
 // its own interaction set in depth-first order; threads of a warp are Morton
 // neighbours, so they mostly read the same elements.
 template <int kRT>
-__global__ void __launch_bounds__(kRT) k_repulse(const float4 *__restrict__ geo, const int32_t *__restrict__ skip,
-                                                      const uint32_t *__restrict__ T,
+__global__ void __launch_bounds__(kRT) k_repulse(const float4 *geo, const int32_t *skip, const uint32_t *T,
                                                       const int64_t *__restrict__ koff,
                                                       const int32_t *__restrict__ bgraph,
                                                       const float4 *__restrict__ body, int64_t K, float kr,

@@ -54,7 +54,7 @@ __device__ __forceinline__ void box_warp(float4 &b) {
 // body is always entered; any other cell is accepted by the FP32 opening test
 // of the definition.
 template <class Skip>
-__device__ __forceinline__ float2 bh_walk(const float4 *__restrict__ geo, const Skip *__restrict__ skip, float4 bi,
+__device__ __forceinline__ float2 bh_walk(const float4 *geo, const Skip *skip, float4 bi,
                                           float kmi, float theta2, uint32_t self, uint32_t cur, uint32_t end,
                                           unsigned &inter) {
     float fx = 0.0f, fy = 0.0f;

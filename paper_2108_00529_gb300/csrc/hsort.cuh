@@ -149,8 +149,8 @@ inline HsBuffers hs_for(HsBuffers h, int nb) {
 struct HsSampled {
     const unsigned long long *key;
     const uint32_t *id;
-    __device__ unsigned long long key_at(int u) const { return __ldg(&key[u]); }
-    __device__ uint32_t id_at(int u) const { return __ldg(&id[u]); }
+    __device__ unsigned long long key_at(int u) const { return key[u]; }
+    __device__ uint32_t id_at(int u) const { return id[u]; }
 };
 struct HsPrevious {  // the sorted pairs of the previous iteration
     const unsigned long long *key;
@@ -426,8 +426,7 @@ __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, con
 
 // 3. Every pair to its bucket.
 __global__ void __launch_bounds__(256) k_hs_scatter(const uint32_t *__restrict__ hint, int64_t K, HsBuffers h,
-                                                    const unsigned long long *__restrict__ tmp_key,
-                                                    const uint32_t *__restrict__ tmp_bucket,
+                                                    const unsigned long long *tmp_key, const uint32_t *tmp_bucket,
                                                     unsigned long long *__restrict__ slot_key,
                                                     uint32_t *__restrict__ slot_id) {
     chain_wait();

@@ -348,7 +348,7 @@ struct LevelBits {
 // tile's blocks take tiles in order from a counter, so a tile's look-back waits
 // only for tiles that already run.
 __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
-    const unsigned long long *__restrict__ keys, const uint32_t *__restrict__ perm, int64_t K,
+    const unsigned long long *keys, const uint32_t *perm, int64_t K,
     const float2 *__restrict__ pos, const uint32_t *__restrict__ mass, const float4 *__restrict__ frames,
     const int32_t *__restrict__ bgraph, int L, int gbits, int leaf_cap, float4 *__restrict__ body, TileArrays T,
     uint32_t *dev_status, int spin_limit) {
@@ -389,6 +389,12 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
 
     // bodies and boundaries, neighbouring threads on neighbouring bodies
     uint32_t heaviest = 0u, least = 255u, greatest = 0u, ds = 0u;
+    uint32_t ids[kTileItems];
+#pragma unroll
+    for (int r = 0; r < kTileItems; ++r) {  // every load before any store: plain loads do not pass them
+        const int64_t s = t0 + r * kTileThreads + tid;
+        ids[r] = s < t0 + n ? perm[s] : 0u;
+    }
 #pragma unroll
     for (int r = 0; r < kTileItems; ++r) {
         const int e = r * kTileThreads + tid;
@@ -396,7 +402,7 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile(
         uint32_t m = 0u, d = 255u;
         uint2 U = make_uint2(0u, 0u);
         if (e < n) {
-            const uint32_t i = perm[s];
+            const uint32_t i = ids[r];
             const float2 p = pos[i];
             U = fixed_point(p, frames[bgraph ? bgraph[i] : 0]);
             m = mass[i];
