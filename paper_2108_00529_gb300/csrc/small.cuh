@@ -431,6 +431,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
         bool wide = false;
         for (int r = lo + (tid >> 5); r < hi && A.off; r += kSmallThreads / 32) {
             const int64_t b = A.off[k0 + r], e = A.off[k0 + r + 1];
+            wide |= b < e && (b < c_lo || e > c_hi);  // offsets that fall somewhere: rows past the block's range
             for (int64_t x = b + lane; x < e; x += 32) {
                 const int64_t j = int64_t(A.adj[x]) - k0;
                 const bool ok = j >= 0 && j < K;  // an invalid entry adds nothing
