@@ -30,7 +30,7 @@
  *             streams are made by the first such call of a host thread on a
  *             device (make it outside any stream capture) and live until the
  *             process ends; each step makes and destroys four CUDA events.
- *             (Steps and runs on graphs of up to 2,048 bodies and 524,288 CSR
+ *             (Steps and runs on graphs of up to 2,048 bodies and 131,072 CSR
  *             entries are one kernel on `stream` itself.)
  * Scratch.    The library allocates no memory.  Each stage takes a caller
  *             workspace `ws` of `ws_bytes` bytes (256-byte aligned), sized by

@@ -40,8 +40,12 @@ constexpr int kSmallRank = 32;           // largest bin ranked by counting
 // CSR entries a block keeps (weights below 2^21): what is left of its shared
 // memory.  200 steps at 1,764 bodies took 9,683 us with 8,192, and 7,239 with
 // 10,240, lighter moments and the sums merged by a warp.
-constexpr int kSmallCache = 10240;
-constexpr int64_t kSmallEntries = int64_t(1) << 19;  // CSR entries of a graph, at most
+constexpr int kSmallCache = 9664;
+// CSR entries of a graph, at most.  Half of them may lie in one block's rows, and are
+// read from memory in every step: 100 steps of 2,048 bodies 4.4 ms with 118,286 even
+// entries (general path 7.5), 7.6 with 489,116, but 16.4 with 332,304 of which half
+// lie in an eighth of the rows.
+constexpr int64_t kSmallEntries = int64_t(1) << 17;
 constexpr int kSmallChunk = 256;         // steps per launch, at most
 static_assert(kSmallMax == 4 * kSmallThreads, "four bodies a thread");
 static_assert(kSmallMax <= kSmallCluster * kSmallHalf, "a thread per node");
@@ -70,6 +74,7 @@ struct SmallMem {
     union {
         LevelBits<kSmallMax / 32> bits;
         MomP Pq[kSmallThreads + 1];      // then: moments before every fourth body
+        float2 fa[kSmallHalf];           // then: attraction of the block's long rows
     } w;
     unsigned long long some[32];         // of the bits
     union {
@@ -91,9 +96,13 @@ struct SmallMem {
     unsigned long long red[kSmallThreads / 32][5];
     float4 box[kSmallThreads / 32];
     uint32_t wsum[2][kSmallThreads / 32];  // of the sort, of the cells
+    int2 long_span[kSmallHalf];          // the block's rows of more than att_short entries
+    uint8_t long_rows[kSmallHalf];       // their nodes in the block
+    uint32_t longs, next;                // how many, and the next of them to sum
     uint32_t cells, greatest;
     double speed;
 };
+static_assert(sizeof(SmallMem) <= 227 * 1024, "shared memory of a block");
 
 // Exclusive block scan of one value per thread.
 __device__ __forceinline__ uint32_t small_scan(uint32_t x, uint32_t *wsum) {
@@ -342,52 +351,79 @@ __device__ uint32_t small_tree(SmallMem &m, int K, int L, int leaf_cap) {
     return cells;
 }
 
-// Attraction of one row [b, e) summed in the general path's order (k_att_*):
-// short rows by their thread, the others by the whole warp, one after the
-// other.  entry(x): neighbour and weight of CSR entry x (weight 0: none).
+// Attraction of one row [b, e) summed in the general path's order (k_att_*): a
+// short row by its thread, a longer one by a warp.  entry(x, p, &wf): position and
+// weight of CSR entry x (weight 0: none).
 template <class Entry>
-__device__ __forceinline__ float2 small_rows(const SmallMem &m, bool have, int64_t b, int64_t e, int att_short,
-                                             float2 pi, Entry entry) {
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ float2 small_short_row(int64_t b, int64_t e, float2 p, Entry entry) {
     float ax = 0.0f, ay = 0.0f;
-    const int64_t len = have ? e - b : 0;
-    if (len <= att_short) {
 #pragma unroll 4
-        for (int64_t x = b; x < b + len; ++x) {
-            float wf;
-            const float2 pj = entry(x, pi, &wf);
-            ax += wf * (pj.x - pi.x);
-            ay += wf * (pj.y - pi.y);
-        }
-    }
-    for (unsigned todo = __ballot_sync(0xFFFFFFFFu, len > att_short); todo; todo &= todo - 1u) {
-        const int src = __ffs(todo) - 1;
-        const int64_t rb = __shfl_sync(0xFFFFFFFFu, b, src), rl = __shfl_sync(0xFFFFFFFFu, len, src);
-        const float2 p = make_float2(__shfl_sync(0xFFFFFFFFu, pi.x, src), __shfl_sync(0xFFFFFFFFu, pi.y, src));
-        const bool block_row = rl > kAttMedium;  // a block's 256 threads: eight warps' sums, added in order
-        float tx = 0.0f, ty = 0.0f;
-        for (int vw = 0; vw < (block_row ? 8 : 1); ++vw) {
-            float sx = 0.0f, sy = 0.0f;
-            for (int64_t t = vw * 32 + lane; t < rl; t += block_row ? 256 : 32) {
-                float wf;
-                const float2 pj = entry(rb + t, p, &wf);
-                sx += wf * (pj.x - p.x);
-                sy += wf * (pj.y - p.y);
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                sx += __shfl_xor_sync(0xFFFFFFFFu, sx, d);
-                sy += __shfl_xor_sync(0xFFFFFFFFu, sy, d);
-            }
-            tx = vw ? tx + sx : sx;
-            ty = vw ? ty + sy : sy;
-        }
-        if (lane == src) {
-            ax = tx;
-            ay = ty;
-        }
+    for (int64_t x = b; x < e; ++x) {
+        float wf;
+        const float2 pj = entry(x, p, &wf);
+        ax += wf * (pj.x - p.x);
+        ay += wf * (pj.y - p.y);
     }
     return make_float2(ax, ay);
+}
+// kIn: entries of a lane in flight.
+template <int kIn, class Entry>
+__device__ __forceinline__ float2 small_warp_row(int64_t b, int64_t e, float2 p, Entry entry) {
+    const int lane = threadIdx.x & 31;
+    const bool block_row = e - b > kAttMedium;  // a block's 256 threads: eight warps' sums, added in order
+    const int stride = block_row ? 256 : 32;
+    float tx = 0.0f, ty = 0.0f;
+    for (int vw = 0; vw < (block_row ? 8 : 1); ++vw) {
+        float sx = 0.0f, sy = 0.0f;
+        for (int64_t x0 = b + vw * 32 + lane; x0 < e; x0 += kIn * stride) {
+            float wf[kIn];
+            float2 pj[kIn];
+#pragma unroll
+            for (int k = 0; k < kIn; ++k) {
+                const int64_t x = x0 + k * stride;
+                wf[k] = 0.0f;
+                if (x < e) pj[k] = entry(x, p, &wf[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < kIn; ++k) {
+                if (x0 + k * stride >= e) break;
+                sx += wf[k] * (pj[k].x - p.x);
+                sy += wf[k] * (pj[k].y - p.y);
+            }
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            sx += __shfl_xor_sync(0xFFFFFFFFu, sx, d);
+            sy += __shfl_xor_sync(0xFFFFFFFFu, sy, d);
+        }
+        tx = vw ? tx + sx : sx;
+        ty = vw ? ty + sy : sy;
+    }
+    return make_float2(tx, ty);
+}
+// The block's long rows, taken one after the other by whichever warp is free;
+// row(b, e, p): the sum of the row [b, e), whose node is at p.  Whole warps call it,
+// the walkers when they are done, as long as more than kSmallKeep rows are left: fewer
+// are summed before the last walker is done.  (A thread's own rows summed by its
+// warp, one after the other, left hubs to one warp: 100 steps of 1,500 bodies and
+// 226,212 entries, half of them in an eighth of the rows, 24.7 ms; so 11.6.)
+constexpr uint32_t kSmallKeep = 16;
+__device__ __forceinline__ bool small_rows_left(const SmallMem &m, uint32_t all) {
+    const uint32_t keep = threadIdx.x >= kSmallHalf ? kSmallKeep : 0u;
+    return __shfl_sync(0xFFFFFFFFu, *static_cast<const volatile uint32_t *>(&m.next), 0) + keep < all;
+}
+template <class Row>
+__device__ __forceinline__ void small_long_rows(SmallMem &m, int lo, Row row) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t all = m.longs;
+    while (small_rows_left(m, all)) {
+        const uint32_t q = __shfl_sync(0xFFFFFFFFu, lane == 0 ? atomicAdd(&m.next, 1u) : 0u, 0);
+        if (q >= all) break;
+        const int local = m.long_rows[q];
+        const int2 span = m.long_span[q];
+        const float2 f = row(span.x, span.y, m.pos[lo + local]);
+        if (lane == 0) m.w.fa[local] = f;
+    }
 }
 
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constant__ SmallArgs A) {
@@ -453,7 +489,19 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
         *wf = ok ? __uint2float_rn(__ldg(A.w + x)) : 0.0f;
         return ok ? m.pos[j] : own;
     };
-    if (tid == 0) m.speed = A.speed[g];
+    auto row_cached = [&](int b, int e, float2 p) { return small_warp_row<2>(b, e, p, entry_cached); };
+    auto row_global = [&](int b, int e, float2 p) { return small_warp_row<8>(b, e, p, entry_global); };
+    if (tid == 0) {
+        m.speed = A.speed[g];
+        m.longs = m.next = 0u;
+    }
+    __syncthreads();
+    const bool is_long = re - rb > A.att_short;
+    if (is_long) {
+        const uint32_t q = atomicAdd(&m.longs, 1u);
+        m.long_rows[q] = uint8_t(tid);
+        m.long_span[q] = make_int2(int(rb), int(re));
+    }
     cluster.sync();
     unsigned long long inter_total = 0ull;
     unsigned inter = 0u;
@@ -473,15 +521,17 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
                 cluster.map_shared_rank(m.frep, owner)[id - owner * per] = fr;
             }
             inter_total += inter;
-        } else {
-            if (node) p = m.pos[mine];
-            if (A.off)
-                fa = cached ? small_rows(m, node, rb, re, A.att_short, p, entry_cached)
-                            : small_rows(m, node, rb, re, A.att_short, p, entry_global);
+        } else if (node) {
+            p = m.pos[mine];
+            if (!is_long) fa = cached ? small_short_row(rb, re, p, entry_cached) : small_short_row(rb, re, p, entry_global);
+        }
+        if (small_rows_left(m, m.longs)) {
+            if (cached) small_long_rows(m, lo, row_cached); else small_long_rows(m, lo, row_global);
         }
         cluster.sync();  // the repulsions have arrived
         float2 st = make_float2(0.0f, 0.0f);
         if (node) {
+            if (is_long) fa = m.w.fa[tid];
             f = force_sum(fa, mass, p, m.frep[mine - lo], A.kg, A.strong);
             st = swing_traction(mass, f.x, f.y, fp.x, fp.y);
         }
@@ -494,6 +544,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
             }
         }
         cluster.sync();  // every block's sums, and nobody reads positions any more
+        if (tid == 0) m.next = 0u;
         if (warp == 0) {
             auto part = [&](int q, int k) {
                 if (q >= C * kSmallSums) return xsum_zero();
