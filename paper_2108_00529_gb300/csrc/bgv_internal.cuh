@@ -349,7 +349,7 @@ struct CommScratch {
     unsigned long long *best;       // packed (edge index, label) proposals
     uint32_t *jump;                 // labels after a pointer-jumping step
     uint32_t *map;                  // bit map of the nodes that pass the round's threshold
-    uint32_t *any;                  // [2] a bit of the round's map is set (by round parity)
+    float2 *weight;                 // [2] degrees of the nodes that pass the round's threshold, and of all (by parity)
 };
 void carve_comm(Carver &c, int64_t m, int32_t n, CommScratch &s, bool batched = false);
 // growth 0: the threshold is multiplied by its first value every round (the

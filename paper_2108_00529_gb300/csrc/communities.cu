@@ -17,7 +17,14 @@
 // anything.  With more nodes than bits, a bit stands for 2^shift neighbouring
 // ids and is set if any of them passes; the exact test follows on the gathered
 // degrees either way.  Measured: 3 rounds over 10 M R-MAT edges on 2^20 nodes
-// 178 us with the map, 452 with the gathers alone.
+// 114 us with the map, 386 with the gathers alone.
+//
+// Gathers in flight need room in the L1 that the map takes away: a map of 200 KB per
+// SM halved the rate of rounds in which nearly all edges pass (3 rounds over 10 M
+// uniform edges on 3.2 M nodes 1,115 us, 427 with the gathers alone), so a block's
+// map is 64 KB at most, two blocks share an SM (batched, whose words are twice as
+// wide, one), and from the round on in which nearly all edges would pass there is no
+// map: 443 us.
 //
 // Batched form: each node also carries its graph's threshold, (degree,
 // label, threshold) in one 16-byte word, so a propose still gathers one
@@ -29,8 +36,8 @@
 namespace bgv {
 namespace {
 constexpr int kThreads = 256;
-constexpr int kRoundThreads = 1024;  // one block per SM: the bit map takes most of its shared memory
-constexpr int kMapBytes = 208 * 1024;
+constexpr int kRoundThreads = 1024;
+constexpr int kMapBytes = 64 * 1024;
 constexpr unsigned long long kNone = ~0ull;
 
 // Ids per bit of the map, as a shift: the finest that fits.
@@ -68,30 +75,32 @@ __device__ __forceinline__ bool endpoints_ok(int32_t u, int32_t v, int32_t n, ui
     return u != v;
 }
 
-__device__ __forceinline__ void offer(unsigned long long *best, int32_t w, uint32_t e, uint32_t lab) {
-    const unsigned long long cand = (static_cast<unsigned long long>(e) << 32) | lab;
-    // The slot only decreases, so a stale read can only be larger than the
-    // current value: skipping when cand is not below it is always safe.
-    if (cand < __ldcg(&best[w])) atomicMin(&best[w], cand);
-}
-
-// The rule and the offer of one edge from both endpoints' state, (degree,
-// label) or, batched, (degree, label, threshold, first threshold): both
-// endpoints belong to one graph, so the threshold carried by u is the graph's.
-__device__ __forceinline__ void propose_edge(int32_t u, int32_t v, uint32_t e, uint2 su, uint2 sv, uint32_t D,
-                                             int tie_mode, unsigned long long *best) {
-    uint32_t lab;
-    const int32_t w = edge_rule(u, v, su.x, su.y, sv.x, sv.y, D, tie_mode, &lab);
-    if (w >= 0) offer(best, w, e, lab);
+// The offers of two edges: each joins best[w] (w < 0: none) as (edge index, label).
+// Both slots are read before either is written, so their round trips overlap.  A
+// slot only decreases, so a stale read can only be larger than the current value:
+// skipping when the offer is not below it is always safe.
+__device__ __forceinline__ void offer_two(unsigned long long *best, const int32_t (&w)[2], const uint32_t (&e)[2],
+                                          const uint32_t (&lab)[2]) {
+    unsigned long long now[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) now[j] = w[j] >= 0 ? __ldcg(&best[w[j]]) : 0ull;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const unsigned long long cand = (static_cast<unsigned long long>(e[j]) << 32) | lab[j];
+        if (cand < now[j]) atomicMin(&best[w[j]], cand);
+    }
 }
 
 // Edges from which a round filters them by the map.  Below, the map's way through
 // L2 costs more than the gathers it saves: ten rounds over 11,000 edges 160 us with
 // it and 136 without, four over 180,000 109 and 108, eight over 247,000 of an R-MAT
-// graph 132 and 159.  Where nearly every node passes, as on an even graph whose
-// threshold is the usual degree, the map saves nothing and a round is up to 8 %
-// longer than without (nine rounds over 1.08 M edges 240 us against 223).
+// graph 132 and 159.
 constexpr int64_t kMapMin = int64_t(1) << 17;
+// Largest share of the degrees that lies in nodes below the threshold, for a map: with
+// 0.9 about 0.8 of the edges pass it.  Seven rounds over 582,515 edges of an R-MAT graph
+// 132 us with 0.9, 143 with 0.7 and 158 with three quarters of the nodes, most of which
+// have few edges; three over 5 M uniform edges 166, 169 and 178.
+constexpr float kMapShare = 0.9f;
 
 // All rounds in one persistent kernel (cooperative launch, every block
 // resident): initial state and bit map, then per round the map into shared
@@ -104,37 +113,68 @@ constexpr int64_t kMapMin = int64_t(1) << 17;
 // checked their endpoints).  The barrier waits are bounded and report
 // BGV_DEV_TIMEOUT.  kB: the batched form.
 template <bool kB>
-__global__ void __launch_bounds__(kRoundThreads, 1) k_comm_rounds(
+__global__ void __launch_bounds__(kRoundThreads, kB ? 1 : 2) k_comm_rounds(
     const int32_t *__restrict__ edges, int64_t m, int32_t n, const uint32_t *__restrict__ deg_est,
     const int32_t *__restrict__ node_graph, const uint32_t *__restrict__ D0, int32_t passes, uint32_t threshold,
     uint32_t growth, int tie_mode, int32_t jumps, uint2 *state, uint4 *bstate, unsigned long long *best, uint32_t *jump,
-    uint32_t *map, int shift, int words, int filter, uint32_t *any, int32_t *__restrict__ labels, uint32_t *__restrict__ deg_out,
+    uint32_t *map, int shift, int words, int filter, float2 *weight, int32_t *__restrict__ labels, uint32_t *__restrict__ deg_out,
     uint32_t *status, WsHeader *hdr, int spin_limit) {
     extern __shared__ uint4 map_sh4[];
     const uint32_t *map_sh = reinterpret_cast<const uint32_t *>(map_sh4);
-    constexpr int kLoads = kB ? 1 : 3;  // int4 (two edges each) per thread in flight: 64 registers
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     const int64_t t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
-    // Every lane takes the 2^shift nodes of one map bit, so a warp's vote is a
-    // word of the map; `pass(v)` brings node v to the next round and says
-    // whether it passes that round's threshold.
+    __shared__ float2 part[kRoundThreads / 32];
+    // A warp takes the 2^shift rows of 32 nodes of one map word (lane t: the rows'
+    // votes of bit t); `pass(v, d)` brings node v to the next round and says whether
+    // it passes that round's threshold, and its degree d.  Adds the degrees (each
+    // plus one) of the nodes that pass, and of all, to weight[slot].
     auto each_node = [&](int slot, auto pass) {
-        const int64_t groups = int64_t(words) * 32;
-        for (int64_t q = t0; q < groups; q += stride) {  // whole warps: groups and stride are multiples of 32
-            bool ok = false;
-            const int64_t v0 = q << shift, v1 = (q + 1) << shift;
-            for (int64_t v = v0; v < v1 && v < n; ++v) ok |= pass(v);
-            if (!filter) continue;
-            const uint32_t word = __ballot_sync(0xFFFFFFFFu, ok);
-            if (lane == 0) {
-                map[q >> 5] = word;
-                if (word) any[slot] = 1u;
+        float passing = 0.0f, all = 0.0f;
+        for (int64_t w = t0 >> 5; w < words; w += stride >> 5) {
+            bool bit = false;
+            for (int j = 0; j < 1 << shift; ++j) {
+                const int64_t v = (((w << shift) + j) << 5) + lane;
+                uint32_t d = 0u;
+                const bool ok = v < n && pass(v, d);
+                if (!filter) continue;
+                const float dw = v < n ? __uint2float_rn(d) + 1.0f : 0.0f;
+                passing += ok ? dw : 0.0f;
+                all += dw;
+                const uint32_t row = __ballot_sync(0xFFFFFFFFu, ok);
+                if (shift >= 5) {  // rows lie inside one bit
+                    bit |= row != 0u && (j >> (shift - 5)) == lane;
+                } else {           // 32 >> shift bits in a row
+                    const int per = 32 >> shift, first = (lane & (per - 1)) << shift;
+                    bit |= lane / per == j && ((row >> first) & ((2u << ((1 << shift) - 1)) - 1u)) != 0u;
+                }
             }
+            if (!filter) continue;
+            const uint32_t word = __ballot_sync(0xFFFFFFFFu, bit);
+            if (lane == 0) map[w] = word;
+        }
+        if (!filter) return;
+        auto warp_sum = [&]() {
+#pragma unroll
+            for (int k = 16; k > 0; k >>= 1) {
+                passing += __shfl_xor_sync(0xFFFFFFFFu, passing, k);
+                all += __shfl_xor_sync(0xFFFFFFFFu, all, k);
+            }
+        };
+        warp_sum();
+        if (lane == 0) part[threadIdx.x >> 5] = make_float2(passing, all);
+        __syncthreads();
+        if (threadIdx.x >= 32) return;
+        passing = part[lane].x;
+        all = part[lane].y;
+        warp_sum();
+        if (lane == 0 && all > 0.0f) {
+            atomicAdd(&weight[slot].x, passing);
+            atomicAdd(&weight[slot].y, all);
         }
     };
-    each_node(0, [&](int64_t v) {
-        const uint32_t d = deg_est[v];
+    each_node(0, [&](int64_t v, uint32_t &d) {
+        d = deg_est[v];
         best[v] = kNone;
         if (kB) {
             const uint32_t d0 = D0[node_graph[v]];
@@ -147,40 +187,37 @@ __global__ void __launch_bounds__(kRoundThreads, 1) k_comm_rounds(
     if (!grid_barrier(&hdr->bar, spin_limit, status)) return;
     const int4 *e2 = reinterpret_cast<const int4 *>(edges);
     const int64_t pairs = m >> 1;
+    bool use = false;  // the round's map
     auto passes_map = [&](int32_t x) {
         const uint32_t b = uint32_t(x) >> shift;
-        return !filter || ((map_sh[b >> 5] >> (b & 31u)) & 1u) != 0u;
+        return !use || ((map_sh[b >> 5] >> (b & 31u)) & 1u) != 0u;
     };
     // both endpoints in range (else reported), not a loop, and both on the map
     auto wanted = [&](int32_t u, int32_t v) { return endpoints_ok(u, v, n, status) && passes_map(u) && passes_map(v); };
     unsigned long long D = threshold;
     const unsigned long long factor = growth ? growth : threshold;
     for (int32_t p = 0; p < passes; ++p) {
-        if (!filter || p == 0 || __ldcg(&any[p & 1]) != 0u) {
+        const float2 wt = filter ? __ldcg(&weight[p & 1]) : make_float2(1.0f, 1.0f);
+        use = filter && wt.x <= kMapShare * wt.y;
+        // thresholds do not fall: nearly all edges pass from here on (all blocks read
+        // the same sums)
+        if (!use) filter = 0;
+        if (p == 0 || wt.x > 0.0f) {
             const uint4 *src = reinterpret_cast<const uint4 *>(map);
-            if (filter) {
+            if (use) {
                 for (int i = threadIdx.x; i < words / 4; i += kRoundThreads) map_sh4[i] = __ldcg(src + i);
                 __syncthreads();
             }
-            for (int64_t q0 = t0; q0 < pairs; q0 += stride * kLoads) {
-                int4 e[kLoads];
-                bool go[2 * kLoads];
+            // two edges and the gathers of both at once
+            auto edge_pair = [&](const int4 e, const bool (&go)[2], const uint32_t (&index)[2]) {
+                uint2 su[2], sv[2];
+                uint32_t thr[2];
 #pragma unroll
-                for (int r = 0; r < kLoads; ++r)  // past the end: a loop, which is never wanted
-                    e[r] = q0 + r * stride < pairs ? __ldcs(e2 + q0 + r * stride) : make_int4(0, 0, 0, 0);
-#pragma unroll
-                for (int r = 0; r < kLoads; ++r) {
-                    go[2 * r] = wanted(e[r].x, e[r].y);
-                    go[2 * r + 1] = wanted(e[r].z, e[r].w);
-                }
-                uint2 su[2 * kLoads], sv[2 * kLoads];
-                uint32_t thr[2 * kLoads];
-#pragma unroll
-                for (int j = 0; j < 2 * kLoads; ++j) {
-                    const int32_t u = (j & 1) ? e[j >> 1].z : e[j >> 1].x, v = (j & 1) ? e[j >> 1].w : e[j >> 1].y;
+                for (int j = 0; j < 2; ++j) {
+                    const int32_t u = j ? e.z : e.x, v = j ? e.w : e.y;
                     thr[j] = uint32_t(D);
                     su[j] = sv[j] = make_uint2(0xFFFFFFFFu, 0u);
-                    if (go[j] && kB) {
+                    if (go[j] && kB) {  // both endpoints belong to one graph: u's threshold is the graph's
                         const uint4 a = __ldcg(&bstate[u]), b = __ldcg(&bstate[v]);
                         su[j] = make_uint2(a.x, a.y);
                         sv[j] = make_uint2(b.x, b.y);
@@ -190,33 +227,33 @@ __global__ void __launch_bounds__(kRoundThreads, 1) k_comm_rounds(
                         sv[j] = __ldcg(&state[v]);
                     }
                 }
+                int32_t w[2];
+                uint32_t lab[2] = {0u, 0u};
 #pragma unroll
-                for (int j = 0; j < 2 * kLoads; ++j) {
-                    const int32_t u = (j & 1) ? e[j >> 1].z : e[j >> 1].x, v = (j & 1) ? e[j >> 1].w : e[j >> 1].y;
-                    if (go[j])
-                        propose_edge(u, v, uint32_t(2 * (q0 + (j >> 1) * stride) + (j & 1)), su[j], sv[j], thr[j],
-                                     tie_mode, best);
-                }
+                for (int j = 0; j < 2; ++j)
+                    w[j] = go[j] ? edge_rule(j ? e.z : e.x, j ? e.w : e.y, su[j].x, su[j].y, sv[j].x, sv[j].y, thr[j],
+                                             tie_mode, &lab[j])
+                                 : -1;
+                offer_two(best, w, index, lab);
+            };
+            for (int64_t q = t0; q < pairs; q += stride) {
+                const int4 e = __ldcs(e2 + q);
+                const bool go[2] = {wanted(e.x, e.y), wanted(e.z, e.w)};
+                const uint32_t index[2] = {uint32_t(2 * q), uint32_t(2 * q + 1)};
+                if (go[0] || go[1]) edge_pair(e, go, index);
             }
             if ((m & 1) && t0 == 0) {
-                const int32_t u = edges[2 * (m - 1)], v = edges[2 * (m - 1) + 1];
-                if (wanted(u, v)) {
-                    if (kB) {
-                        const uint4 a = __ldcg(&bstate[u]), b = __ldcg(&bstate[v]);
-                        propose_edge(u, v, uint32_t(m - 1), make_uint2(a.x, a.y), make_uint2(b.x, b.y), a.z, tie_mode,
-                                     best);
-                    } else {
-                        propose_edge(u, v, uint32_t(m - 1), __ldcg(&state[u]), __ldcg(&state[v]), uint32_t(D), tie_mode,
-                                     best);
-                    }
-                }
+                const int4 e = make_int4(edges[2 * (m - 1)], edges[2 * (m - 1) + 1], 0, 0);
+                const bool go[2] = {wanted(e.x, e.y), false};
+                const uint32_t index[2] = {uint32_t(m - 1), 0u};
+                edge_pair(e, go, index);
             }
         }
         if (!grid_barrier(&hdr->bar, spin_limit, status)) return;
         D *= factor;
         if (D > 0xFFFFFFFFull) D = 0xFFFFFFFFull;
-        if (t0 == 0) any[p & 1] = 0u;  // read by every block before the barrier; written next after the one below
-        each_node((p + 1) & 1, [&](int64_t v) {
+        if (t0 == 0) weight[p & 1] = make_float2(0.0f, 0.0f);  // read by every block before the barrier; written next after the one below
+        each_node((p + 1) & 1, [&](int64_t v, uint32_t &d) {
             const unsigned long long b = __ldcg(&best[v]);
             if (kB) {
                 uint4 st = __ldcg(&bstate[v]);
@@ -228,6 +265,7 @@ __global__ void __launch_bounds__(kRoundThreads, 1) k_comm_rounds(
                 const unsigned long long nd = static_cast<unsigned long long>(st.z) * (growth ? growth : st.w);
                 st.z = nd > 0xFFFFFFFFull ? 0xFFFFFFFFu : uint32_t(nd);
                 bstate[v] = st;
+                d = st.x;
                 return st.x <= st.z;
             }
             uint2 st = __ldcg(&state[v]);
@@ -237,6 +275,7 @@ __global__ void __launch_bounds__(kRoundThreads, 1) k_comm_rounds(
                 state[v] = st;
                 best[v] = kNone;
             }
+            d = st.x;
             return st.x <= uint32_t(D);
         });
         if (!grid_barrier(&hdr->bar, spin_limit, status)) return;
@@ -303,7 +342,7 @@ void carve_comm(Carver &c, int64_t m, int32_t n, CommScratch &s, bool batched) {
     s.best = c.take<unsigned long long>(size_t(n));
     s.jump = c.take<uint32_t>(size_t(n));
     s.map = c.take<uint32_t>(size_t(map_words(n, map_shift(n))));
-    s.any = c.take<uint32_t>(2);
+    s.weight = c.take<float2>(2);
 }
 
 void carve_mode(Carver &c, int32_t n, int32_t G, ModeScratch &s) {
@@ -338,21 +377,22 @@ int run_communities(const int32_t *edges, int64_t m, int32_t n, const uint32_t *
     unsigned long long *best = s.best;
     uint32_t *jump = s.jump;
     int tmode = tie_mode, limit = spin_limit();
-    uint32_t *map = s.map, *any = s.any;
-    int shift = map_shift(n), words = int(map_words(n, shift));
+    uint32_t *map = s.map;
+    float2 *weight = s.weight;
     int filter = m >= kMapMin ? 1 : 0;
-    BGV_CUDA(cudaMemsetAsync(any, 0, 2 * sizeof(uint32_t), st));
+    int shift = filter ? map_shift(n) : 0, words = int(map_words(n, shift));
+    BGV_CUDA(cudaMemsetAsync(weight, 0, 2 * sizeof(float2), st));
     void *args[] = {&edges, &m, &n, &deg_est, &node_graph, &D0, &passes, &threshold, &growth, &tmode, &jumps,
-                    &state, &bstate, &best, &jump, &map, &shift, &words, &filter, &any, &labels, &deg_out, &status, &hdr, &limit};
+                    &state, &bstate, &best, &jump, &map, &shift, &words, &filter, &weight, &labels, &deg_out, &status, &hdr, &limit};
     const void *kernel = batch ? reinterpret_cast<const void *>(k_comm_rounds<true>)
                                : reinterpret_cast<const void *>(k_comm_rounds<false>);
-    const size_t smem = size_t(words) * sizeof(uint32_t);
+    const size_t smem = filter ? size_t(words) * sizeof(uint32_t) : 0;
     BGV_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMapBytes));
     // no more blocks than there is work for (two edges a thread): a barrier over
     // few blocks is shorter; with four a thread ten rounds over 11,000 edges took 136
     // us, with two 110
     const int64_t work = int64_t(n) > m / 2 ? int64_t(n) : m / 2;
-    const int blocks = coop_blocks(kernel, kRoundThreads, grid_for(work, kRoundThreads, sm_count()), smem);
+    const int blocks = coop_blocks(kernel, kRoundThreads, grid_for(work, kRoundThreads, sm_count() * (batch ? 1 : 2)), smem);
     return launch_coop(kernel, blocks, kRoundThreads, args, st, smem);
 }
 
