@@ -685,7 +685,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf
                                                       uint32_t list_cap, const PsBucket *__restrict__ over) {
     extern __shared__ uint32_t smem[];
     __shared__ uint32_t big[kPsW / (kPsRank + 1) + 1];  // bins too large to rank: start | size << 16
-    __shared__ uint32_t bigs, next_sh;
+    __shared__ uint32_t bigs, next_sh, low_min, low_max;
     const int b = key_bits(*K_dev), s1 = fine_shift(b);
     const uint32_t splits = kSplit ? ctl->over : 0u, planned = ctl->planned;
     const uint32_t count = kSplit ? splits + min(planned, list_cap) : min(ctl->buckets, list_cap) - min(planned, list_cap);
@@ -696,6 +696,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf
             const bool off = *static_cast<volatile uint32_t *>(&ctl->guard) != 0u;
             next_sh = off ? 0xFFFFFFFFu : atomicAdd(kSplit ? &ctl->split_ticket : &ctl->ticket, 1u);
             bigs = 0u;
+            low_min = 0xFFFFFFFFu;
+            low_max = 0u;
         }
         __syncthreads();
         uint32_t q = next_sh;
@@ -746,8 +748,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf
         };
         for (int i = threadIdx.x; i < P2; i += kThreads) pcnt[i] = 0u;
         __syncthreads();
-        each_key([&](uint32_t pr, uint32_t) { atomicAdd(&pcnt[swz(pr)], 1u); });
+        // the range of the low parts: ids that keep to their neighbourhood (graphs side
+        // by side, crawls) leave most of the 2^p values out
+        uint32_t least = 0xFFFFFFFFu, most = 0u;
+        each_key([&](uint32_t pr, uint32_t low) {
+            atomicAdd(&pcnt[swz(pr)], 1u);
+            least = min(least, low);
+            most = max(most, low);
+        });
+        least = __reduce_min_sync(0xFFFFFFFFu, least);
+        most = __reduce_max_sync(0xFFFFFFFFu, most);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&low_min, least);
+            atomicMax(&low_max, most);
+        }
         __syncthreads();
+        least = low_min;
+        const int lb = low_max > least ? 32 - __clz(low_max - least) : 0;  // bits of the range, at most p
         // bins of a primary with c keys: 2^k, about c / 4 (at most c / 2)
         int NB;
         {
@@ -756,7 +773,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf
             uint32_t sum = 0, all;
             for (int i = i0; i < i1; ++i) {
                 const uint32_t c = pcnt[swz(i)];
-                const int k = c > 4 ? min(32 - __clz((c - 1) >> 2), p) : 0;
+                const int k = c > 4 ? min(32 - __clz((c - 1) >> 2), lb) : 0;
                 pcnt[swz(i)] = uint32_t(k) << 24;
                 sum += 1u << k;
             }
@@ -773,7 +790,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf
         auto bin_of = [&](uint32_t pr, uint32_t low, int *k) {
             const uint32_t x = pcnt[swz(pr)];
             *k = int(x >> 24);
-            return (x & 0xFFFFFFu) + (*k ? low >> (p - *k) : 0u);
+            return (x & 0xFFFFFFu) + (*k ? (low - least) >> (lb - *k) : 0u);
         };
         each_key([&](uint32_t pr, uint32_t low) {
             int k;
@@ -809,7 +826,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ps_sort(unsigned long long *buf
             const uint32_t j = bin_of(pr, mine, &k);
             const int lo = j ? int(bins[j - 1]) : 0, hi = int(bins[j]);
             int pos = s;
-            if (k < p) {  // else the bin is one key value
+            if (k < lb) {  // else the bin is one key value
                 if (hi - lo > kPsRank) {
                     if (s == lo) big[atomicAdd(&bigs, 1u)] = uint32_t(lo) | (uint32_t(hi - lo) << 16);
                     continue;

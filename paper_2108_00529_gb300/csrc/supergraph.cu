@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_csr_reduce(const unsigned long 
         __threadfence();
         atomicExch(&flags[tile], tile == 0 ? kRedIncl : kRedAgg);
     }
-    if (threadIdx.x == 32) {
+    if (threadIdx.x == 32 && uint32_t(tile_tot)) {  // a tile inside one run has no weight to find
         const unsigned long long k = skey[red_slot(tn - 1)];
         int64_t lo = t0 + tn, step = 1;  // keys[lo - 1] is in the run
         while (lo < nk && keys[lo] == k) {
