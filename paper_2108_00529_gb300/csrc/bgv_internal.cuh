@@ -208,7 +208,9 @@ int radix_sort_high(SortBuffers &b, const RunFixBuffers &r, int64_t cap, const i
 int radix_sort_high_result(int64_t cap, int end_bit);
 
 // radix_sort in its cooperative form, run only if *guard (device) is above
-// guard_min; the result is in buffer pair 0 (an even number of passes).
+// guard_min; the input is in buffer pair radix_guarded_input(end_bit), the result in
+// pair 0.
+int radix_guarded_input(int end_bit);
 int radix_sort_guarded(SortBuffers &b, int64_t cap, const int64_t *d_count, int end_bit, cudaStream_t s,
                        uint32_t *dev_status, const uint32_t *guard, uint32_t guard_min);
 

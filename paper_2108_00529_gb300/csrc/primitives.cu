@@ -7,6 +7,7 @@
 // the digit offsets stay consistent).
 #include <algorithm>
 #include <atomic>
+#include <utility>
 
 #include "bgv_internal.cuh"
 
@@ -721,12 +722,18 @@ int radix_sort(SortBuffers &b, int64_t cap, const int64_t *d_count, int end_bit,
     return BGV_OK;
 }
 
+int radix_guarded_input(int end_bit) { return (end_bit + 7) / 8 & 1; }
 int radix_sort_guarded(SortBuffers &b, int64_t cap, const int64_t *d_count, int end_bit, cudaStream_t s,
                        uint32_t *dev_status, const uint32_t *guard, uint32_t guard_min) {
-    const int passes = ((end_bit + 7) / 8 + 1) & ~1;
+    const int passes = (end_bit + 7) / 8;
     if (passes > kMaxPasses) return BGV_EINVAL;
+    SortBuffers from = b;  // an odd number of passes starts in buffer pair 1
+    if (radix_guarded_input(end_bit)) {
+        std::swap(from.keys[0], from.keys[1]);
+        std::swap(from.vals[0], from.vals[1]);
+    }
     BGV_CUDA(cudaMemsetAsync(b.counts, 0, sizeof(uint32_t) * size_t(sort_counter_words()), s));
-    return coop_sort(b, cap, d_count, 0, passes, s, dev_status, guard, guard_min);
+    return coop_sort(from, cap, d_count, 0, passes, s, dev_status, guard, guard_min);
 }
 
 // ----------------------------------------------- sort with a local finish

@@ -522,6 +522,9 @@ int run_supergraph(const int32_t *edges, int64_t m, int32_t n, const int32_t *la
     SortBuffers pairs = s.sort_pairs;
     const int64_t *nkeys = reinterpret_cast<const int64_t *>(s.nkeys);
     const bool bucketed = use_pair_sort(m, n);
+    // A row's pairs tie on their low 16 bits far too often for a local
+    // finish on them (hub rows), so every digit gets an LSD pass.
+    const int end_bit = 2 * bits_for(n);  // supernode ids < K <= n
     const uint32_t *guard = bucketed ? &s.ps.ctl->guard : nullptr;
     unsigned long long *cut_cursor = bucketed ? s.cut_cursor : s.nkeys;
     BGV_CUDA(cudaMemsetAsync(cut_cursor, 0, sizeof(unsigned long long), st));
@@ -531,12 +534,10 @@ int run_supergraph(const int32_t *edges, int64_t m, int32_t n, const int32_t *la
     if (m > 0) {
         const int64_t chunks = ((m + 1) / 2 + kCutPairs - 1) / kCutPairs;
         note_launch(), k_cut_pairs<<<grid_for(chunks, 1, sm_count() * 8), kThreads, 0, st>>>(
-            edges, m, n, node_map, K_dev, pairs.keys[0], cut_cursor, guard, status);
+            edges, m, n, node_map, K_dev, pairs.keys[bucketed ? radix_guarded_input(end_bit) : 0], cut_cursor, guard,
+            status);
         BGV_TRY(launch_status());
     }
-    // A row's pairs tie on their low 16 bits far too often for a local
-    // finish on them (hub rows), so every digit gets an LSD pass.
-    const int end_bit = 2 * bits_for(n);  // supernode ids < K <= n
     int res = 0;
     if (bucketed)
         BGV_TRY(radix_sort_guarded(pairs, cap, nkeys, end_bit, st, status, guard, 0u));
