@@ -112,7 +112,14 @@ constexpr int kDegTile = kPlaceThreads * kDegIn * 4; // endpoints per tile
 constexpr uint32_t kDegPiece = 1u << 18;           // endpoints a block counts at a time
 
 inline int deg_ranges(int32_t n) { return (n + kRange - 1) / kRange; }
-inline bool split_degrees(int64_t m, int32_t n) { return m >= kDegSplitMin && deg_ranges(n) <= kMaxRanges; }
+// With few endpoints a node the ranges' runs are short: uniform endpoints, 4.2 M edges on
+// 4 M nodes 197 us with the ranges and 208 without, 5 M on 8 M 318 and 316, 8 M on 8 M
+// 373 and 386; 8 M on 16 M 579 and 557, 16 M on 16 M 753 and 746, 32 M on 16 M 994 and
+// 1,009.
+inline bool split_degrees(int64_t m, int32_t n) {
+    return m >= kDegSplitMin && m >= n && (deg_ranges(n) <= kMaxRanges / 2 || 2 * m >= 3 * int64_t(n)) &&
+           deg_ranges(n) <= kMaxRanges;
+}
 
 // Endpoint j (0..3) of int4 pair e; an odd last edge is half a pair.
 __device__ __forceinline__ int32_t endpoint(const int4 &e, int j) { return j == 0 ? e.x : j == 1 ? e.y : j == 2 ? e.z : e.w; }
