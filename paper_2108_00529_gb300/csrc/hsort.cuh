@@ -57,7 +57,8 @@ constexpr int kHsPairCap = kHsThreads * kHsItems;  // 2048: a chunk of the pair 
 constexpr int kHsCap = kHsPairCap;      // larger buckets take the chunked path
 constexpr int kHsCapBits = 11;
 static_assert(kHsCap == 1 << kHsCapBits, "places of a bucket");
-constexpr int kHsRankSlices = 8;       // slices of the samples per ranking thread
+constexpr int kHsRankSlices = 16;       // slices of the samples per ranking thread
+constexpr int kHsAgainSlices = 8;       // the same of the ranking that returns at once as a rule: fewer blocks
 constexpr int kHsBins = 2048;           // bins of a bucket's words
 constexpr uint32_t kHsRankBin = 32;     // largest bin ranked by counting
 constexpr int kHsSmem = kHsCap + kHsCap / 16;  // skewed shared-memory slots
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(256) k_hs_rank(Samples samples, int ns, int s,
     __shared__ unsigned long long sk[256];
     __shared__ uint32_t si[256];
     __shared__ bool last;
-    const int per = (ns + kHsRankSlices - 1) / kHsRankSlices;
+    const int per = (ns + int(gridDim.y) - 1) / int(gridDim.y);
     const int j0 = blockIdx.y * per;
     const int j1 = min(ns, j0 + per);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -876,7 +877,7 @@ int hinted_sort_place(KeyOf key_of, Split split, const uint32_t *hint, int64_t K
     const bool again = !kSampled && nb > 1;
     if (again) {
         const HsShape sh = hs_shape(nb);
-        const dim3 g((sh.ns + 255) / 256, kHsRankSlices);
+        const dim3 g((sh.ns + 255) / 256, kHsAgainSlices);
         BGV_TRY(launch_chained(early, k_hs_rank<HsCounted>, g, 256, st, HsCounted{tmp_key, hint, K, sh.ns}, sh.ns, sh.s,
                                h));
         BGV_TRY(launch_chained(true, k_hs_count<HsAgain, HsSampled>, grid_for(K, 256, sm_count() * 2), 256, st,
