@@ -142,8 +142,8 @@ int fa2_loop(int64_t K, int64_t nnz, const int32_t *off, const int32_t *adj, con
         return BGV_OK;
     }
     // The first step runs outside the graph, builds the attraction plan and
-    // sorts the bodies with the full radix sort; the captured step reuses the
-    // plan and takes the previous step's order as its sort hint.
+    // sorts the bodies without a hint; the captured step reuses the plan and
+    // takes the previous step's order as its sort's hint and splitters.
     BGV_TRY(run_fa2(1, K, nnz, off, adj, w, mass, p, pos, F, Fprev, speed, nullptr, nullptr, nullptr, hdr, scratch,
                     st, nullptr, true, G, koff));
     if (iterations == 1) return BGV_OK;

@@ -3,10 +3,12 @@
 // One iteration is a fixed chain of kernels with no host round trip:
 //   k_frame     bounding square of the positions (last-block finalise); the
 //               later steps of a run find it made by the tail before them
-//   k_keys      fixed-point coordinates U and 2L-bit Morton keys; clears the
-//               step's counters (the captured step has no memset nodes)
-//   radix sort  (key, body) pairs -> Morton order: LSD passes on the bits
-//               above 24, then each run of equal high bits ordered locally
+//   k_hs_*      (key, body) pairs -> Morton order: fixed-point coordinates U and
+//               2L-bit Morton keys, to buckets between the previous step's
+//               pairs (a first step: between sampled ones), sorted there
+//               (hsort.cuh).  First steps of more than 65,536 bodies take k_keys
+//               and the radix sort: LSD passes on the bits above 24, then each
+//               run of equal high bits ordered locally
 //   k_tile*     bodies in Morton order, quadtree cells with FP32 centres from
 //               exact integer moments, and the depth-first pre-order with skip
 //               indices (tree.cuh)
@@ -306,9 +308,9 @@ __global__ void __launch_bounds__(kThreads) k_att_plan(int64_t K, const int32_t 
 
 // Short rows: one lane each, by up to 64 blocks per SM: blocks that end early leave
 // their places to the main chain (500 steps of 1 M bodies with uniform rows 175.4 ms
-// with 16 per SM, 170.6 with 64).  Where as many entries or more lie in medium rows,
-// whose launch follows, only `wave` blocks work, 16 per SM (150 steps of 3.2 M bodies
-// of an R-MAT graph 161.7 ms with 16, 169 with 64).
+// with 16 per SM, 170.6 with 64).  Where there is a medium row, whose launch follows,
+// for every 32 short ones or more, only `wave` blocks work, 16 per SM (150 steps of
+// 3.2 M bodies of an R-MAT graph 161.7 ms with 16, 169 with 64).
 __global__ void __launch_bounds__(kThreads, 5) k_att_short(int64_t K, const int32_t *__restrict__ off,
                                                         const int32_t *__restrict__ adj,
                                                         const uint32_t *__restrict__ w,
@@ -840,9 +842,9 @@ int set_fa2_tune(const Fa2Tune &t) {
     return BGV_OK;
 }
 
-// How a step after the first of a run finds the Morton order, process
-// wide: 1 (default) the hinted sort from the previous step's order, 0 the
-// full radix sort every step.  Both give the same order.
+// How a step finds the Morton order, process wide: 1 (default) by buckets, from the
+// previous step's order or, in a first or single step of up to kHsFirstMax bodies,
+// between sampled keys; 0 by the radix sort in every step.  Both give the same order.
 static std::atomic<int> g_fa2_order{1};
 int fa2_order() { return g_fa2_order.load(std::memory_order_relaxed); }
 int set_fa2_order(int method) {
@@ -1001,9 +1003,8 @@ static int run_fa2_body(int mode, int64_t K, int64_t nnz, const int32_t *csr_off
                                       s.sort.vals[res], &hdr->status, st));
         } else {
             // a first or single step: from id order, with sampled splitters (five
-            // launches; the radix sort, with its local finish, takes nine: a single
-            // step of 60,000 bodies 160.1 against 149.9 us); also clears what later
-            // steps find cleared
+            // launches; the radix sort, with its local finish, takes nine); also
+            // clears what later steps find cleared
             HsClears clr;
             clr.u32 = s.tree.flags;
             clr.n_u32 = tile_flag_words(K);
