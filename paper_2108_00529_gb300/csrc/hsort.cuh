@@ -25,7 +25,7 @@
 //      last block turns the counts into bucket starts.  When the keys have
 //      moved as a whole (a caller's own start that expands, a frame that a few
 //      bodies stretch), many of them lie between two of the previous splitters:
-//      with a bucket of more than kHsPoor pairs the step takes samples of its
+//      with a bucket of more than hs_poor pairs the step takes samples of its
 //      own keys after all and counts again.  Those two kernels follow every count
 //      and return at once as a rule.
 //   3. Scatter: every pair to its bucket (one atomic per bucket per warp).
@@ -62,7 +62,12 @@ constexpr int kHsAgainSlices = 8;       // the same of the ranking that returns 
 constexpr int kHsBins = 2048;           // bins of a bucket's words
 constexpr uint32_t kHsRankBin = 32;     // largest bin ranked by counting
 constexpr int kHsSmem = kHsCap + kHsCap / 16;  // skewed shared-memory slots
-constexpr uint32_t kHsPoor = 2 * kHsCap;  // a larger bucket and the sort counts again
+// The sort counts again with a larger bucket than this: where the second count has eight
+// samples a bucket, nearly all its buckets stay in shared memory, and a bucket of one
+// block's chunks and merges costs more than that count (80 us for 2,049 to 4,096 pairs,
+// 27 for the rest; 10 steps of 140,000 bodies at scales e^0 to e^14 2,283 us with a line
+// of 4,096 and 2,105 so).  With four samples or two some of its buckets are larger too.
+__host__ __device__ constexpr uint32_t hs_poor(int nb) { return nb <= 512 ? kHsCap : 2 * kHsCap; }
 
 inline int64_t hs_max_keys() { return int64_t(kHsMaxBuckets) * kHsBucket; }
 
@@ -342,7 +347,7 @@ struct HsAgain {};
 
 // 2. Keys and buckets in hint order, counts per bucket; the last block
 // writes the bucket starts, or, with previous splitters and a bucket of more than
-// kHsPoor pairs, asks for the second count (KeyOf = HsAgain).
+// hs_poor pairs, asks for the second count (KeyOf = HsAgain).
 template <class KeyOf, class Split>
 __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, const uint32_t *__restrict__ hint,
                                                   int64_t K, int nb, HsBuffers h, unsigned long long *tmp_key,
@@ -419,7 +424,7 @@ __global__ void __launch_bounds__(256) k_hs_count(KeyOf key_of, Split split, con
     }
     if (threadIdx.x == 0) h.start[nb] = uint32_t(K);
     if (kAgain && threadIdx.x == 0) *h.poor = 0u;
-    if (kWatch && __syncthreads_or(most > kHsPoor)) {
+    if (kWatch && __syncthreads_or(most > hs_poor(nb))) {
         for (int b = threadIdx.x; b < nb; b += blockDim.x) h.count[b] = 0u;
         if (threadIdx.x == 0) *h.poor = 1u;
     }
